@@ -16,6 +16,7 @@
 
 #include <limits>
 
+#include "smallest.cuh"
 #include "warp_la.cuh"
 
 // Column-scaled conditioning estimate of an upper R whose columns came from a
@@ -272,7 +273,7 @@ __device__ void finish_column(const ColArgs& a, int j, int k, int m, int l, int 
   R r2 = R(0);
   for (int r = lane; r < m; r += DIAF_WARP) {
     SD s = sc_zero<SD>();
-    for (int q = 0; q < k; ++q) s += Ts[r + q * LDT] * wv[q];
+    for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
     if (ix.inI[r] >= 0) s -= vv[ix.inI[r]];
     r2 += sc_abs2(s);
   }
@@ -472,6 +473,21 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
       Tw[r + c * LDT] = (r < m && ix.inI[r] >= 0) ? sc_zero<S>() : Ts[r + c * LDT];
     }
     __syncwarp();
+    S xw = sc_zero<S>();
+    bool direct = false;
+    if constexpr (kSmallestFits<S, KMAX>)
+      direct = warp_smallest_vector<S, S, KMAX, LDT, KP>(Ts, ix.inI, Tw, wv, vv, m, k, lane, &xw);
+    __syncwarp();
+    if (direct) {
+      if (lane < k) wv[lane] = xw;
+    } else {
+    if constexpr (kSmallestFits<S, KMAX>) {  // the attempt overwrote the working tile
+      for (int i = lane; i < me * k; i += DIAF_WARP) {
+        int r = i % me, c = i / me;
+        Tw[r + c * LDT] = (r < m && ix.inI[r] >= 0) ? sc_zero<S>() : Ts[r + c * LDT];
+      }
+      __syncwarp();
+    }
     warp_householder_qr_rs<S, LDT, KMAX, MMAX / DIAF_WARP>(Tw, me, k, lane);
     for (int i = lane; i < k * k; i += DIAF_WARP) {
       int r = i % k, c = i / k;
@@ -494,12 +510,13 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
     if (smin <= 1e-14 * smax || m - inrows < k) flags |= DIAF_FLAG_RANK_DEFICIENT;
     if (k > 1 && (snext - smin) <= 1e-6 * smax) flags |= DIAF_FLAG_DEGENERATE;
     for (int q = lane; q < k; q += DIAF_WARP) wv[q] = Vj[q + imin * KP];
+    }
     __syncwarp();
     for (int t = lane; t < l; t += DIAF_WARP) {
       S s = sc_zero<S>();
       int r = ix.Iloc[t];
       if (r >= 0)
-        for (int q = 0; q < k; ++q) s += Ts[r + q * LDT] * wv[q];
+        for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
       vv[t] = s;
     }
     __syncwarp();

@@ -5,7 +5,8 @@
 // (w_j, v_j) are refined in FP64 against the FP64 tile and the residual
 // ||A w - v|| is evaluated in FP64.
 //
-//   DIAF-S: the FP32 Jacobi gives R-hat V = U diag(sigma); x0 = V e_min.
+//   DIAF-S: w by warp_smallest_vector (smallest.cuh) where that form takes the
+//     column; otherwise the FP32 Jacobi gives R-hat V = U diag(sigma); x0 = V e_min.
 //     With H = A-hat^* A-hat taken from the FP64 tile, V^* H V is diagonal to
 //     FP32 accuracy, so one correction in that basis,
 //       d = x^* H x / x^* x,  r = H x - d x,
@@ -146,24 +147,6 @@ struct MixedLayout {
   static constexpr size_t bytes() { return (raw() + 15) / 16 * 16; }
 };
 
-// lane c < k: (T^* z)_c in FP64 over the m tile rows.  Tiles of up to 16
-// columns split the rows between the two half-warps (alternate rows, one
-// shuffle to combine), halving the FP64 instructions of the product.
-template <class SD, int LDT, int KMAX>
-__device__ __forceinline__ SD tile_adj_mul(const SD* Ts, const SD* zz, int m, int k, int lane) {
-  SD g = sc_zero<SD>();
-  if constexpr (KMAX <= 16) {
-    const int c = lane & 15;
-    if (c < k)
-      for (int r = lane >> 4; r < m; r += 2) g += sc_cmul(Ts[r + c * LDT], zz[r]);
-    g += shfl_xor(g, 16);
-  } else {
-    if (lane < k)
-      for (int r = 0; r < m; ++r) g += sc_cmul(Ts[r + lane * LDT], zz[r]);
-  }
-  return g;
-}
-
 template <class S, int KMAX, int MMAX, int ALG>
 __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
                                    typename DoubleOf<S>::T* Ts, typename DoubleOf<S>::T* Tx, int lane) {
@@ -290,6 +273,24 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
   DIAF_PHASE(4);
 
   if (ALG == DIAF_ALG_S) {
+    // ---- A-hat (I_j rows zeroed) in FP32, its smallest singular vector by
+    // inverse iteration; the columns that form cannot take go on to the FP32
+    // QR of A-hat and the Jacobi SVD of R-hat
+    for (int c = 0; c < k; ++c)
+      for (int r = lane; r < m; r += DIAF_WARP)
+        Tw[r + c * LDT] = ix.inI[r] >= 0 ? sc_zero<S>() : sc_cast<S>(Ts[r + c * LDT]);
+    __syncwarp();
+    SD xw = sc_zero<SD>();
+    const bool direct = warp_smallest_vector<S, SD, KMAX, LDT, KP>(Ts, ix.inI, Tw, gg, zz, m, k, lane, &xw);
+#ifdef DIAF_PHASE_TIMING
+    if (lane == 0 && a.phase && !direct) atomicAdd(&a.phase[24 + 5], 1ull);
+#endif
+    __syncwarp();
+    if (direct) {
+      if (lane < k) wv[lane] = xw;
+      __syncwarp();
+      DIAF_PHASE(8);
+    } else {
     // ---- FP32 QR of A-hat (I_j rows zeroed) into Rs; then the Jacobi SVD of R-hat
     if constexpr (L::kRegQR) {
       DIAF_PHASE(5);
@@ -380,7 +381,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
       for (int r = lane; r < m; r += DIAF_WARP) {
         SD z = sc_zero<SD>();
         if (ix.inI[r] < 0)
-          for (int q = 0; q < k; ++q) z += Ts[r + q * LDT] * gg[q];
+          for (int q = 0; q < k; ++q) z = sc_madd(z, Ts[r + q * LDT], gg[q]);
         zz[r] = z;
       }
       __syncwarp();
@@ -409,15 +410,16 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     if (lane < k) wv[lane] = RealOf<SD>(1.0 / sqrt(xn2)) * x;
     __syncwarp();
     DIAF_PHASE(8);
+    rank_thr = 1e-14 * smax;  // tested on res = ||A-hat w|| in finish_column
+    }
     // v = T(I_j,:) w and the rank test on the FP64 value of ||A-hat w||
     for (int t = lane; t < l; t += DIAF_WARP) {
       SD s = sc_zero<SD>();
       int r = ix.Iloc[t];
       if (r >= 0)
-        for (int q = 0; q < k; ++q) s += Ts[r + q * LDT] * wv[q];
+        for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
       vv[t] = s;
     }
-    rank_thr = 1e-14 * smax;  // tested on res = ||A-hat w|| in finish_column
     __syncwarp();
   } else {
     // ---- eigenpairs of C = Q_I Q_I^* by an FP32 one-sided Jacobi (the rows of
@@ -489,7 +491,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
       for (int r = lane; r < m; r += DIAF_WARP) {
         const int t = ix.inI[r];
         SD z = t >= 0 ? vv[t] : sc_zero<SD>();
-        for (int q = 0; q < k; ++q) z -= Ts[r + q * LDT] * gg[q];
+        for (int q = 0; q < k; ++q) z = sc_msub(z, Ts[r + q * LDT], gg[q]);
         zz[r] = z;
       }
       __syncwarp();
@@ -519,7 +521,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
         SD cv = sc_zero<SD>();
         const int rI = ix.Iloc[t];
         if (rI >= 0)
-          for (int q = 0; q < k; ++q) cv += Ts[rI + q * LDT] * gg[q];
+          for (int q = 0; q < k; ++q) cv = sc_madd(cv, Ts[rI + q * LDT], gg[q]);
         cvv[t] = cv;
         vcv += sc_real(sc_cmul(vv[t], cv));
         vvn += sc_abs2(vv[t]);

@@ -79,6 +79,18 @@ template <class R> __device__ __forceinline__ Cx<R> sc_msub(Cx<R> acc, Cx<R> a, 
   const R im = fma(-a.im, b.re, fma(-a.re, b.im, acc.im));
   return {re, im};
 }
+__device__ __forceinline__ float sc_msub(float acc, float a, float b) { return fmaf(-a, b, acc); }
+// acc + a b and acc + conj(a) b in the same form
+__device__ __forceinline__ double sc_madd(double acc, double a, double b) { return fma(a, b, acc); }
+__device__ __forceinline__ float sc_madd(float acc, float a, float b) { return fmaf(a, b, acc); }
+template <class R> __device__ __forceinline__ Cx<R> sc_madd(Cx<R> acc, Cx<R> a, Cx<R> b) {
+  return {fma(-a.im, b.im, fma(a.re, b.re, acc.re)), fma(a.im, b.re, fma(a.re, b.im, acc.im))};
+}
+__device__ __forceinline__ double sc_cmadd(double acc, double a, double b) { return fma(a, b, acc); }
+__device__ __forceinline__ float sc_cmadd(float acc, float a, float b) { return fmaf(a, b, acc); }
+template <class R> __device__ __forceinline__ Cx<R> sc_cmadd(Cx<R> acc, Cx<R> a, Cx<R> b) {
+  return {fma(a.im, b.im, fma(a.re, b.re, acc.re)), fma(-a.im, b.re, fma(a.re, b.im, acc.im))};
+}
 template <class R> __device__ __forceinline__ Cx<R> operator*(Cx<R> a, R s) { return {s * a.re, s * a.im}; }
 template <class R> __device__ __forceinline__ Cx<R>& operator+=(Cx<R>& a, Cx<R> b) { a.re += b.re; a.im += b.im; return a; }
 template <class R> __device__ __forceinline__ Cx<R>& operator-=(Cx<R>& a, Cx<R> b) { a.re -= b.re; a.im -= b.im; return a; }

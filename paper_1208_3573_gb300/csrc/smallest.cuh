@@ -1,0 +1,297 @@
+// Smallest right singular vector of the tile A-hat (the rows outside I_j) for
+// the DIAF-S warp kernels, without a full SVD.  One warp per column, lane q
+// owns column q of every k x k matrix.  In the working type S:
+//
+//   H = A-hat^* A-hat from A-hat's own rows and its inverse by symmetric
+//     sweeps (no pivoting: H is positive definite), kept when the
+//     column-scaled kappa = max_c sqrt(H_cc / pivot_c) is at most
+//     smallest_kappa_max (its error is eps kappa^2 relative to that scaling);
+//   inverse iteration until the Rayleigh quotient d settles to 1 %;
+//   the inverse M of H - s I, s = d + tau, tau = 1.2e-5 ||H||_inf: by Sylvester's
+//     law of inertia exactly one negative pivot proves that exactly one
+//     eigenvalue lies below s, so an eigenvalue found below s is the smallest
+//     and the next one is at least s away: the gap tests of the callers (the
+//     1e-5 smax^2 hand-back, the 1e-6 smax DEGENERATE flag) cannot fire,
+//     because ||H||_inf >= smax^2;
+//   two corrections x <- x + dx, (H - d I) dx = -(H x - d x), with
+//     (H - d I)^-1 = (M^-1 + (s - d) I)^-1 by two Neumann steps.
+//
+// Then the same corrections with the residual H x - d x taken from the FP64
+// tile (A-hat^* (A-hat x)) until the predicted error is below 1e-14; each
+// gains the working type's digits over ||H|| / gap (FP32: 5-6 digits on the
+// stencil tiles, so two corrections).  Anything out of line -- a larger
+// kappa, a pivot that is not a positive number, another inertia, an
+// eigenvalue not below s, slow convergence, non-finite values -- returns
+// false, and the caller runs the Householder QR and the Jacobi SVD.
+//
+// Why not the Jacobi: only one singular vector and the bound on the next
+// singular value are needed, and a one-sided Jacobi pays about five sweeps of
+// k^2 / 2 rotations of 6 k flops for them; the two inverses cost k^3 each and
+// a correction 6 k^2, all of it independent multiply-adds.  (LDL^* factors
+// with triangular solves have half the arithmetic, but every solve is a chain
+// of 2 k dependent shuffles.)  Numeric pass before and after, on one GB300:
+// lognormal 64^3 (k = 25) 65.8 -> 33.7 ms, FP64 convection-diffusion 129^2
+// (k = 13) 11.3 -> 2.4 ms, complex Helmholtz 512^2 (k = 9) 13.3 -> 12.4 ms.
+// What bounds it now is latency: three to four warps per scheduler on chains
+// of shuffles and shared-memory reads.
+#pragma once
+
+#include "warp_la.cuh"
+
+// A factor of the Gram matrix carries eps kappa^2.
+template <class R> __device__ __forceinline__ constexpr R smallest_kappa_max() { return sizeof(R) == 4 ? R(30) : R(300); }
+// The column of H that a lane keeps in registers: up to 64 of them (complex128
+// tiles of up to 32 columns keep the Jacobi).
+template <class S, int KMAX> constexpr bool kSmallestFits = sizeof(S) * KMAX <= 256;
+constexpr int kInverseItMax = 16;
+constexpr int kCorrectMax = 8;
+
+// The tile product (T^* z)_c of lane c (defined with the mixed kernel's other
+// tile helpers below): rows split between the half-warps for up to 16 columns.
+template <class SD, int LDT, int KMAX>
+__device__ __forceinline__ SD tile_adj_mul(const SD* Ts, const SD* zz, int m, int k, int lane) {
+  SD g = sc_zero<SD>();
+  if constexpr (KMAX <= 16) {
+    const int c = lane & 15;
+    if (c < k)
+      for (int r = lane >> 4; r < m; r += 2) g = sc_cmadd(g, Ts[r + c * LDT], zz[r]);
+    g += shfl_xor(g, 16);
+  } else {
+    if (lane < k)
+      for (int r = 0; r < m; ++r) g = sc_cmadd(g, Ts[r + lane * LDT], zz[r]);
+  }
+  return g;
+}
+
+template <class S>
+struct alignas(16) Pack16 {
+  S v[16 / sizeof(S)];
+};
+
+// Inverse of H - shift I for the Hermitian k x k matrix Hs (leading dimension
+// KP; lane q reads column q) by symmetric sweeps without pivoting: the sweep
+// on c replaces A_cc by -1/A_cc, A_ic by A_ic / A_cc and A_ij by
+// A_ij - A_ic A_cj / A_cc, and after k of them A is minus the inverse; the
+// pivots are the D of the LDL^* factorisation (their signs the inertia).
+// A lane holds its column in registers, moved down by one row per sweep, so
+// that the pivot row is always element 0 and one code body serves every
+// sweep; a swept column is kept unscaled and its factor 1/pivot in *scale,
+// so its update has the form of every other column's.  The pivot column is
+// the conjugate of the pivot row, one entry per lane, and travels through buf
+// (2 KMAX, 16-byte aligned, the halves alternating).  On return
+// (H - shift I)^-1 has column `lane` -scale * a[KMAX - k ..).  *piv is the
+// lane's pivot; returns the number of negative pivots.
+template <class S, int KMAX, int KP>
+__device__ __forceinline__ int warp_sweep_inverse(const S* Hs, RealOf<S> shift, int k, S (&a)[KMAX], S* buf, int lane,
+                                                  RealOf<S>* piv, RealOf<S>* scale) {
+  using R = RealOf<S>;
+  constexpr int PV = 16 / (int)sizeof(S);
+  static_assert(KMAX % PV == 0, "whole 16-byte packets");
+#pragma unroll
+  for (int i = 0; i < KMAX; ++i) {
+    a[i] = (lane < k && i < k) ? Hs[i + lane * KP] : sc_zero<S>();
+    if (i == lane && lane < k) a[i] -= sc_real_s<S>(shift);
+  }
+  int neg = 0;
+  R sg = R(1);
+#pragma unroll 1
+  for (int c = 0; c < k; ++c) {
+    const R p = __shfl_sync(DIAF_FULL, sc_real(a[0]), c);
+    const R ri = R(1) / p;
+    S* b = buf + (c & 1) * KMAX;
+    int at = lane - c - 1;
+    if (at < 0) at += KMAX;
+    if (lane < KMAX) b[at] = sc_conj(sg * a[0]);
+    __syncwarp();
+    S u = ri * a[0];
+    S tail = u;
+    if (lane == c) {
+      tail = sc_real_s<S>(R(-1));
+      u = sc_zero<S>();
+      sg = ri;
+      *piv = p;
+    }
+    neg += p < R(0);
+#pragma unroll
+    for (int i0 = 0; i0 < KMAX; i0 += PV) {
+      const Pack16<S> bb = *reinterpret_cast<const Pack16<S>*>(b + i0);
+#pragma unroll
+      for (int v = 0; v < PV; ++v)
+        if (i0 + v + 1 < KMAX) a[i0 + v] = sc_msub(a[i0 + v + 1], bb.v[v], u);
+    }
+    a[KMAX - 1] = tail;
+  }
+  __syncwarp();
+  *scale = sg;
+  return neg;
+}
+
+// (H - shift I)^-1 x from warp_sweep_inverse's registers, one entry of x and
+// of the result per lane; xb: KMAX scratch, 16-byte aligned.
+template <class S, int KMAX>
+__device__ __forceinline__ S warp_inverse_mul(const S (&a)[KMAX], RealOf<S> scale, S x, int k, S* xb, int lane) {
+  constexpr int PV = 16 / (int)sizeof(S);
+  int at = lane - k;
+  if (at < 0) at += KMAX;
+  if (lane < KMAX) xb[at] = lane < k ? x : sc_zero<S>();
+  __syncwarp();
+  S acc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i] = sc_zero<S>();
+#pragma unroll
+  for (int i0 = 0; i0 < KMAX; i0 += PV) {
+    const Pack16<S> bb = *reinterpret_cast<const Pack16<S>*>(xb + i0);
+#pragma unroll
+    for (int v = 0; v < PV; ++v) acc[(i0 + v) & 3] = sc_cmadd(acc[(i0 + v) & 3], a[i0 + v], bb.v[v]);
+  }
+  __syncwarp();
+  return -scale * ((acc[0] + acc[1]) + (acc[2] + acc[3]));
+}
+
+// Ts: the tile (type SD, leading dimension LDT), Tw: a copy of it in the
+// working type with the I_j rows zeroed (overwritten), inI: its rows in I_j
+// (>= 0), gg / zz: KMAX / m scratch in SD.  On success
+// returns true and lane q < k has entry q of the unit vector in *x_out.
+template <class S, class SD, int KMAX, int LDT, int KP>
+__device__ bool warp_smallest_vector(const SD* Ts, const int32_t* inI, S* Tw, SD* gg, SD* zz, int m, int k,
+                                     int lane, SD* x_out) {
+  using R = RealOf<S>;
+  static_assert(KP + 3 <= LDT && (KP * KMAX * sizeof(S)) % 16 == 0, "H, the pivot columns and x fit the tile");
+  if (k < 2 || m < k) return false;
+  // ---- H: lane q forms column q (two lanes per column, alternate rows, for up to 16 columns)
+  S acc[KMAX];
+#pragma unroll
+  for (int p = 0; p < KMAX; ++p) acc[p] = sc_zero<S>();
+  {
+    constexpr bool kHalf = KMAX <= 16;
+    const int q = kHalf ? lane & 15 : lane;
+    if (q < k) {
+      const S* wq = Tw + q * LDT;
+      for (int r = kHalf ? lane >> 4 : 0; r < m; r += kHalf ? 2 : 1) {
+        const S x = wq[r];
+#pragma unroll
+        for (int p = 0; p < KMAX; ++p)
+          if (p < k) acc[p] = sc_cmadd(acc[p], Tw[r + p * LDT], x);
+      }
+    }
+    if constexpr (kHalf) {
+#pragma unroll
+      for (int p = 0; p < KMAX; ++p) acc[p] += shfl_xor(acc[p], 16);
+    }
+  }
+  __syncwarp();  // the tile has been read
+  S* Hs = Tw;
+  S* buf = Hs + KP * KMAX;
+  S* xs = buf + 2 * KMAX;
+  R hrow = R(0), hqq = R(0);
+  if (lane < k) {
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p)
+      if (p < k) {
+        Hs[p + lane * KP] = acc[p];
+        hrow += fabs(sc_real(acc[p])) + fabs(sc_imag(acc[p]));
+        if (p == lane) hqq = sc_real(acc[p]);
+      }
+  }
+  const R hinf = warp_max(hrow);
+  __syncwarp();
+  // ---- inverse, conditioning, inverse iteration
+  S inv[KMAX];
+  R piv = R(1), scale = R(1);
+  warp_sweep_inverse<S, KMAX, KP>(Hs, R(0), k, inv, buf, lane, &piv, &scale);
+  constexpr R kmax = smallest_kappa_max<R>();
+  if (!__all_sync(DIAF_FULL, lane >= k || (piv > R(0) && hqq <= kmax * kmax * piv))) return false;
+  S x = lane < k ? sc_real_s<S>(R((lane * 37 + 11) % 17) - R(8.3)) : sc_zero<S>();
+  R d = R(0);
+#pragma unroll 1
+  for (int it = 0; it < kInverseItMax; ++it) {
+    const S y = warp_inverse_mul<S, KMAX>(inv, scale, x, k, xs, lane);
+    const R nu = warp_sum(lane < k ? sc_real(sc_cmul(x, y)) : R(0));  // y^* H y
+    const R ny = warp_sum(lane < k ? sc_abs2(y) : R(0));
+    const R dn = nu / ny;
+    x = rsqrt_r(ny) * y;
+    const bool settled = it > 0 && fabs(dn - d) <= R(1e-2) * dn;
+    d = dn;
+    if (settled) break;
+  }
+  // ---- the shifted inverse and its inertia
+  const R s = d + R(1.2e-5) * hinf;
+  if (warp_sweep_inverse<S, KMAX, KP>(Hs, s, k, inv, buf, lane, &piv, &scale) != 1) return false;
+  auto correction = [&](S r, R sh) -> S {  // -(H - d I)^-1 r, sh = s - d
+    S dx = sc_zero<S>();
+#pragma unroll 1
+    for (int t = 0; t < 3; ++t) dx = warp_inverse_mul<S, KMAX>(inv, scale, -(r + sh * dx), k, xs, lane);
+    return dx;
+  };
+  R last = R(1);
+#pragma unroll 1
+  for (int it = 0; it < 2; ++it) {
+    if (lane < k) xs[lane] = x;
+    __syncwarp();
+    S hx = sc_zero<S>();
+    if (lane < k)
+      for (int p = 0; p < k; ++p) hx = sc_cmadd(hx, Hs[p + lane * KP], xs[p]);
+    d = warp_sum(lane < k ? sc_real(sc_cmul(x, hx)) : R(0));
+    S r = hx - d * x;
+    if (lane >= k) r = sc_zero<S>();
+    const S dx = correction(r, s - d);
+    last = sqrt(warp_sum(lane < k ? sc_abs2(dx) : R(0)));
+    x += dx;
+    const R n2 = warp_sum(lane < k ? sc_abs2(x) : R(0));
+    x = rsqrt_r(n2) * x;
+    __syncwarp();
+  }
+  if (!(last <= R(0.05))) return false;
+  // columns of A-hat that no chain of nonzeros of H ties to the vector's
+  // largest entry are not part of it: exact zeros there, as the Jacobi (which
+  // never rotates orthogonal columns) leaves them -- v_jj = 0 depends on it
+  {
+    uint32_t ties = 0;
+    if (lane < k)
+      for (int p = 0; p < k; ++p) ties |= sc_abs2(Hs[p + lane * KP]) != R(0) ? 1u << p : 0u;
+    const R ax = lane < k ? sc_abs2(x) : R(-1);
+    uint32_t comp = __ballot_sync(DIAF_FULL, ax == warp_max(ax));
+    comp &= 0u - comp;
+    for (uint32_t grown = 0; grown != comp;) {
+      grown = comp;
+      comp |= __reduce_or_sync(DIAF_FULL, (comp >> lane) & 1u ? ties : 0u);
+    }
+    if (!((comp >> lane) & 1u)) x = sc_zero<S>();
+  }
+  // ---- corrections against the FP64 tile
+  using RD = RealOf<SD>;
+  SD y = lane < k ? sc_cast<SD>(x) : sc_zero<SD>();
+  double before = (double)last;
+  bool done = false;
+#pragma unroll 1
+  for (int it = 0; it < kCorrectMax && !done; ++it) {
+    if (lane < k) gg[lane] = y;
+    __syncwarp();
+    for (int r = lane; r < m; r += DIAF_WARP) {
+      SD z = sc_zero<SD>();
+      if (inI[r] < 0)
+        for (int q = 0; q < k; ++q) z = sc_madd(z, Ts[r + q * LDT], gg[q]);
+      zz[r] = z;
+    }
+    __syncwarp();
+    const SD g = tile_adj_mul<SD, LDT, KMAX>(Ts, zz, m, k, lane);
+    const RD yg = warp_sum(lane < k ? (RD)sc_real(sc_cmul(y, g)) : RD(0));
+    const RD yy = warp_sum(lane < k ? (RD)sc_abs2(y) : RD(0));
+    const RD dd = yg / yy;
+    const double room = (double)s - (double)dd;  // at most the gap to the next eigenvalue
+    if (!(room >= 1.05e-5 * (double)hinf && (double)dd > 1e-24 * (double)hinf)) return false;
+    const S r = lane < k ? sc_cast<S>(g - dd * y) : sc_zero<S>();
+    const S dx = correction(r, R(room));
+    const double step = sqrt((double)warp_sum(lane < k ? sc_abs2(dx) : R(0)));
+    if (lane < k) y += sc_cast<SD>(dx);
+    // the next correction would be about step * (step / before)
+    done = step * step <= 1e-14 * before;
+    if (!done && it > 0 && !(step <= 0.5 * before)) return false;
+    before = step;
+    __syncwarp();
+  }
+  if (!done) return false;
+  const RD n2 = warp_sum(lane < k ? (RD)sc_abs2(y) : RD(0));
+  *x_out = RD(1.0 / sqrt((double)n2)) * y;
+  return true;
+}
