@@ -668,9 +668,8 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
         DIAF_CU(thread_columns_shape(M, K, np.h_bc[0], &np.tsh));
         np.ta.M = M;
         np.ta.K = K;
-        np.ta.arena = thread_arena_floats(M, K);
         np.ta.nquads = np.tsh.nquads;
-        nc.add(&np.ta.slab, (size_t)np.tsh.nquads * thread_slab_doubles(M, K));
+        nc.add(&np.ta.slab, (size_t)np.tsh.nquads * thread_slab_doubles(M, thread_instance(K)));
         nc.add(&np.ta.defer_list, np.h_bc[0]);
         np.ta.defer_count = np.work + 3 * kNumBuckets;
         np.thread_cols = np.tsh.grid > 0;

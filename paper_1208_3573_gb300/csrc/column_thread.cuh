@@ -2,37 +2,47 @@
 // tiles (k_j <= 16, m_j <= 32, the size bucket of stencil operators).
 //
 // A quad of lanes runs the whole column -- gather, FP32 Householder QR of T,
-// leverage keys, the V rule of Sec. 3.1, FP32 Householder QR of A-hat (T with
-// the I_j rows removed), cyclic one-sided Jacobi SVD of its R, the FP64
-// second-order correction of the smallest right singular vector in the FP32
-// singular basis, v = T(I_j,:) w, phase, FP64 residual and scatter -- with the
-// same arithmetic as the warp kernel of column_mixed.cuh (the same FP32
-// factorisations, key-error bound, hand-back tests and FP64 correction).  A
-// warp works on eight columns at once: lane s of a quad owns the rows
-// r = s (mod 4) of every column-major array of its column, so the per-column
-// dependency chains carry two-step quad reductions instead of warp-wide ones,
-// and no lane idles on the short vectors of these tiles.
+// leverage keys, the V rule of Sec. 3.1, the smallest right singular vector of
+// A-hat (T with the I_j rows removed), v = T(I_j,:) w, phase, FP64 residual
+// and scatter -- with the same arithmetic as the warp kernel of
+// column_mixed.cuh (the same FP32 factorisations, key-error bound, hand-back
+// tests, and the method of smallest.cuh for the singular vector).  A warp
+// works on eight columns at once: lane s of a quad owns the rows r = s (mod 4)
+// of the tile and of every k x k matrix, so the per-column dependency chains
+// carry two-step quad reductions instead of warp-wide ones, and no lane idles
+// on the short vectors of these tiles.
 //
-// Storage: the FP32 working matrix, keys and Jacobi norms in shared memory,
-// element e of quad c at smem[32 (e / 4) + 8 (e mod 4) + c] (the 32 lanes of
-// a warp reading four consecutive elements each hit 32 distinct banks); the
-// FP64 tile in a global slab laid out the same way across all quads of the
-// grid (coalesced); the k-vectors of the FP64 correction in registers.
+// Storage: FP32 arrays in shared memory, element e of quad c at
+// smem[32 (e / 4) + 8 (e mod 4) + c] (the 32 lanes of a warp reading four
+// consecutive elements each hit 32 distinct banks); the FP64 tile in a global
+// slab, four rows of one column side by side, interleaved across all quads of
+// the grid (coalesced).  The kernel is instantiated for KMAX = 8, 13 and 16
+// columns: the k x k matrices are swept and multiplied in registers with
+// static indices (rows and columns from k on are an identity block), so a
+// tile pays for KMAX columns.
 //
 // A column this kernel does not finish itself -- an empty or fixed-pattern
 // column, a tile beyond its capacity or with fewer rows than columns, a tile
 // too ill-conditioned for the FP32 factors, FP32 keys that cannot decide I_j,
-// a singular gap too small for the correction -- goes to the defer list, which
-// the warp kernel of column_mixed.cuh then runs (with its own FP64 keys and
-// FP64 hand-back).
+// a smallest singular vector out of the direct method's reach -- goes to the
+// defer list, which the warp kernel of column_mixed.cuh then runs (with its
+// own FP64 keys, Jacobi and FP64 hand-back).
+//
+// What it replaced: a one-sided Jacobi SVD of the R of a second Householder QR
+// took 52 % of the cycles and the correction in its basis 20 %.  Numeric pass on
+// convection-diffusion 256^2 (25 x 13 tiles) 1.40 -> 0.72 ms, 843 -> 253 M
+// instructions; power-law bucket 0 (k = 3 .. 16) 3.6 -> 2.2 ms.  What bounds it
+// now is latency (30 % of the issue slots, 16 warps per SM by registers and by
+// shared memory): waits on shared memory and shuffles, then on the slab, with
+// 35 % of the cycles in the FP64 corrections (two passes over the tile at 1/64
+// of the FP32 rate).
 #pragma once
 
 #include "column.cuh"
 
 struct ThreadArgs {
   int M, K;              // capacity of this launch (rows, columns)
-  int arena;             // shared-memory floats per column
-  double* slab;          // FP64 per quad of the grid: the tile T (M * K) and z (M), thread_slab_doubles
+  double* slab;          // FP64 tile per quad of the grid: thread_slab_doubles each
   int nquads;            // quads of the grid (the slab's interleave)
   int32_t* defer_list;   // columns left to the warp kernel
   int32_t* defer_count;
@@ -43,20 +53,26 @@ constexpr int kQuad = 4;            // lanes per column
 constexpr int kQuadCols = 8;        // columns per warp
 constexpr int kQuadWarps = 1;       // warps per block
 
-// Shared-memory floats per column for capacity (M, K): the working matrix
-// max(M K, 2 K^2), keys (M), Jacobi norms (K); rounded up to whole rows of 4.
-__host__ __device__ constexpr int thread_arena_floats(int M, int K) {
-  return ((M * K > 2 * K * K ? M * K : 2 * K * K) + M + K + 3) / 4 * 4;
+// Columns of the kernel instance for tiles of at most K columns.
+__host__ __device__ constexpr int thread_instance(int K) { return K <= 8 ? 8 : (K <= 13 ? 13 : 16); }
+
+// Shared-memory floats per column for capacity (M, K) of the KMAX instance:
+// first the QR's M x K matrix, the keys (M) and the gather's K column ranges
+// (8 bytes each, 8-byte aligned); then the rows of A-hat, 4 ceil(KMAX / 4)
+// floats each; then H or its inverse (KMAX columns of 4 ceil(KMAX / 4) rows)
+// and the FP64 vector x (KMAX), in whole groups of 4 elements.
+__host__ __device__ constexpr int thread_arena_floats(int M, int K, int KMAX) {
+  const int ku = (KMAX + 3) / 4;
+  const int a = (M * K + M + 3) / 4 * 4 + 2 * ((K + 3) / 4 * 4);
+  const int b = M * 4 * ku;
+  const int c = 4 * ku * KMAX + 2 * 4 * ku;
+  return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
-// FP64 shared-memory scratch per column: the refined vector x (K), rounded
-// up to whole rows of 4.
-__host__ __device__ constexpr int thread_arena_doubles(int M, int K) { return (void)M, (K + 3) / 4 * 4; }
-// FP64 slab doubles per quad: the tile T (M K) and z = A-hat x (M), each
-// rounded up to whole rows of 4.
-__host__ __device__ constexpr int thread_slab_doubles(int M, int K) { return (M * K + 3) / 4 * 4 + (M + 3) / 4 * 4; }
+// FP64 slab doubles per quad: row r of column q at 4 ((r / 4) KMAX + q) + r mod 4.
+__host__ __device__ constexpr int thread_slab_doubles(int M, int KMAX) { return (M + 3) / 4 * KMAX * 4; }
 // Shared-memory bytes of one warp (eight columns).
-__host__ __device__ constexpr size_t thread_warp_smem(int M, int K) {
-  return sizeof(float) * (size_t)thread_arena_floats(M, K) * 8 + sizeof(double) * (size_t)thread_arena_doubles(M, K) * 8;
+__host__ __device__ constexpr size_t thread_warp_smem(int M, int K, int KMAX) {
+  return sizeof(float) * (size_t)thread_arena_floats(M, K, KMAX) * 8;
 }
 
 // Element e of this quad's interleaved shared-memory array (base already
@@ -76,19 +92,7 @@ __device__ __forceinline__ double qsum(double v, unsigned qm) {
   return v;
 }
 
-// Round-robin Jacobi schedule of the warp kernels for qq = 2, 4, ..., 16
-// columns (k rounded up to even): kPairTab[qq/2 - 1][round][pair] = (a << 4) | b,
-// with b >= k marking a bye; filled once on the host.
-constexpr int kPairRounds = kThreadKMax - 1, kPairSlots = kThreadKMax / 2;
-static __constant__ uint8_t kPairTab[kThreadKMax / 2][kPairRounds][kPairSlots];
-
 constexpr int kQR = kThreadMMax / 4;  // most rows a lane owns in a column of the tile
-#ifndef DIAF_QUAD_JACOBI_PAIRS
-#define DIAF_QUAD_JACOBI_PAIRS 4
-#endif
-constexpr int kJP = DIAF_QUAD_JACOBI_PAIRS;  // disjoint pairs of a round rotated together
-constexpr int kQK = kThreadKMax / 4;  // most rows a lane owns in a column of a k x k matrix
-
 // Householder QR in place of the m x k column-major matrix at W (ld m,
 // m >= k), FP32: reflector c maps W(c:m, c) to beta e_1 (the reflectors of
 // warp_householder_qr).  Lane `sub` works on its rows (held in registers for
@@ -134,9 +138,104 @@ __device__ __forceinline__ void quad_qr(float* W, int m, int k, int sub, unsigne
   __syncwarp(qm);
 }
 
+// Inverse of H - shift I by symmetric sweeps (smallest.cuh), the rows spread
+// over the quad: lane `sub` holds rows sub + 4u in a[u], moved one column to
+// the left per sweep so that the pivot column is always element 0; a swept row
+// is kept unscaled and its factor 1/pivot in sg[u].  The pivot row goes round
+// by shuffles.  H: element (u, q) of lane `sub` at H[32 (u KMAX + q)] (base
+// offset by 8 sub).  piv[u] receives the pivots; the inverse's row sub + 4u is
+// -sg[u] a[u].
 template <int KMAX>
-__device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j, float* S, double* D, double* G,
-                                  int sub, unsigned qm) {
+__device__ __forceinline__ void quad_sweep_inverse(const float* H, float shift, float (&a)[(KMAX + 3) / 4][KMAX],
+                                                   float (&piv)[(KMAX + 3) / 4], float (&sg)[(KMAX + 3) / 4], int sub,
+                                                   unsigned qm) {
+  constexpr int KU = (KMAX + 3) / 4;
+#pragma unroll
+  for (int u = 0; u < KU; ++u) {
+    sg[u] = 1.0f;
+    piv[u] = 1.0f;
+#pragma unroll
+    for (int q = 0; q < KMAX; ++q) {
+      a[u][q] = H[32 * (u * KMAX + q)];
+      if ((q >> 2) == u && (q & 3) == sub) a[u][q] -= shift;
+    }
+  }
+#pragma unroll
+  for (int uc = 0; uc < KU; ++uc) {  // pivot column c = 4 uc + sc
+    constexpr int kLast = KMAX - 4 * (KU - 1);  // columns of the last group
+#pragma unroll 1
+    for (int sc = 0; sc < (uc == KU - 1 ? kLast : 4); ++sc) {
+      float b[KMAX];
+#pragma unroll
+      for (int q = 0; q < KMAX; ++q) b[q] = __shfl_sync(qm, a[uc][q], sc, 4);
+      const float ri = __fdividef(1.0f, b[0]);
+      float f[KU];
+#pragma unroll
+      for (int u = 0; u < KU; ++u) f[u] = a[u][0] * ri;
+      const bool own = sub == sc;
+      const float tail = own ? -1.0f : f[uc];
+      if (own) {
+        piv[uc] = b[0];
+        sg[uc] = ri;
+        f[uc] = 0.0f;
+      }
+#pragma unroll
+      for (int u = 0; u < KU; ++u) {
+#pragma unroll
+        for (int q = 0; q + 1 < KMAX; ++q) a[u][q] = fmaf(-f[u], b[q + 1], a[u][q + 1]);
+        a[u][KMAX - 1] = u == uc ? tail : f[u];
+      }
+    }
+  }
+}
+
+// y = (matrix) x for x and y spread over the quad like the rows; the lane's
+// element (row sub + 4u, column q) in registers, or in shared memory at
+// H[32 (u KMAX + q)].
+template <int KMAX>
+__device__ __forceinline__ void quad_mul_reg(const float (&a)[(KMAX + 3) / 4][KMAX], const float (&x)[(KMAX + 3) / 4],
+                                             float (&y)[(KMAX + 3) / 4], unsigned qm) {
+  constexpr int KU = (KMAX + 3) / 4;
+  float t[KU];
+#pragma unroll
+  for (int u = 0; u < KU; ++u) t[u] = 0.0f;
+#pragma unroll
+  for (int q = 0; q < KMAX; ++q) {
+    const float xq = __shfl_sync(qm, x[q >> 2], q & 3, 4);
+#pragma unroll
+    for (int u = 0; u < KU; ++u) t[u] = fmaf(a[u][q], xq, t[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < KU; ++u) y[u] = t[u];
+}
+template <int KMAX>
+__device__ __forceinline__ void quad_mul_smem(const float* H, const float (&x)[(KMAX + 3) / 4],
+                                              float (&y)[(KMAX + 3) / 4], unsigned qm) {
+  constexpr int KU = (KMAX + 3) / 4;
+  float t[KU];
+#pragma unroll
+  for (int u = 0; u < KU; ++u) t[u] = 0.0f;
+#pragma unroll
+  for (int q = 0; q < KMAX; ++q) {
+    const float xq = __shfl_sync(qm, x[q >> 2], q & 3, 4);
+#pragma unroll
+    for (int u = 0; u < KU; ++u) t[u] = fmaf(H[32 * (u * KMAX + q)], xq, t[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < KU; ++u) y[u] = t[u];
+}
+
+template <int KU>
+__device__ __forceinline__ float quad_dot(const float (&x)[KU], const float (&y)[KU], unsigned qm) {
+  float s = 0.0f;
+#pragma unroll
+  for (int u = 0; u < KU; ++u) s = fmaf(x[u], y[u], s);
+  return qsum(s, qm);
+}
+
+template <int KMAX>
+__device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j, float* S, double* G, int sub,
+                                  unsigned qm) {
   static_assert(KMAX <= kThreadKMax, "tile capacity");
   const int k = a.Wcp[j + 1] - a.Wcp[j];
   const int m = a.m[j];
@@ -152,15 +251,11 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
     defer();
     return;
   }
-  const int M = ta.M, K = ta.K;
-  const int wsz = M * K > 2 * K * K ? M * K : 2 * K * K;
-  float* W = S;  // working matrix at element 0, keys at wsz, Jacobi norms at wsz + M
-  const int HK = wsz, NR = wsz + M;
-  // FP64 tile (ld m): element e of this quad at G[(e / 4) 4 nquads + (e mod 4)],
-  // element e + 4u at gptr(e)[u gstride]
+  constexpr int KU = (KMAX + 3) / 4;  // rows of a k x k matrix a lane owns
+  float* W = S;            // QR working matrix (ld m), keys from element HK on
+  const int HK = ta.M * ta.K;
+  // FP64 tile: rows 4t .. 4t + 3 of column q at G[(t KMAX + q) gstride .. + 3]
   const size_t gstride = (size_t)4 * ta.nquads;
-  auto gptr = [&](int e) { return G + (size_t)(e >> 2) * gstride + (e & 3); };
-  auto T = [&](int e) -> double& { return *gptr(e); };
   const int nown = (m - sub + 3) >> 2;  // own tile rows: sub, sub + 4, ...
   DIAF_PHASE_START();
 
@@ -172,20 +267,21 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
   const double* Av = reinterpret_cast<const double*>(a.Av);
   auto RS = [&](int r) -> int32_t& { return *reinterpret_cast<int32_t*>(qptr(W, HK + r)); };
   for (int r = sub; r < m; r += 4) RS(r) = Rj[r];
-  // the entry range of A(:, J_j[q]) as an int pair in FP64 scratch slot q
-  // (free until the correction)
-  auto CR = [&](int q) -> int2& { return *reinterpret_cast<int2*>(qptr(D, q)); };
+  // the entry range of A(:, J_j[q]) as an int pair behind the keys
+  double* const C = reinterpret_cast<double*>(S - (threadIdx.x & 31) / 4) +
+                    (size_t)((HK + ta.M + 3) / 4 * 4) * 4 + (threadIdx.x & 31) / 4;
+  auto CR = [&](int q) -> int2& { return *reinterpret_cast<int2*>(qptr(C, q)); };
   for (int q = sub; q < k; q += 4) {
     const int c = J[q];
     CR(q) = make_int2(a.Acp[c], a.Acp[c + 1]);
   }
   for (int q = 0; q < k; ++q) {
-    double* gq = gptr(q * m + sub);
+    double* gq = G + q * gstride + sub;
     float* wq = qptr(W, q * m + sub);
 #pragma unroll
     for (int t = 0; t < kQR; ++t)
       if (t < nown) {
-        gq[t * gstride] = 0.0;
+        gq[t * KMAX * gstride] = 0.0;
         wq[32 * t] = 0.0f;
       }
   }
@@ -205,7 +301,7 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
         }
       }
       const double v = Av[p];
-      T(r + q * m) = v;
+      G[((r >> 2) * KMAX + q) * gstride + (r & 3)] = v;
       QS(W, r + q * m) = (float)v;
     }
   }
@@ -250,8 +346,10 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
     const bool two = t + 1 < nown;
     float z[KMAX], y[KMAX];
     float h = 0.0f, h1 = 0.0f;
+    const double* g0 = G + t * KMAX * gstride + sub;
+    const double* g1 = g0 + KMAX * gstride;
 #pragma unroll
-    for (int c = 0; c < KMAX; ++c) {
+    for (int c = 0; c < KMAX; ++c, g0 += gstride, g1 += gstride) {
       z[c] = 0.0f;
       y[c] = 0.0f;
       if (c < k) {
@@ -259,8 +357,8 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
         const float* P1 = qptr(W, c * m + 1);
         const float* P2 = qptr(W, c * m + 2);
         const float* P3 = qptr(W, c * m + 3);
-        float acc = (float)T(r + c * m);
-        float acc1 = two ? (float)T(r + 4 + c * m) : 0.0f;
+        float acc = (float)*g0;
+        float acc1 = two ? (float)*g1 : 0.0f;
 #pragma unroll
         for (int p2 = 0; p2 < c; ++p2) {
           const float* P = (p2 & 3) == 0 ? P0 : ((p2 & 3) == 1 ? P1 : ((p2 & 3) == 2 ? P2 : P3));
@@ -333,356 +431,277 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
   for (int r = sub; r < m; r += 4)
     if ((inI >> r) & 1u) a.Vri[v0 + pos_of(r)] = Rj[r];
 
-  // ---- FP32 QR of A-hat (the I_j rows zeroed), its conditioning
+  // ---- A-hat's rows in FP32 (the I_j rows zeroed), row-major in groups of 4
   DIAF_PHASE(4);
-  float ch[KMAX];
-  // own rows of every column first (independent loads), the column norms
-  // from shared memory after
-  for (int q = 0; q < k; ++q) {
-    const double* gq = gptr(q * m + sub);
-    float* wq = qptr(W, q * m + sub);
-    float f[kQR];
+  __syncwarp(qm);  // the keys and the QR's matrix have been read
+  for (int t = 0; t < nown; ++t) {
+    const int r = sub + 4 * t;
+    const bool out = (inI >> r) & 1u;
+    const double* g = G + t * KMAX * gstride + sub;
+    float* row = S + r * KU * 32;
 #pragma unroll
-    for (int t = 0; t < kQR; ++t) f[t] = (t < nown && !((inI >> (sub + 4 * t)) & 1u)) ? (float)gq[t * gstride] : 0.0f;
-#pragma unroll
-    for (int t = 0; t < kQR; ++t)
-      if (t < nown) wq[32 * t] = f[t];
-  }
-#pragma unroll
-  for (int q = 0; q < KMAX; ++q) {
-    float s2 = 0.0f;
-    if (q < k) {
-      const float* wq = qptr(W, q * m + sub);
-#pragma unroll
-      for (int t = 0; t < kQR; ++t)
-        if (t < nown) s2 = fmaf(wq[32 * t], wq[32 * t], s2);
+    for (int q = 0; q < 4 * KU; ++q, g += gstride) {
+      float v = 0.0f;
+      if (q < KMAX && q < k && !out) v = (float)*g;
+      row[(q >> 2) * 32 + (q & 3) * 8] = v;
     }
-    ch[q] = 0.0f;
-    if (q < k) ch[q] = sqrtf(qsum(s2, qm));
   }
   __syncwarp(qm);
-  quad_qr(W, m, k, sub, qm);
-  float kh = 0.0f;
-  bool zdiag = false;  // R-hat singular (A-hat rank deficient): V is accumulated in the sweeps instead
-#pragma unroll
-  for (int q = 0; q < KMAX; ++q)
-    if (q < k) {
-      const float d = fabsf(QS(W, q + q * m));
-      kh = fmaxf(kh, d > 0.0f ? ch[q] / d : (ch[q] > 0.0f ? INFINITY : 0.0f));
-      zdiag |= d == 0.0f;
-    }
-  if (!(kh <= kMixedKappaMax)) { defer(); return; }
-
-  // ---- R-hat to ld k at W[0, k^2) column by column (a column's new place
+  // ---- H = A-hat^T A-hat: the lane's rows sub + 4u
   DIAF_PHASE(6);
-  // lies below every later column's old one), and a copy R0 of it at
-  // W[k^2, 2k^2) for recovering V after the sweeps.  Lane `sub` owns rows
-  // sub + 4u (u < nk) of every k x k column.
-  const int nk = (k - sub + 3) >> 2;
-  for (int c = 0; c < k; ++c) {
-    const float* src = qptr(W, c * m + sub);
-    float t4[kQK];
+  float a4[KU][KMAX];
 #pragma unroll
-    for (int u = 0; u < kQK; ++u) t4[u] = (u < nk && sub + 4 * u <= c) ? src[32 * u] : 0.0f;
-    __syncwarp(qm);
-    float* dst = qptr(W, c * k + sub);
+  for (int u = 0; u < KU; ++u)
 #pragma unroll
-    for (int u = 0; u < kQK; ++u)
-      if (u < nk) dst[32 * u] = t4[u];
-    __syncwarp(qm);
-  }
-  const int VO = k * k;  // R0, or V = I when R-hat is singular
-  for (int c = 0; c < k; ++c) {
-    const float* src = qptr(W, c * k + sub);
-    float* dst = qptr(W, VO + c * k + sub);
+    for (int q = 0; q < KMAX; ++q) a4[u][q] = 0.0f;
+  for (int r = 0; r < m; ++r) {
+    const float* row = S + r * KU * 32;
+    float own[KU];
 #pragma unroll
-    for (int u = 0; u < kQK; ++u)
-      if (u < nk) dst[32 * u] = zdiag ? (sub + 4 * u == c ? 1.0f : 0.0f) : src[32 * u];
-  }
-
-  // ---- one-sided Jacobi on R-hat in the warp kernels' round-robin order
-  DIAF_PHASE(5);
-  // (the rotations are applied to R-hat only: V is recovered afterwards from
-  // R-hat V = B as R0^-1 B, which costs one triangular solve per column
-  // instead of a second pair of column updates per rotation; a singular
-  // R-hat has no R0^-1, and then V is accumulated in the rotations)
-  // (in round rnd, position p >= 1 holds column 1 + ((p - 1 + rnd) mod L) and
-  // positions p, qq - 1 - p pair up), with their rotation and stopping rules:
-  // skip below tol = k eps_32, stop after a sweep without a rotation of
-  // |gamma|^2 >= tol alpha beta; norms carried through rotations.  The pairs
-  // of a round are disjoint: kJP of them are rotated together (independent
-  // chains).
-  // Every lane of the quad writes the same norms.
-  uint32_t flags = 0;
-  {
-    float nf2 = 0.0f;
-    for (int c = 0; c < k; ++c) {
-      const float* pc = qptr(W, c * k + sub);
+    for (int u = 0; u < KU; ++u) own[u] = row[u * 32 + sub * 8];
 #pragma unroll
-      for (int u = 0; u < kQK; ++u)
-        if (u < nk) nf2 = fmaf(pc[32 * u], pc[32 * u], nf2);
+    for (int q = 0; q < KMAX; ++q) {
+      const float v = row[(q >> 2) * 32 + (q & 3) * 8];
+#pragma unroll
+      for (int u = 0; u < KU; ++u) a4[u][q] = fmaf(own[u], v, a4[u][q]);
     }
-    nf2 = qsum(nf2, qm);
-    const float tol = (float)k * FLT_EPSILON;
-    const float tol2 = tol * tol;
-    const float tiny = tol2 * nf2;
-    const int qq = (k + 1) & ~1;
-    const int npairs = qq / 2;
-    const int L = qq - 1;
-    const uint8_t* tab = &kPairTab[npairs - 1][0][0];
-    auto pair_of = [&](int pr, int rnd) -> int2 {
-      if (pr >= npairs) return make_int2(-1, -1);
-      const int ab = tab[rnd * kPairSlots + pr];
-      const int x = ab >> 4, y = ab & 15;
-      return y < k ? make_int2(x, y) : make_int2(-1, -1);  // a bye for the padding column
-    };
-    int sweep = 1;
-    for (; sweep <= kMaxSweeps; ++sweep) {
-      for (int c = 0; c < k; ++c) {
-        const float* pc = qptr(W, c * k + sub);
-        float s2 = 0.0f;
-#pragma unroll
-        for (int u = 0; u < kQK; ++u)
-          if (u < nk) s2 = fmaf(pc[32 * u], pc[32 * u], s2);
-        QS(W, NR + c) = qsum(s2, qm);
-      }
-      bool large = false;
-      if (k >= 2) {
-        for (int rnd = 0; rnd < L; ++rnd) {
-          for (int pr = 0; pr < npairs; pr += kJP) {
-            int pa[kJP], pb[kJP];
-#pragma unroll
-            for (int h = 0; h < kJP; ++h) {
-              const int2 ph = pair_of(pr + h, rnd);
-              pa[h] = ph.x;
-              pb[h] = ph.y;
-            }
-            float xa[kJP][kQK], xb[kJP][kQK], g[kJP];
-            float *ga[kJP], *gb[kJP];
-#pragma unroll
-            for (int h = 0; h < kJP; ++h) {
-              const bool act = pb[h] >= 0;
-              ga[h] = qptr(W, (act ? pa[h] : 0) * k + sub);
-              gb[h] = qptr(W, (act ? pb[h] : 0) * k + sub);
-              g[h] = 0.0f;
-#pragma unroll
-              for (int u = 0; u < kQK; ++u) {
-                xa[h][u] = (act && u < nk) ? ga[h][32 * u] : 0.0f;
-                xb[h][u] = (act && u < nk) ? gb[h][32 * u] : 0.0f;
-                g[h] = fmaf(xa[h][u], xb[h][u], g[h]);
-              }
-            }
-#pragma unroll
-            for (int h = 0; h < kJP; ++h) g[h] += __shfl_xor_sync(qm, g[h], 1);
-#pragma unroll
-            for (int h = 0; h < kJP; ++h) g[h] += __shfl_xor_sync(qm, g[h], 2);
-#pragma unroll
-            for (int h = 0; h < kJP; ++h) {
-              if (pb[h] < 0) continue;
-              const float al = QS(W, NR + pa[h]), be = QS(W, NR + pb[h]);
-              const float g2 = g[h] * g[h];
-              if (!(al > tiny && be > tiny && g2 > 0.0f && g2 > tol2 * (al * be))) continue;
-              if (g2 >= tol * (al * be)) large = true;
-              const float ag = fabsf(g[h]);
-              const float d = be - al;
-              const float t = __fdividef(copysignf(2.0f * ag, d), fabsf(d) + sqrtf(d * d + 4.0f * g2));
-              const float cs = rsqrtf(1.0f + t * t), sn = cs * t;
-              const float ssn = g[h] < 0.0f ? -sn : sn, scs = g[h] < 0.0f ? -cs : cs;  // y = sign(g) b
-#pragma unroll
-              for (int u = 0; u < kQK; ++u)
-                if (u < nk) {
-                  ga[h][32 * u] = fmaf(-ssn, xb[h][u], cs * xa[h][u]);
-                  gb[h][32 * u] = fmaf(scs, xb[h][u], sn * xa[h][u]);
-                }
-              if (zdiag) {  // V accumulated: R0^-1 B does not exist
-                float* va = qptr(W, VO + pa[h] * k + sub);
-                float* vb = qptr(W, VO + pb[h] * k + sub);
-#pragma unroll
-                for (int u = 0; u < kQK; ++u)
-                  if (u < nk) {
-                    const float xv = va[32 * u], yv = vb[32 * u];
-                    va[32 * u] = fmaf(-ssn, yv, cs * xv);
-                    vb[32 * u] = fmaf(scs, yv, sn * xv);
-                  }
-              }
-              QS(W, NR + pa[h]) = al - t * ag;
-              QS(W, NR + pb[h]) = be + t * ag;
-            }
-          }
-        }
-      }
-      if (!large) break;
-    }
-    if (sweep > kMaxSweeps) flags |= DIAF_FLAG_JACOBI_NOCONV;
   }
-  __syncwarp(qm);
-
-  // ---- singular values (column norms of R-hat V), the smallest and its gap
+  __syncwarp(qm);  // the rows have been read
+  float hinf = 0.0f, hd[KU];
+#pragma unroll
+  for (int u = 0; u < KU; ++u) {
+    float hs = 0.0f;
+    hd[u] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < KMAX; ++q) {
+      hs += fabsf(a4[u][q]);
+      if ((q >> 2) == u && (q & 3) == sub) hd[u] = a4[u][q];
+    }
+    hinf = fmaxf(hinf, hs);
+  }
+  hinf = fmaxf(hinf, __shfl_xor_sync(qm, hinf, 1));
+  hinf = fmaxf(hinf, __shfl_xor_sync(qm, hinf, 2));
+  // an exactly zero column of A-hat (all its entries in I_j) is an exact zero
+  // singular value with w = e_c: only the gap to the others is left to check
+  uint32_t zeros = 0;
+  float* const Hs = S + sub * 8;
+#pragma unroll
+  for (int u = 0; u < KU; ++u) {
+    const int row = sub + 4 * u;
+    const bool zero = row < k && hd[u] == 0.0f;
+    if (zero) zeros |= 1u << row;
+    const bool pad = zero || row >= k;  // those rows: a diagonal of the others' size
+    if (pad) hd[u] = hinf;
+#pragma unroll
+    for (int q = 0; q < KMAX; ++q)
+      Hs[32 * (u * KMAX + q)] = (pad && (q >> 2) == u && (q & 3) == sub) ? hinf : a4[u][q];
+  }
+  zeros |= __shfl_xor_sync(qm, zeros, 1);
+  zeros |= __shfl_xor_sync(qm, zeros, 2);
+  if ((zeros & (zeros - 1u)) != 0 || !(hinf > 0.0f)) { defer(); return; }
+  float piv[KU], sg[KU], x[KU];
+  float s = 1.2e-5f * hinf;  // the shift; d is added unless there is a zero column
+  auto conditioned = [&]() {  // column-scaled kappa <= kGramKappaMax from the pivots
+    bool ok = true;
+#pragma unroll
+    for (int u = 0; u < KU; ++u)
+      ok &= sub + 4 * u >= k || (piv[u] > 0.0f && hd[u] <= kGramKappaMax * kGramKappaMax * piv[u]);
+    return (__ballot_sync(qm, ok) & qm) == qm;
+  };
+  if (zeros == 0) {
+    DIAF_PHASE(5);
+    quad_sweep_inverse<KMAX>(Hs, 0.0f, a4, piv, sg, sub, qm);
+    if (!conditioned()) { defer(); return; }
+#pragma unroll
+    for (int u = 0; u < KU; ++u) x[u] = sub + 4 * u < k ? (float)(((sub + 4 * u) * 37 + 11) % 17) - 8.3f : 0.0f;
+    float d = 0.0f;
+#pragma unroll 1
+    for (int it = 0; it < kInverseItMax; ++it) {
+      float y[KU];
+      quad_mul_reg<KMAX>(a4, x, y, qm);
+#pragma unroll
+      for (int u = 0; u < KU; ++u) y[u] *= -sg[u];
+      const float nu = quad_dot<KU>(x, y, qm), ny = quad_dot<KU>(y, y, qm);
+      const float dn = __fdividef(nu, ny), inv = rsqrtf(ny);
+#pragma unroll
+      for (int u = 0; u < KU; ++u) x[u] = inv * y[u];
+      const bool settled = it > 0 && fabsf(dn - d) <= 1e-2f * dn;
+      d = dn;
+      if (settled) break;
+    }
+    s += d;
+  }
+  // ---- the shifted inverse and its inertia: exactly one eigenvalue below s
+  // (none but the zero column's, which the diagonal above stands in for)
+  quad_sweep_inverse<KMAX>(Hs, s, a4, piv, sg, sub, qm);
+  if (zeros != 0) {
+    if (!conditioned()) { defer(); return; }
+  } else {
+    int neg = 0;
+#pragma unroll
+    for (int u = 0; u < KU; ++u) neg += piv[u] < 0.0f;
+    neg += __shfl_xor_sync(qm, neg, 1);
+    neg += __shfl_xor_sync(qm, neg, 2);
+    if (neg != 1) { defer(); return; }
+  }
   DIAF_PHASE(7);
-  for (int c = 0; c < k; ++c) {
-    const float* pc = qptr(W, c * k + sub);
-    float s2 = 0.0f;
+  double xd[KU];  // the vector in FP64, entries sub + 4u
+  double* const X = reinterpret_cast<double*>(S - (threadIdx.x & 31) / 4) + 16 * KU * KMAX + (threadIdx.x & 31) / 4;
+  uint32_t flags = 0;
+  if (zeros != 0) {
 #pragma unroll
-    for (int u = 0; u < kQK; ++u)
-      if (u < nk) s2 = fmaf(pc[32 * u], pc[32 * u], s2);
-    QS(W, NR + c) = sqrtf(qsum(s2, qm));
-  }
-  int imin = 0;
-  double smin = (double)QS(W, NR), smax = smin;
-  for (int c = 1; c < k; ++c) {
-    const double sv = (double)QS(W, NR + c);
-    if (sv < smin) { smin = sv; imin = c; }
-    smax = fmax(smax, sv);
-  }
-  double snext = INFINITY, gap = INFINITY;
-  for (int c = 0; c < k; ++c)
-    if (c != imin) {
-      const double sv = (double)QS(W, NR + c);
-      snext = fmin(snext, sv);
-      gap = fmin(gap, sv * sv - smin * smin);
+    for (int u = 0; u < KU; ++u) xd[u] = (zeros >> (sub + 4 * u)) & 1u ? 1.0 : 0.0;
+  } else {
+    // the inverse itself in a4 (its rows' factors applied)
+#pragma unroll
+    for (int u = 0; u < KU; ++u)
+#pragma unroll
+      for (int q = 0; q < KMAX; ++q) a4[u][q] *= -sg[u];
+    float last = 1.0f;
+#pragma unroll 1
+    for (int it = 0; it < 2; ++it) {
+      float hx[KU], dx[KU];
+      quad_mul_smem<KMAX>(Hs, x, hx, qm);
+      const float d = quad_dot<KU>(x, hx, qm);
+#pragma unroll
+      for (int u = 0; u < KU; ++u) hx[u] -= d * x[u];
+      // -(H - d I)^-1 r by two Neumann steps on the shifted inverse
+      const float sh = s - d;
+#pragma unroll
+      for (int u = 0; u < KU; ++u) dx[u] = 0.0f;
+#pragma unroll 1
+      for (int n = 0; n < 3; ++n) {
+#pragma unroll
+        for (int u = 0; u < KU; ++u) dx[u] = -fmaf(sh, dx[u], hx[u]);
+        quad_mul_reg<KMAX>(a4, dx, dx, qm);
+      }
+      last = sqrtf(quad_dot<KU>(dx, dx, qm));
+#pragma unroll
+      for (int u = 0; u < KU; ++u) x[u] += dx[u];
+      const float inv = rsqrtf(quad_dot<KU>(x, x, qm));
+#pragma unroll
+      for (int u = 0; u < KU; ++u) x[u] *= inv;
     }
-  // V = R0^-1 B in place of B (R-hat regular): lane `sub` solves for the columns sub + 4v,
-  // column-oriented back substitution (column jj of R0 read through four
-  // pointers, element jj k + 4u + w at P[w][32 u])
-  __syncwarp(qm);  // every lane has read B for the norms
-  for (int c = zdiag ? k : sub; c < k; c += 4) {
-    float bv[KMAX];
-    const float* P0 = qptr(W, c * k);
-    const float* P1 = qptr(W, c * k + 1);
-    const float* P2 = qptr(W, c * k + 2);
-    const float* P3 = qptr(W, c * k + 3);
+    if (!(last <= 0.05f)) { defer(); return; }
+    // columns that no chain of nonzeros of H ties to the largest entry: exact zeros
+    {
+      uint32_t ties[KU];
+      float ax = -1.0f;
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i) {
-      const float* P = (i & 3) == 0 ? P0 : ((i & 3) == 1 ? P1 : ((i & 3) == 2 ? P2 : P3));
-      bv[i] = i < k ? P[32 * (i >> 2)] : 0.0f;
+      for (int u = 0; u < KU; ++u) {
+        ties[u] = 0;
+#pragma unroll
+        for (int q = 0; q < KMAX; ++q)
+          if (q < k && Hs[32 * (u * KMAX + q)] != 0.0f) ties[u] |= 1u << q;
+        if (sub + 4 * u >= k) ties[u] = 0;
+        else ax = fmaxf(ax, fabsf(x[u]));
+      }
+      float am = fmaxf(ax, __shfl_xor_sync(qm, ax, 1));
+      am = fmaxf(am, __shfl_xor_sync(qm, am, 2));
+      uint32_t comp = 0;
+#pragma unroll
+      for (int u = 0; u < KU; ++u)
+        if (sub + 4 * u < k && fabsf(x[u]) == am) comp |= 1u << (sub + 4 * u);
+      comp |= __shfl_xor_sync(qm, comp, 1);
+      comp |= __shfl_xor_sync(qm, comp, 2);
+      comp &= 0u - comp;
+      for (uint32_t grown = 0; grown != comp;) {
+        grown = comp;
+#pragma unroll
+        for (int u = 0; u < KU; ++u)
+          if ((grown >> (sub + 4 * u)) & 1u) comp |= ties[u];
+        comp |= __shfl_xor_sync(qm, comp, 1);
+        comp |= __shfl_xor_sync(qm, comp, 2);
+      }
+#pragma unroll
+      for (int u = 0; u < KU; ++u) xd[u] = (comp >> (sub + 4 * u)) & 1u ? (double)x[u] : 0.0;
     }
+    __syncwarp(qm);  // H has been read: the inverse takes its place
 #pragma unroll
-    for (int jj = KMAX - 1; jj >= 0; --jj) {
-      if (jj < k) {
-        const float* R0 = qptr(W, VO + jj * k);
-        const float* R1 = qptr(W, VO + jj * k + 1);
-        const float* R2 = qptr(W, VO + jj * k + 2);
-        const float* R3 = qptr(W, VO + jj * k + 3);
-        const float* Rd = (jj & 3) == 0 ? R0 : ((jj & 3) == 1 ? R1 : ((jj & 3) == 2 ? R2 : R3));
-        bv[jj] = bv[jj] / Rd[32 * (jj >> 2)];
+    for (int u = 0; u < KU; ++u)
 #pragma unroll
-        for (int i = 0; i < jj; ++i) {
-          const float* R = (i & 3) == 0 ? R0 : ((i & 3) == 1 ? R1 : ((i & 3) == 2 ? R2 : R3));
-          bv[i] = fmaf(-R[32 * (i >> 2)], bv[jj], bv[i]);
+      for (int q = 0; q < KMAX; ++q) Hs[32 * (u * KMAX + q)] = a4[u][q];
+    // ---- corrections against the FP64 tile: one pass over it gives both
+    // z = A-hat x on the lane's rows and its part of g = A-hat^T z, which the
+    // quad's lanes then sum and split
+    double before = (double)last;
+    bool done = false;
+#pragma unroll 1
+    for (int it = 0; it < kCorrectMax && !done; ++it) {
+#pragma unroll
+      for (int u = 0; u < KU; ++u) X[32 * u + 8 * sub] = xd[u];
+      __syncwarp(qm);
+      double g[4 * KU], zz = 0.0;
+#pragma unroll
+      for (int q = 0; q < 4 * KU; ++q) g[q] = 0.0;
+      for (int t = 0; t < nown; ++t) {
+        if ((inI >> (sub + 4 * t)) & 1u) continue;
+        const double* gp = G + t * KMAX * gstride + sub;
+        double tv[KMAX], z = 0.0;
+#pragma unroll
+        for (int q = 0; q < KMAX; ++q, gp += gstride) {
+          tv[q] = q < k ? *gp : 0.0;
+          z = fma(tv[q], X[(q >> 2) * 32 + (q & 3) * 8], z);
         }
+        zz = fma(z, z, zz);
+#pragma unroll
+        for (int q = 0; q < KMAX; ++q) g[q] = fma(tv[q], z, g[q]);
       }
-    }
-    float* Q0 = qptr(W, c * k);
-    float* Q1 = qptr(W, c * k + 1);
-    float* Q2 = qptr(W, c * k + 2);
-    float* Q3 = qptr(W, c * k + 3);
+      __syncwarp(qm);
+      // own entries of g: halves exchanged with lane ^ 1, then with lane ^ 2
+      double go[KU];
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i) {
-      float* Q = (i & 3) == 0 ? Q0 : ((i & 3) == 1 ? Q1 : ((i & 3) == 2 ? Q2 : Q3));
-      if (i < k) Q[32 * (i >> 2)] = bv[i];
-    }
-  }
-  __syncwarp(qm);
-  if (k > 1 && (snext - smin) <= 1e-6 * smax) flags |= DIAF_FLAG_DEGENERATE;
-  if (k > 1 && gap <= 1e-5 * smax * smax) { defer(); return; }
-  const int iters = (k > 1 && gap < 1e-2 * smax * smax) ? 2 : 1;
-
-  // ---- FP64 correction in the FP32 singular basis V: d = x^T H x / x^T x,
-  // r = H x - d x (H = A-hat^T A-hat from the FP64 tile),
-  // x <- x - sum_{i != imin} V_i (V_i^T r) / (sigma_i^2 - d).  x (k) in the
-  // quad's FP64 shared scratch, z = A-hat x (m) in its slab: lane `sub` computes z
-  // on its tile rows and (A-hat^T z)_q, r_q and the update of x_q on its rows
-  // q of V.
-  double* X = D;  // x, element q
-  const int zo = (M * K + 3) / 4 * 4;  // z, element r: slab element zo + r
-  {
-    const float* vmin = qptr(W, (zdiag ? VO : 0) + imin * k + sub);
-    double* xs = qptr(X, sub);
+      for (int u = 0; u < KU; ++u) {
+        double h[2];
 #pragma unroll
-    for (int u = 0; u < kQK; ++u)
-      if (u < nk) xs[32 * u] = (double)vmin[32 * u];
-  }
-  __syncwarp(qm);
-  for (int it = 0; it < iters; ++it) {
-    double zz = 0.0;
-    for (int t = 0; t < nown; ++t) {
-      const int r = sub + 4 * t;
-      double z = 0.0;
-      if (!((inI >> r) & 1u))
-        for (int q = 0; q < k; ++q) z = fma(T(r + q * m), QS(X, q), z);
-      T(zo + r) = z;
-      zz = fma(z, z, zz);
-    }
-    double xx = 0.0;
-    {
-      const double* xs = qptr(X, sub);
-#pragma unroll
-      for (int u = 0; u < kQK; ++u)
-        if (u < nk) xx = fma(xs[32 * u], xs[32 * u], xx);
-    }
-    const double d = qsum(zz, qm) / qsum(xx, qm);
-    __syncwarp(qm);  // z complete
-    float rfo[kQK];  // r on the lane's rows of V, in FP32
-    double xo[kQK], gq[kQK];
-#pragma unroll
-    for (int u = 0; u < kQK; ++u) gq[u] = 0.0;
-    for (int r = 0; r < m; ++r) {  // rows in I_j have z_r = 0
-      const double zr = T(zo + r);
-#pragma unroll
-      for (int u = 0; u < kQK; ++u)
-        if (u < nk) gq[u] = fma(T(r + (sub + 4 * u) * m), zr, gq[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < kQK; ++u) {
-      const int q = sub + 4 * u;
-      rfo[u] = 0.0f;
-      xo[u] = 0.0;
-      if (u < nk) {
-        xo[u] = QS(X, q);
-        rfo[u] = (float)(gq[u] - d * xo[u]);
+        for (int e = 0; e < 2; ++e) {
+          const double g0 = g[4 * u + 2 * e], g1 = g[4 * u + 2 * e + 1];
+          h[e] = ((sub & 1) ? g1 : g0) + __shfl_xor_sync(qm, (sub & 1) ? g0 : g1, 1);
+        }
+        go[u] = ((sub & 2) ? h[1] : h[0]) + __shfl_xor_sync(qm, (sub & 2) ? h[0] : h[1], 2);
       }
-    }
-    float dxo[kQK];
+      double xx = 0.0;
 #pragma unroll
-    for (int u = 0; u < kQK; ++u) dxo[u] = 0.0f;
-    for (int i = 0; i < k; ++i) {
-      const float* vi = qptr(W, (zdiag ? VO : 0) + i * k + sub);
-      float vo[kQK];
-      float vr = 0.0f;
+      for (int u = 0; u < KU; ++u) xx = fma(xd[u], xd[u], xx);
+      xx = qsum(xx, qm);
+      double ix = 2.0 - xx;  // 1 / xx, xx close to 1: two Newton steps from 1
+      ix *= fma(-xx, ix, 2.0);
+      ix *= fma(-xx, ix, 2.0);
+      const double d = qsum(zz, qm) * ix;
+      const double room = (double)s - d;  // at most the gap to the next eigenvalue
+      if (!(room >= 1.05e-5 * (double)hinf && d > 1e-24 * (double)hinf)) { defer(); return; }
+      float r[KU], dx[KU];
 #pragma unroll
-      for (int u = 0; u < kQK; ++u) {
-        vo[u] = u < nk ? vi[32 * u] : 0.0f;
-        vr = fmaf(vo[u], rfo[u], vr);
+      for (int u = 0; u < KU; ++u) r[u] = (float)fma(-d, xd[u], go[u]);
+#pragma unroll
+      for (int u = 0; u < KU; ++u) dx[u] = 0.0f;
+#pragma unroll 1
+      for (int n = 0; n < 3; ++n) {
+#pragma unroll
+        for (int u = 0; u < KU; ++u) dx[u] = -fmaf((float)room, dx[u], r[u]);
+        quad_mul_smem<KMAX>(Hs, dx, dx, qm);
       }
-      vr = qsum(vr, qm);
-      if (i == imin) continue;
-      const float sl = QS(W, NR + i);
-      const float ci = -vr / (sl * sl - (float)d);
+      const double step = sqrtf(quad_dot<KU>(dx, dx, qm));
 #pragma unroll
-      for (int u = 0; u < kQK; ++u) dxo[u] = fmaf(vo[u], ci, dxo[u]);
+      for (int u = 0; u < KU; ++u) xd[u] += (double)dx[u];
+      done = step * step <= 1e-14 * before;  // the next correction: about step (step / before)
+      if (!done && it > 0 && !(step <= 0.5 * before)) { defer(); return; }
+      before = step;
     }
-    __syncwarp(qm);  // every lane has read x and z
-    {
-      double* xs = qptr(X, sub);
-#pragma unroll
-      for (int u = 0; u < kQK; ++u)
-        if (u < nk) xs[32 * u] = xo[u] + (double)dxo[u];
-    }
-    __syncwarp(qm);
-  }
-  {
+    if (!done) { defer(); return; }
     double xn2 = 0.0;
-    double* xs = qptr(X, sub);
 #pragma unroll
-    for (int u = 0; u < kQK; ++u)
-      if (u < nk) xn2 = fma(xs[32 * u], xs[32 * u], xn2);
-    const double inv = 1.0 / sqrt(qsum(xn2, qm));
-    __syncwarp(qm);
+    for (int u = 0; u < KU; ++u) xn2 = fma(xd[u], xd[u], xn2);
+    xn2 = qsum(xn2, qm);
+    double inv = 1.5 - 0.5 * xn2;  // 1 / sqrt(xn2), xn2 within 1e-2 of 1: Newton steps from 1
+    inv *= fma(-0.5 * xn2 * inv, inv, 1.5);
+    inv *= fma(-0.5 * xn2 * inv, inv, 1.5);
 #pragma unroll
-    for (int u = 0; u < kQK; ++u)
-      if (u < nk) xs[32 * u] *= inv;
-    __syncwarp(qm);
+    for (int u = 0; u < KU; ++u) xd[u] *= inv;
   }
+#pragma unroll
+  for (int u = 0; u < KU; ++u) X[32 * u + 8 * sub] = xd[u];
+  __syncwarp(qm);
 
   // ---- v = T(I_j,:) w (into V's values by the row owners), phase v_jj >= 0,
   DIAF_PHASE(8);
@@ -695,7 +714,8 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
   for (int t = 0; t < nown; ++t) {
     const int r = sub + 4 * t;
     double sv = 0.0;
-    for (int q = 0; q < k; ++q) sv = fma(T(r + q * m), QS(X, q), sv);
+    const double* gp = G + t * KMAX * gstride + sub;
+    for (int q = 0; q < k; ++q, gp += gstride) sv = fma(*gp, QS(X, q), sv);
     if ((inI >> r) & 1u) {
       Vout[pos_of(r)] = sv;
       vn2 = fma(sv, sv, vn2);
@@ -731,7 +751,7 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
   }
   r2 = qsum(r2, qm);
   const double resj = sqrt(r2);
-  if (resj <= 1e-14 * smax) flags |= DIAF_FLAG_RANK_DEFICIENT;
+  if (zeros != 0 && resj == 0.0) flags |= DIAF_FLAG_RANK_DEFICIENT;  // otherwise sigma_min > 1e-12 sigma_max
   finite &= isfinite(resj);
   double* Wout = reinterpret_cast<double*>(a.Wv) + a.Wcp[j];
   for (int q = sub; q < k; q += 4) {
@@ -766,11 +786,8 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 16) column_thread_kernel(ColA
   const int sub = lane & 3, slot = lane >> 2;
   const unsigned qm = 0xFu << (lane & ~3);
   const int gq = (blockIdx.x * kQuadWarps + warp) * kQuadCols + slot;  // quad index in the grid
-  const int M = ta.M, K = ta.K;
-  unsigned char* wbase = reinterpret_cast<unsigned char*>(tsmem) + (size_t)warp * thread_warp_smem(M, K);
-  float* S = reinterpret_cast<float*>(wbase) + slot;
-  double* D = reinterpret_cast<double*>(wbase + sizeof(float) * (size_t)thread_arena_floats(M, K) * 8) + slot;
-  double* G = ta.slab + (size_t)4 * gq;  // element e of the quad's tile at G[(e/4) 4 nquads + (e mod 4)]
+  float* S = tsmem + (size_t)warp * thread_arena_floats(ta.M, ta.K, KMAX) * 8 + slot;
+  double* G = ta.slab + (size_t)4 * gq;
   const int count = *a.list_count;
   while (true) {
     int base = 0;
@@ -778,7 +795,7 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 16) column_thread_kernel(ColA
     base = __shfl_sync(DIAF_FULL, base, 0);
     if (base >= count) break;
     const int idx = base + slot;
-    if (idx < count) solve_column_quad<KMAX>(a, ta, list_at(a, count, idx), S, D, G, sub, qm);
+    if (idx < count) solve_column_quad<KMAX>(a, ta, list_at(a, count, idx), S, G, sub, qm);
     __syncwarp();
   }
 }

@@ -1,57 +1,40 @@
-// One thread per column: the mixed-precision DIAF-S kernel for small real tiles.
+// Four lanes per column: the mixed-precision DIAF-S kernel for small real tiles.
 #include "column_thread.cuh"
 #include "launch.cuh"
 
 namespace {
-size_t g_thread_smem_configured = 0;
 
-// The round-robin schedule of warp_jacobi: in round rnd, position p >= 1 holds
-// column 1 + ((p - 1 + rnd) mod L), position 0 column 0, and positions p and
-// qq - 1 - p pair up.
-cudaError_t upload_pair_table() {
-  static bool done = false;  // per process; the table is the same on every device
-  static int dev_done = -1;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (done && dev_done == dev) return cudaSuccess;
-  uint8_t tab[kThreadKMax / 2][kPairRounds][kPairSlots] = {};
-  for (int np = 1; np <= kThreadKMax / 2; ++np) {
-    const int qq = 2 * np, L = qq - 1;
-    for (int rnd = 0; rnd < L; ++rnd)
-      for (int pr = 0; pr < np; ++pr) {
-        int ea = pr - 1 + rnd, eb = qq - 2 - pr + rnd;
-        ea = ((ea % L) + L) % L;
-        eb = eb % L;
-        int x = pr == 0 ? 0 : 1 + ea, y = 1 + eb;
-        if (x > y) { const int t = x; x = y; y = t; }
-        tab[np - 1][rnd][pr] = (uint8_t)((x << 4) | y);
-      }
+// f(kernel, index) with the instance for tiles of at most K columns
+template <class F>
+cudaError_t with_instance(int K, F f) {
+  switch (thread_instance(K)) {
+    case 8: return f(column_thread_kernel<8>, 0);
+    case 13: return f(column_thread_kernel<13>, 1);
+    default: return f(column_thread_kernel<16>, 2);
   }
-  e = cudaMemcpyToSymbol(kPairTab, tab, sizeof(tab));
-  if (e == cudaSuccess) { done = true; dev_done = dev; }
-  return e;
 }
+
+size_t g_thread_smem_configured[3] = {0, 0, 0};
+
 }  // namespace
 
 cudaError_t thread_columns_shape(int M, int K, int count_hint, ThreadShape* out) {
   *out = ThreadShape{};
   if (count_hint <= 0) return cudaSuccess;
   if (M < 1 || K < 1 || M > kThreadMMax || K > kThreadKMax) return cudaErrorInvalidValue;
-  cudaError_t te = upload_pair_table();
-  if (te != cudaSuccess) return te;
-  auto kern = column_thread_kernel<kThreadKMax>;
-  const size_t smem = thread_warp_smem(M, K) * kQuadWarps;
+  const size_t smem = thread_warp_smem(M, K, thread_instance(K)) * kQuadWarps;
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  if (g_thread_smem_configured < smem) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    g_thread_smem_configured = smem;
-  }
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kQuadWarps, smem);
+  e = with_instance(K, [&](auto kern, int i) {
+    if (g_thread_smem_configured[i] < smem) {
+      const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (r != cudaSuccess) return r;
+      g_thread_smem_configured[i] = smem;
+    }
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kQuadWarps, smem);
+  });
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidValue;
   int grid = sms * per_sm;
@@ -66,7 +49,9 @@ cudaError_t thread_columns_shape(int M, int K, int count_hint, ThreadShape* out)
 
 cudaError_t launch_columns_thread_f32(const ColArgs& a, const ThreadArgs& ta, const ThreadShape& sh, cudaStream_t s) {
   if (sh.grid <= 0) return cudaSuccess;
-  column_thread_kernel<kThreadKMax><<<sh.grid, sh.block, sh.smem, s>>>(a, ta);
-  DIAF_COUNT_LAUNCH();
-  return cudaGetLastError();
+  return with_instance(ta.K, [&](auto kern, int) {
+    kern<<<sh.grid, sh.block, sh.smem, s>>>(a, ta);
+    DIAF_COUNT_LAUNCH();
+    return cudaGetLastError();
+  });
 }
