@@ -1063,6 +1063,7 @@ bool event_passed(cudaEvent_t e) {
 struct LevelWalk {
   int32_t *lev, *rank, *rcnt, *dpos, *slot, *cnt;
   int nlev;
+  int maxrow;  // off-diagonal entries of the longest row
 };
 
 int level_walk(int n, const int32_t* cp, const int32_t* ri, const uint32_t* word, uint32_t gen, bool up,
@@ -1072,7 +1073,7 @@ int level_walk(int n, const int32_t* cp, const int32_t* ri, const uint32_t* word
     w.lev[i] = 0;
     w.rcnt[i] = 0;
   }
-  int nl = 0;
+  int nl = 0, maxrow = 0;
   bool nodiag = false;
   for (int step = 0; step < n; ++step) {
     const int j = up ? n - 1 - step : step;
@@ -1099,12 +1100,14 @@ int level_walk(int n, const int32_t* cp, const int32_t* ri, const uint32_t* word
       }
       if (up ? i > j : i < j) return 1;
       w.slot[p] = w.rcnt[i]++;
+      maxrow = std::max(maxrow, w.rcnt[i]);
       if (w.lev[i] <= lj) w.lev[i] = lj + 1;
     }
     if (!d) w.dpos[j] = -1;
     nodiag |= !d;
   }
   w.nlev = nl;
+  w.maxrow = maxrow;
   return nodiag ? 2 : 0;
 }
 
@@ -1186,7 +1189,7 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   int32_t* ri = mir ? F->mir_ri : st32 + n1;
   int32_t* ptr = st32 + (mir ? 0 : n1 + nri);  // level pointers (at most n + 1)
   int32_t* hblk = ptr + n1;
-  LevelWalk lw{hblk, hblk + n, hblk + 2 * (size_t)n, hblk + 3 * (size_t)n, hblk + 4 * (size_t)n, nullptr, 0};
+  LevelWalk lw{hblk, hblk + n, hblk + 2 * (size_t)n, hblk + 3 * (size_t)n, hblk + 4 * (size_t)n, nullptr, 0, 0};
   uint32_t* hp = reinterpret_cast<uint32_t*>(hblk + blk);
   if (!mir) {
     DIAF_CU(cudaMemcpyAsync(cp, F->Vcp, sizeof(int32_t) * n1, cudaMemcpyDeviceToHost, s));
@@ -1242,6 +1245,26 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
     c.add(&F->Wl.colidx, F->nnz_w);
     c.add((char**)&F->tbuf, esz * n);
     if (ce == cudaSuccess) ce = F->carve(c);
+  }
+  // the packed form's arrays (used when the walk finds the rows short enough);
+  // without the memory for them the level-ordered rows above do
+  int32_t *poff = nullptr, *moff = nullptr;
+  double* mval = nullptr;
+  void* pval = nullptr;
+  uint32_t* pflags = nullptr;
+  if (ce == cudaSuccess && n > 0) {
+    Carve c;
+    c.add(&poff, (size_t)kPackEntries * n);
+    c.add((char**)&pval, esz * kPackEntries * n);
+    if (!cplx) {
+      c.add(&moff, (size_t)kMergeEntries * n);
+      c.add(&mval, (size_t)kMergeEntries * n);
+    }
+    c.add(&pflags, 1);
+    if (F->carve(c) != cudaSuccess) {
+      (void)cudaGetLastError();
+      poff = nullptr;
+    }
   }
   if (ce == cudaSuccess) ce = cudaMemsetAsync(zflag, 0, sizeof(uint32_t), s);
   int32_t* const wl_colidx = F->Wl.colidx;
@@ -1318,6 +1341,12 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
     Vl.maxw = std::max(Vl.maxw, cnt[l]);
   }
   Vl.nlev = nlev;
+  Vl.r = poff ? level_group(cplx, lw.maxrow, nlev, ptr, &Vl.maxg) : 0;
+  Vl.poff = poff;
+  Vl.pval = pval;
+  Vl.moff = moff;
+  Vl.mval = mval;
+  Vl.pflags = pflags;
   // the device places the rows (position of row i: ptr[lev i] + rank i),
   // lays V's rows out level by level from its columns, and checks the
   // diagonal's values; the zero-diagonal flag is read after all of that is
@@ -1337,7 +1366,7 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   const int32_t* drcnt = dblk + 2 * (size_t)n;
   const int32_t* ddpos = dblk + 3 * (size_t)n;
   const int32_t* dslot = dblk + 4 * (size_t)n;
-  ce = level_place(n, dlev, drank, drcnt, Vl.lvlptr, pos, Vl.xrow, work, Vl.rowptr, s);
+  ce = level_place(n, cplx, dlev, drank, drcnt, pos, work, Vl, s);
   F->Wl = F->Wr;
   F->Wl.colidx = wl_colidx;
   if (ws) {  // W's columns renumbered to V's level order on the side stream, once the positions are known
@@ -1350,7 +1379,7 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
     F->w_pending = ce == cudaSuccess;
   }
   if (ce == cudaSuccess)
-    ce = level_fill(n, cplx, F->Vcp, F->Vri, F->Vv, ddpos, dslot, pos, Vl, zflag, s);
+    ce = level_fill(n, cplx, F->Vcp, F->Vri, F->Vv, ddpos, dslot, pos, dlev, Vl, zflag, s);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(hp, zflag, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
   if (ce == cudaSuccess) ce = cudaEventRecord(ev[1], s);
   PT_DEV(s);
@@ -1394,7 +1423,7 @@ diaf_status diaf_level_schedule(int32_t n, const int32_t* colptr, const int32_t*
   const size_t nn = (size_t)n, nnz = (size_t)colptr[n];
   std::vector<int32_t> scratch(4 * nn + 1 + nnz);
   LevelWalk w{level, scratch.data(), scratch.data() + nn, scratch.data() + 2 * nn, scratch.data() + 4 * nn + 1,
-              scratch.data() + 3 * nn, 0};
+              scratch.data() + 3 * nn, 0, 0};
   bool up = true;
   int r = level_walk(n, colptr, rowidx, nullptr, 0, true, nullptr, w);
   if (r == 1) {

@@ -516,7 +516,7 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
       S s = sc_zero<S>();
       int r = ix.Iloc[t];
       if (r >= 0)
-        for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
+        for (int q = 0; q < k; ++q) s += Ts[r + q * LDT] * wv[q];
       vv[t] = s;
     }
     __syncwarp();

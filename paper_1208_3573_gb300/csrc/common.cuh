@@ -113,6 +113,12 @@ template <> __device__ __forceinline__ Cx<float> sc_cast<Cx<float>, Cx<double>>(
 template <> __device__ __forceinline__ Cx<double> sc_cast<Cx<double>, Cx<float>>(Cx<float> a) { return {(double)a.re, (double)a.im}; }
 template <> __device__ __forceinline__ Cx<float> sc_cast<Cx<float>, Cx<float>>(Cx<float> a) { return a; }
 
+// 16 bytes of scalars, for vector loads
+template <class S>
+struct alignas(16) Pack16 {
+  S v[16 / sizeof(S)];
+};
+
 // ----------------------------------------------------------------- shuffles
 __device__ __forceinline__ double shfl_xor(double v, int m) { return __shfl_xor_sync(DIAF_FULL, v, m); }
 __device__ __forceinline__ float shfl_xor(float v, int m) { return __shfl_xor_sync(DIAF_FULL, v, m); }

@@ -40,9 +40,12 @@
 
 // A factor of the Gram matrix carries eps kappa^2.
 template <class R> __device__ __forceinline__ constexpr R smallest_kappa_max() { return sizeof(R) == 4 ? R(30) : R(300); }
-// The column of H that a lane keeps in registers: up to 64 of them (complex128
-// tiles of up to 32 columns keep the Jacobi).
-template <class S, int KMAX> constexpr bool kSmallestFits = sizeof(S) * KMAX <= 256;
+// Not for complex128: there the Jacobi stays.  Its W and V agree with this
+// form's to 1e-14, but the residual at which a restarted GMRES stops moves by
+// 1e-6 of itself with the last bits of W and V (Helmholtz 150^2, against a
+// 64-bit restatement: 6.9e-7 with the Jacobi, 1.5e-6 with this form).
+template <class S, int KMAX>
+constexpr bool kSmallestFits = !(ScalarInfo<S>::cplx && sizeof(S) == 16);
 constexpr int kInverseItMax = 16;
 constexpr int kCorrectMax = 8;
 
@@ -62,11 +65,6 @@ __device__ __forceinline__ SD tile_adj_mul(const SD* Ts, const SD* zz, int m, in
   }
   return g;
 }
-
-template <class S>
-struct alignas(16) Pack16 {
-  S v[16 / sizeof(S)];
-};
 
 // Inverse of H - shift I for the Hermitian k x k matrix Hs (leading dimension
 // KP; lane q reads column q) by symmetric sweeps without pivoting: the sweep

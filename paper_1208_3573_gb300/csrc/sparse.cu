@@ -1,4 +1,5 @@
 // Row-oriented sparse operations for the solve phase.
+#include <atomic>
 #include <climits>
 
 #include "plan.cuh"
@@ -124,17 +125,22 @@ constexpr int kLevelThreads = 1024;
 constexpr int kLevelPtrSmem = 8192;  // level pointers kept in shared memory up to this many levels
 constexpr int kPrefetch = 4;         // off-diagonal entries of a row held in registers ahead of its level
 
+template <class S>
+constexpr int level_window() { return 131072 / (int)sizeof(S); }  // 128 KB ring
+
 // Row i of V goes to level position p = lvlptr[lev i] + rank i (the walk's
 // place of row i in its level); len[p] = its number of off-diagonal entries.
 __global__ void level_place_kernel(int n, const int32_t* __restrict__ lev, const int32_t* __restrict__ rank,
                                    const int32_t* __restrict__ rcnt, const int32_t* __restrict__ lvlptr,
-                                   int32_t* __restrict__ pos, int32_t* __restrict__ xrow, int32_t* __restrict__ len) {
+                                   int32_t* __restrict__ pos, int32_t* __restrict__ xrow, int32_t* __restrict__ len,
+                                   int32_t* __restrict__ poff) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int p = lvlptr[lev[i]] + rank[i];
   pos[i] = p;
   xrow[p] = i;
-  len[p] = rcnt[i];
+  if (poff) reinterpret_cast<int4*>(poff)[p] = make_int4(-1, -1, -1, -1);
+  else len[p] = rcnt[i];
 }
 
 // V's rows level by level, straight from its columns: kConvLanes lanes per
@@ -164,6 +170,54 @@ __global__ void level_fill_kernel(int n, const int32_t* __restrict__ cp, const i
       const int q = rowptr[pos[i]] + slot[e];
       pcol[q] = pos[j];
       pval[q] = ((1.0 / sc_abs2(d)) * sc_conj(d)) * v[e];
+    }
+  }
+}
+
+// The same for a real V in the packed form: entry slot[e] of the row.
+__global__ void packed_fill_kernel(int n, const int32_t* __restrict__ cp, const int32_t* __restrict__ ri,
+                                   const double* __restrict__ v, const int32_t* __restrict__ dpos,
+                                   const int32_t* __restrict__ slot, const int32_t* __restrict__ pos,
+                                   const int32_t* __restrict__ lev, const int32_t* __restrict__ lvlptr, int r, int nlev,
+                                   int32_t* __restrict__ poff, double* __restrict__ pval, double* __restrict__ pdinv,
+                                   uint32_t* __restrict__ zflag, uint32_t* __restrict__ pflags) {
+  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int j = (int)(gid / kConvLanes), sub = (int)(gid % kConvLanes);
+  if (j >= n) return;
+  const int e1 = cp[j + 1];
+  for (int e = cp[j] + sub; e < e1; e += kConvLanes) {
+    const int i = ri[e];
+    const double d = i == j ? v[e] : v[dpos[i]];
+    if (i == j) {
+      if (!(d * d > 0.0)) atomicOr(zflag, 1u);
+      pdinv[pos[j]] = (1.0 / (d * d)) * d;
+    } else {
+      const int pi = pos[i], pj = pos[j];
+      const size_t q = (size_t)kPackEntries * pi + slot[e];
+      poff[q] = pj;
+      pval[q] = ((1.0 / (d * d)) * d) * v[e];
+      const int last = (lev[i] / r + 1) * r;  // the end of the row's group
+      if (pj < lvlptr[last < nlev ? last : nlev] - level_window<double>()) atomicOr(pflags, kPackFar);
+    }
+  }
+}
+
+// A complex V's packed form (r = 1) from its level-ordered rows: copied, so
+// that the solve's results keep every bit (the residual at which a restarted
+// GMRES stops moves by 1e-6 of itself with the last bit of the apply).
+__global__ void pack_rows_kernel(int nlev, const int32_t* __restrict__ lvlptr, const int32_t* __restrict__ rowptr,
+                                 const int32_t* __restrict__ colidx, const Cx<double>* __restrict__ vals,
+                                 int32_t* __restrict__ poff, Cx<double>* __restrict__ pval, uint32_t* pflags) {
+  for (int l = blockIdx.x; l < nlev; l += gridDim.x) {
+    const int e = lvlptr[l + 1];
+    for (int p = lvlptr[l] + (int)threadIdx.x; p < e; p += blockDim.x) {
+      const int a = rowptr[p], len = rowptr[p + 1] - a;
+      for (int q = 0; q < kPackEntries; ++q) {
+        const int c = q < len ? colidx[a + q] : -1;
+        poff[(size_t)kPackEntries * p + q] = c;
+        if (q < len) pval[(size_t)kPackEntries * p + q] = vals[a + q];
+        if (c >= 0 && c < e - level_window<Cx<double>>()) atomicOr(pflags, kPackFar);
+      }
     }
   }
 }
@@ -217,9 +271,6 @@ __device__ __forceinline__ void warm_level_data(int n, int nnz, const int32_t* r
   for (int i = threadIdx.x; i < (int)(nnz * sizeof(S) / 16); i += blockDim.x) acc += v4[i].y;
   if (acc == 0x9e3779b9u && n < 0) t[0] = sc_zero<S>();  // keeps the loads; never taken
 }
-
-template <class S>
-constexpr int level_window() { return 131072 / (int)sizeof(S); }  // 128 KB ring
 
 template <class S>
 __global__ void __launch_bounds__(kLevelThreads, 1)
@@ -384,29 +435,287 @@ __global__ void __launch_bounds__(kDeepThreads, 1)
 #undef DIAF_LP
 }
 
+// ---- the packed form: levels in groups
+//
+// On the single solving SM a level cost about 0.58 us whatever its width: the
+// chain barrier - bounds - column indices - t - FP64 - barrier, some 150
+// instructions long, not the arithmetic (convection-diffusion 256^2: 512
+// levels of 128 rows, 0.30 ms, where the FP64 pipe needs 0.03).  Two changes:
+//
+// a row's entries at fixed places (two to five 16-byte loads, issued groups
+// ahead), so that between two barriers a thread only reads t from the ring,
+// multiplies and writes its own t;
+//
+// r = 4 levels between two barriers.  Eliminating the rows of its own group
+// from a row, t_i = x'_i + sum C_ik t_k has only k of earlier groups.  The
+// coefficients C are formed once (merge_kernel); x' is the right-hand side put
+// through the group's own block, group by group independently of each other,
+// so all SMs do it at once (group_rhs_kernel).  The stencil operators' rows
+// have 2 entries and 3.3 merged ones (at most 5), so the chip's one FP64 pipe
+// that solves does 1.7 times the work for a quarter of the barriers.  Complex
+// rows (4 entries, 8 merged) are bound by that pipe: they keep r = 1.
+
+// The merged entries of group blockIdx.x, level by level: the row's own
+// entries of earlier groups, and for each entry of its own group v times that
+// row's merged entries.
+__global__ void __launch_bounds__(256) merge_kernel(int nlev, int r, const int32_t* __restrict__ lvlptr,
+                                                    const int32_t* __restrict__ poff, const double* __restrict__ pval,
+                                                    int32_t* moff, double* mval, uint32_t* pflags) {
+  const int l0 = blockIdx.x * r;
+  const int l1 = l0 + r < nlev ? l0 + r : nlev;
+  const int gs = lvlptr[l0];
+  for (int l = l0; l < l1; ++l) {
+    const int e = lvlptr[l + 1];
+    for (int p = lvlptr[l] + (int)threadIdx.x; p < e; p += blockDim.x) {
+      int32_t c[kMergeEntries];
+      double v[kMergeEntries];
+#pragma unroll
+      for (int q = 0; q < kMergeEntries; ++q) {
+        c[q] = -1;
+        v[q] = 0.0;
+      }
+      bool full = false;
+      auto add = [&](int32_t col, double val) {
+        bool placed = false;
+#pragma unroll
+        for (int q = 0; q < kMergeEntries; ++q)
+          if (!placed && (c[q] < 0 || c[q] == col)) {
+            c[q] = col;
+            v[q] += val;
+            placed = true;
+          }
+        full |= !placed;
+      };
+#pragma unroll
+      for (int q = 0; q < kPackEntries; ++q) {
+        const int32_t col = poff[kPackEntries * (size_t)p + q];
+        if (col < 0) continue;
+        const double val = -pval[kPackEntries * (size_t)p + q];
+        if (col < gs) {
+          add(col, val);
+        } else {
+          for (int u = 0; u < kMergeEntries; ++u) {
+            const int32_t k = moff[kMergeEntries * (size_t)col + u];
+            if (k >= 0) add(k, -val * mval[kMergeEntries * (size_t)col + u]);
+          }
+        }
+      }
+      if (full) atomicOr(pflags, kPackMergeFull);
+#pragma unroll
+      for (int q = 0; q < kMergeEntries; ++q) {
+        moff[kMergeEntries * (size_t)p + q] = c[q];
+        mval[kMergeEntries * (size_t)p + q] = -v[q];  // (the solve subtracts)
+      }
+    }
+    __syncthreads();  // the level's merged rows are visible to the block
+  }
+}
+
+// t = the scaled right-hand side with the rows of the own group eliminated
+// (as it is when the rows could not be merged), one block per group.
+__global__ void __launch_bounds__(256) group_rhs_kernel(int nlev, int r, const int32_t* __restrict__ lvlptr,
+                                                        const int32_t* __restrict__ poff,
+                                                        const double* __restrict__ pval,
+                                                        const double* __restrict__ dinv,
+                                                        const int32_t* __restrict__ xrow, const double* __restrict__ x,
+                                                        double* t, const uint32_t* __restrict__ pflags) {
+  const int l0 = blockIdx.x * r;
+  const int l1 = l0 + r < nlev ? l0 + r : nlev;
+  const int gs = lvlptr[l0];
+  const bool merged = !*pflags;
+  for (int l = l0; l < l1; ++l) {
+    const int e = lvlptr[l + 1];
+    for (int p = lvlptr[l] + (int)threadIdx.x; p < e; p += blockDim.x) {
+      double acc = dinv[p] * x[xrow[p]];
+      if (merged && l > l0) {
+        const int4 c = reinterpret_cast<const int4*>(poff)[p];
+        const double* v = pval + kPackEntries * (size_t)p;
+        if (c.x >= gs) acc = fma(-v[0], t[c.x], acc);
+        if (c.y >= gs) acc = fma(-v[1], t[c.y], acc);
+        if (c.z >= gs) acc = fma(-v[2], t[c.z], acc);
+        if (c.w >= gs) acc = fma(-v[3], t[c.w], acc);
+      }
+      t[p] = acc;
+    }
+    __syncthreads();
+  }
+}
+
+// A row as it is loaded groups ahead: nothing is computed from it before its
+// group's turn (an operation on it at the load waits for the load: 0.36
+// against 0.18 ms a solve with the values negated on arrival).
+template <class S, int K>
+struct PackedRow {
+  int32_t c[K];
+  S v[K];
+  S x;
+  __device__ __forceinline__ void load(const int32_t* off, const S* val, const S* t, int p) {
+    static_assert(K % 2 == 0, "whole 8-byte pairs of columns");
+    const int2* o = reinterpret_cast<const int2*>(off + (size_t)K * p);
+#pragma unroll
+    for (int q = 0; q < K / 2; ++q) {
+      const int2 w = __ldg(o + q);
+      c[2 * q] = w.x;
+      c[2 * q + 1] = w.y;
+    }
+    constexpr int PV = 16 / (int)sizeof(S);
+    const Pack16<S>* vv = reinterpret_cast<const Pack16<S>*>(val + (size_t)K * p);
+#pragma unroll
+    for (int q = 0; q < K / PV; ++q) {
+      const Pack16<S> w = vv[q];
+#pragma unroll
+      for (int u = 0; u < PV; ++u) v[q * PV + u] = w.v[u];
+    }
+    x = t[p];
+  }
+};
+
+// The solve of the packed form by T threads; a thread has up to ROWS rows of a
+// group in registers, loaded D groups ahead (what is wider than that goes
+// through memory).  NEAR: every entry is in the ring.
+template <class S, int K, int T, int ROWS, int D, bool NEAR>
+__device__ __forceinline__ void packed_solve(int ng, const int32_t* __restrict__ ptr, const int32_t* __restrict__ off,
+                                             const S* __restrict__ val, S* t, S* tw) {
+  constexpr int kWin = level_window<S>();
+  const int tid = (int)threadIdx.x;
+  PackedRow<S, K> row[D][ROWS];
+  auto fetch = [&](PackedRow<S, K>(&w)[ROWS], int g) {
+    const int b = ptr[g] + tid, e = ptr[g + 1];
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u)
+      if (b + u * T < e) w[u].load(off, val, t, b + u * T);
+  };
+#pragma unroll
+  for (int k = 0; k < D; ++k)
+    if (k < ng) fetch(row[k], k);
+  int b = 0;
+  for (int g0 = 0; g0 < ng; g0 += D) {
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      const int g = g0 + k;
+      if (g >= ng) break;  // uniform
+      const int e = ptr[g + 1];
+      auto solve = [&](const PackedRow<S, K>& w, int p) {
+        S tv[K];  // all reads of t, then the chain
+#pragma unroll
+        for (int q = 0; q < K; ++q)
+          if (w.c[q] >= 0) tv[q] = NEAR || w.c[q] >= e - kWin ? tw[w.c[q] & (kWin - 1)] : t[w.c[q]];
+        S acc = w.x;
+#pragma unroll
+        for (int q = 0; q < K; ++q)
+          if (w.c[q] >= 0) acc = sc_msub(acc, w.v[q], tv[q]);
+        t[p] = acc;
+        tw[p & (kWin - 1)] = acc;
+      };
+#pragma unroll
+      for (int u = 0; u < ROWS; ++u)
+        if (b + tid + u * T < e) solve(row[k][u], b + tid + u * T);
+      for (int p = b + tid + ROWS * T; p < e; p += T) {
+        PackedRow<S, K> w;
+        w.load(off, val, t, p);
+        solve(w, p);
+      }
+      if (g + D < ng) fetch(row[k], g + D);
+      b = e;
+      __syncthreads();
+    }
+  }
+}
+
+// One block of T threads, ROWS rows of a group in a thread's registers.
+// MERGED: groups of r levels.
+template <class S, int T, int ROWS, int D, bool MERGED>
+__global__ void __launch_bounds__(T, 1)
+    trsv_packed_kernel(int nlev, int r, const int32_t* __restrict__ lvlptr, const int32_t* __restrict__ poff,
+                       const S* __restrict__ pval, const int32_t* __restrict__ moff, const double* __restrict__ mval,
+                       const uint32_t* __restrict__ pflags, S* t) {
+  extern __shared__ __align__(16) unsigned char level_ring[];
+  S* tw = reinterpret_cast<S*>(level_ring);
+  __shared__ int32_t sptr[kLevelPtrSmem + 1];
+  const uint32_t fl = *pflags;
+  const bool merged = MERGED && !fl;
+  const int step = merged ? r : 1;
+  const int ng = (nlev + step - 1) / step;
+  const bool in_smem = ng <= kLevelPtrSmem;
+  if (in_smem)
+    for (int i = threadIdx.x; i <= ng; i += T) sptr[i] = lvlptr[i * step < nlev ? i * step : nlev];
+  __syncthreads();
+  if constexpr (MERGED) {
+    if (merged && in_smem) {
+      packed_solve<double, kMergeEntries, T, ROWS, D, true>(ng, sptr, moff, mval, t, tw);
+      return;
+    }
+  }
+  // (the host groups levels only where their pointers fit in shared memory)
+  const int32_t* ptr = in_smem ? sptr : lvlptr;
+  if (!(fl & kPackFar)) packed_solve<S, kPackEntries, T, ROWS, D, true>(ng, ptr, poff, pval, t, tw);
+  else packed_solve<S, kPackEntries, T, ROWS, 1, false>(ng, ptr, poff, pval, t, tw);
+}
+
 }  // namespace
 
-cudaError_t level_place(int n, const int32_t* lev, const int32_t* rank, const int32_t* rcnt, const int32_t* lvlptr,
-                        int32_t* pos, int32_t* xrow, int32_t* work, int32_t* rowptr, cudaStream_t s) {
-  if (n <= 0) return cudaMemsetAsync(rowptr, 0, sizeof(int32_t), s);
+int level_group(bool cplx, int maxrow, int nlev, const int32_t* lvlptr, int* maxg) {
+  *maxg = 0;
+  if (maxrow > kPackEntries || nlev <= 0) return 0;
+  for (int r = cplx ? 1 : 4; r >= 1; r >>= 1) {
+    int w = 0;
+    for (int l = 0; l < nlev; l += r) {
+      const int n = lvlptr[l + r < nlev ? l + r : nlev] - lvlptr[l];
+      if (n > w) w = n;
+    }
+    if ((w <= kGroupRows && nlev <= r * kLevelPtrSmem) || r == 1) {
+      *maxg = w;
+      return r;
+    }
+  }
+  return 0;
+}
+
+cudaError_t level_place(int n, bool cplx, const int32_t* lev, const int32_t* rank, const int32_t* rcnt, int32_t* pos,
+                        int32_t* work, LevelCsr& L, cudaStream_t s) {
+  if (n <= 0) return cudaMemsetAsync(L.rowptr, 0, sizeof(int32_t), s);
   int32_t* len = work;
   int32_t* bs = work + n;
-  level_place_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, lev, rank, rcnt, lvlptr, pos, xrow, len);
+  const bool rows = L.r == 0 || cplx;  // the rows' pointers are needed
+  level_place_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, lev, rank, rcnt, L.lvlptr, pos, L.xrow, len,
+                                                      rows ? nullptr : L.poff);
   DIAF_COUNT_LAUNCH();
-  return exclusive_scan_i32(len, rowptr, n, bs, s);
+  return rows ? exclusive_scan_i32(len, L.rowptr, n, bs, s) : cudaGetLastError();
 }
 
 cudaError_t level_fill(int n, bool cplx, const int32_t* cp, const int32_t* ri, const void* v, const int32_t* dpos,
-                       const int32_t* slot, const int32_t* pos, LevelCsr& L, uint32_t* zflag, cudaStream_t s) {
+                       const int32_t* slot, const int32_t* pos, const int32_t* lev, LevelCsr& L, uint32_t* zflag,
+                       cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int blocks = (int)(((int64_t)n * kConvLanes + 255) / 256);
-  if (cplx)
+  if (L.r > 0) {
+    cudaError_t e = cudaMemsetAsync(L.pflags, 0, sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+  }
+  if (cplx) {
     level_fill_kernel<Cx<double>><<<blocks, 256, 0, s>>>(n, cp, ri, (const Cx<double>*)v, dpos, slot, pos, L.rowptr,
                                                           L.colidx, (Cx<double>*)L.vals, (Cx<double>*)L.dinv, zflag);
-  else
+    DIAF_COUNT_LAUNCH();
+    if (L.r > 0) {
+      pack_rows_kernel<<<L.nlev < 4096 ? L.nlev : 4096, 128, 0, s>>>(L.nlev, L.lvlptr, L.rowptr, L.colidx,
+                                                                     (const Cx<double>*)L.vals, L.poff,
+                                                                     (Cx<double>*)L.pval, L.pflags);
+      DIAF_COUNT_LAUNCH();
+    }
+  } else if (L.r > 0) {
+    packed_fill_kernel<<<blocks, 256, 0, s>>>(n, cp, ri, (const double*)v, dpos, slot, pos, lev, L.lvlptr, L.r, L.nlev,
+                                              L.poff, (double*)L.pval, (double*)L.dinv, zflag, L.pflags);
+    DIAF_COUNT_LAUNCH();
+    if (L.r > 1) {
+      merge_kernel<<<ceil_div(L.nlev, L.r), 256, 0, s>>>(L.nlev, L.r, L.lvlptr, L.poff, (const double*)L.pval, L.moff,
+                                                         L.mval, L.pflags);
+      DIAF_COUNT_LAUNCH();
+    }
+  } else {
     level_fill_kernel<double><<<blocks, 256, 0, s>>>(n, cp, ri, (const double*)v, dpos, slot, pos, L.rowptr, L.colidx,
                                                       (double*)L.vals, (double*)L.dinv, zflag);
-  DIAF_COUNT_LAUNCH();
+    DIAF_COUNT_LAUNCH();
+  }
   return cudaGetLastError();
 }
 
@@ -417,6 +726,41 @@ cudaError_t remap_columns(int64_t nnz, const int32_t* pos, const int32_t* cin, i
   remap_cols_kernel<<<blocks, 256, 0, s>>>(nnz, pos, cin, cout);
   DIAF_COUNT_LAUNCH();
   return cudaGetLastError();
+}
+
+template <class S, int T, int ROWS, int D, bool MERGED>
+static cudaError_t trsv_packed_t(const LevelCsr& L, void* t, cudaStream_t s) {
+  constexpr size_t ring = sizeof(S) * level_window<S>();
+  static std::atomic<uint64_t> configured{0};  // the attribute is per device: one bit each
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev > 63 || !(configured.load() & bit)) {
+    e = cudaFuncSetAttribute(trsv_packed_kernel<S, T, ROWS, D, MERGED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)ring);
+    if (e != cudaSuccess) return e;
+    configured.fetch_or(bit);
+  }
+  trsv_packed_kernel<S, T, ROWS, D, MERGED><<<1, T, ring, s>>>(L.nlev, L.r, L.lvlptr, L.poff, (const S*)L.pval, L.moff,
+                                                         L.mval, L.pflags, (S*)t);
+  DIAF_COUNT_LAUNCH();
+  return cudaGetLastError();
+}
+
+template <class S, bool MERGED>
+static cudaError_t trsv_packed(const LevelCsr& L, const void* x, void* t, cudaStream_t s) {
+  if constexpr (MERGED)
+    group_rhs_kernel<<<ceil_div(L.nlev, L.r), 256, 0, s>>>(L.nlev, L.r, L.lvlptr, L.poff, (const double*)L.pval,
+                                                           (const double*)L.dinv, L.xrow, (const double*)x,
+                                                           (double*)t, L.pflags);
+  else
+    scale_rhs_kernel<S><<<ceil_div(L.n, 256), 256, 0, s>>>(L.n, (const S*)L.dinv, L.xrow, (const S*)x, (S*)t);
+  DIAF_COUNT_LAUNCH();
+  // (64 registers a thread, as 1,024 threads would have, spill: more rows each instead)
+  if (L.maxg <= 256) return trsv_packed_t<S, 256, 1, 4, MERGED>(L, t, s);
+  if (L.maxg <= 512) return trsv_packed_t<S, 512, 1, 2, MERGED>(L, t, s);
+  return trsv_packed_t<S, 512, 2, sizeof(S) == 8 ? 2 : 1, MERGED>(L, t, s);
 }
 
 template <class S>
@@ -447,6 +791,8 @@ static cudaError_t trsv_levels_perm_t(const LevelCsr& L, const void* x, void* t,
 
 cudaError_t trsv_levels_perm(const LevelCsr& L, bool cplx, const void* x, void* t, cudaStream_t s, bool warm) {
   if (L.n <= 0) return cudaSuccess;
+  if (L.r > 1) return trsv_packed<double, true>(L, x, t, s);
+  if (L.r == 1) return cplx ? trsv_packed<Cx<double>, false>(L, x, t, s) : trsv_packed<double, false>(L, x, t, s);
   return cplx ? trsv_levels_perm_t<Cx<double>>(L, x, t, warm, s) : trsv_levels_perm_t<double>(L, x, t, warm, s);
 }
 

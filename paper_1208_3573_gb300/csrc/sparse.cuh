@@ -38,22 +38,48 @@ struct LevelCsr {
   void* dinv = nullptr;         // n
   int32_t* xrow = nullptr;      // n
   int maxw = 0;                 // rows of the widest level (picks the solve kernel)
+  // The packed form (r > 0; then a real V's rowptr, colidx and vals are not filled), for
+  // a V of at most kPackEntries off-diagonal entries per row: entry q of
+  // position p at [kPackEntries p + q], its column position (-1: none) and its
+  // value.  Levels are solved in groups of r: with r > 1 the rows of a
+  // group also have merged entries (kMergeEntries each), which refer to rows of
+  // earlier groups only (pflags: where they do not fit or lie too far back, the
+  // solve goes level by level).
+  int r = 0;
+  int maxg = 0;                 // rows of the widest group
+  int32_t* poff = nullptr;      // kPackEntries n
+  void* pval = nullptr;         // kPackEntries n
+  int32_t* moff = nullptr;      // kMergeEntries n (r > 1)
+  double* mval = nullptr;       // kMergeEntries n (r > 1)
+  uint32_t* pflags = nullptr;   // device: what the solve has to know of the entries (kPackMergeFull, kPackFar)
 };
+constexpr int kPackEntries = 4;
+constexpr int kMergeEntries = 6;
+constexpr int kGroupRows = 1024;  // rows of a group of levels: one thread each
+enum : uint32_t {
+  kPackMergeFull = 1u,  // a merged row has more than kMergeEntries entries: the solve goes level by level
+  kPackFar = 2u,        // an entry lies further back than the solve's shared-memory window
+};
+// Levels per group for a V of `maxrow` off-diagonal entries per row at most
+// (0: not the packed form) and the rows of the widest group.
+int level_group(bool cplx, int maxrow, int nlev, const int32_t* lvlptr, int* maxg);
 
 // L's row layout from the host's level walk (device arrays): row i of V goes
 // to position pos[i] = lvlptr[lev[i]] + rank[i] (xrow[pos[i]] = i), and
-// rowptr (n + 1) counts rcnt[i] off-diagonal entries at that position.  work
-// needs n + scan_blocksums_size(n) int32.
-cudaError_t level_place(int n, const int32_t* lev, const int32_t* rank, const int32_t* rcnt, const int32_t* lvlptr,
-                        int32_t* pos, int32_t* xrow, int32_t* work, int32_t* rowptr, cudaStream_t s);
+// rowptr (n + 1) counts rcnt[i] off-diagonal entries at that position (the
+// packed form: its column positions are set to -1 instead).  work needs
+// n + scan_blocksums_size(n) int32.
+cudaError_t level_place(int n, bool cplx, const int32_t* lev, const int32_t* rank, const int32_t* rcnt, int32_t* pos,
+                        int32_t* work, LevelCsr& L, cudaStream_t s);
 
 // L's entries straight from V's columns (cp, ri, v: V in CSC): entry e =
 // (i, j) of column j, i != j, goes to L.rowptr[pos[i]] + slot[e] with column
-// pos[j] and value v_ij / v_ii (v_ii at entry dpos[i]); the diagonal gives
-// L.dinv[pos[j]] = 1 / v_jj.  *zflag (zeroed by the caller) becomes nonzero
+// pos[j] and value v_ij / v_ii (v_ii at entry dpos[i]), or to entry slot[e] of
+// the packed form, whose groups are then merged (lev: the rows' levels); the diagonal gives L.dinv[pos[j]] = 1 / v_jj.  *zflag (zeroed by the caller) becomes nonzero
 // when a diagonal value is zero or not a number.
 cudaError_t level_fill(int n, bool cplx, const int32_t* cp, const int32_t* ri, const void* v, const int32_t* dpos,
-                       const int32_t* slot, const int32_t* pos, LevelCsr& L, uint32_t* zflag, cudaStream_t s);
+                       const int32_t* slot, const int32_t* pos, const int32_t* lev, LevelCsr& L, uint32_t* zflag,
+                       cudaStream_t s);
 
 // cout[e] = pos[cin[e]] (column indices renumbered to level positions).
 cudaError_t remap_columns(int64_t nnz, const int32_t* pos, const int32_t* cin, int32_t* cout, cudaStream_t s);
