@@ -1248,7 +1248,7 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   }
   // the packed form's arrays (used when the walk finds the rows short enough);
   // without the memory for them the level-ordered rows above do
-  int32_t *poff = nullptr, *moff = nullptr;
+  int32_t *poff = nullptr, *mpos = nullptr, *moff = nullptr;
   double* mval = nullptr;
   void* pval = nullptr;
   uint32_t* pflags = nullptr;
@@ -1257,7 +1257,8 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
     c.add(&poff, (size_t)kPackEntries * n);
     c.add((char**)&pval, esz * kPackEntries * n);
     if (!cplx) {
-      c.add(&moff, (size_t)kMergeEntries * n);
+      c.add(&mpos, (size_t)kMergeEntries * n);
+      c.add(&moff, (size_t)kMergeStride * n);
       c.add(&mval, (size_t)kMergeEntries * n);
     }
     c.add(&pflags, 1);
@@ -1344,6 +1345,7 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   Vl.r = poff ? level_group(cplx, lw.maxrow, nlev, ptr, &Vl.maxg) : 0;
   Vl.poff = poff;
   Vl.pval = pval;
+  Vl.mpos = mpos;
   Vl.moff = moff;
   Vl.mval = mval;
   Vl.pflags = pflags;

@@ -1,6 +1,7 @@
 // Row-oriented sparse operations for the solve phase.
 #include <atomic>
 #include <climits>
+#include <type_traits>
 
 #include "plan.cuh"
 #include "sparse.cuh"
@@ -133,14 +134,19 @@ constexpr int level_window() { return 131072 / (int)sizeof(S); }  // 128 KB ring
 __global__ void level_place_kernel(int n, const int32_t* __restrict__ lev, const int32_t* __restrict__ rank,
                                    const int32_t* __restrict__ rcnt, const int32_t* __restrict__ lvlptr,
                                    int32_t* __restrict__ pos, int32_t* __restrict__ xrow, int32_t* __restrict__ len,
-                                   int32_t* __restrict__ poff) {
+                                   int32_t* __restrict__ poff, double* __restrict__ pval) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int p = lvlptr[lev[i]] + rank[i];
   pos[i] = p;
   xrow[p] = i;
-  if (poff) reinterpret_cast<int4*>(poff)[p] = make_int4(-1, -1, -1, -1);
-  else len[p] = rcnt[i];
+  if (poff) {  // every place empty; its value is read all the same (times zero)
+    reinterpret_cast<int4*>(poff)[p] = make_int4(-1, -1, -1, -1);
+    double2* const v = reinterpret_cast<double2*>(pval) + 2 * (size_t)p;
+    v[0] = v[1] = make_double2(0.0, 0.0);
+  } else {
+    len[p] = rcnt[i];
+  }
 }
 
 // V's rows level by level, straight from its columns: kConvLanes lanes per
@@ -215,7 +221,7 @@ __global__ void pack_rows_kernel(int nlev, const int32_t* __restrict__ lvlptr, c
       for (int q = 0; q < kPackEntries; ++q) {
         const int c = q < len ? colidx[a + q] : -1;
         poff[(size_t)kPackEntries * p + q] = c;
-        if (q < len) pval[(size_t)kPackEntries * p + q] = vals[a + q];
+        pval[(size_t)kPackEntries * p + q] = q < len ? vals[a + q] : sc_zero<Cx<double>>();
         if (c >= 0 && c < e - level_window<Cx<double>>()) atomicOr(pflags, kPackFar);
       }
     }
@@ -460,7 +466,7 @@ __global__ void __launch_bounds__(kDeepThreads, 1)
 // row's merged entries.
 __global__ void __launch_bounds__(256) merge_kernel(int nlev, int r, const int32_t* __restrict__ lvlptr,
                                                     const int32_t* __restrict__ poff, const double* __restrict__ pval,
-                                                    int32_t* moff, double* mval, uint32_t* pflags) {
+                                                    int32_t* mpos, int32_t* moff, double* mval, uint32_t* pflags) {
   const int l0 = blockIdx.x * r;
   const int l1 = l0 + r < nlev ? l0 + r : nlev;
   const int gs = lvlptr[l0];
@@ -494,18 +500,21 @@ __global__ void __launch_bounds__(256) merge_kernel(int nlev, int r, const int32
         if (col < gs) {
           add(col, val);
         } else {
-          for (int u = 0; u < kMergeEntries; ++u) {
-            const int32_t k = moff[kMergeEntries * (size_t)col + u];
-            if (k >= 0) add(k, -val * mval[kMergeEntries * (size_t)col + u]);
-          }
+          const int cnt = moff[kMergeStride * (size_t)col + kMergeEntries];
+          for (int u = 0; u < cnt; ++u)
+            add(mpos[kMergeEntries * (size_t)col + u], -val * mval[kMergeEntries * (size_t)col + u]);
         }
       }
       if (full) atomicOr(pflags, kPackMergeFull);
+      int cnt = 0;
 #pragma unroll
       for (int q = 0; q < kMergeEntries; ++q) {
-        moff[kMergeEntries * (size_t)p + q] = c[q];
+        cnt += c[q] >= 0;
+        mpos[kMergeEntries * (size_t)p + q] = c[q];
+        moff[kMergeStride * (size_t)p + q] = c[q] & (level_window<double>() - 1);
         mval[kMergeEntries * (size_t)p + q] = -v[q];  // (the solve subtracts)
       }
+      moff[kMergeStride * (size_t)p + kMergeEntries] = cnt;
     }
     __syncthreads();  // the level's merged rows are visible to the block
   }
@@ -541,49 +550,67 @@ __global__ void __launch_bounds__(256) group_rhs_kernel(int nlev, int r, const i
   }
 }
 
-// A row as it is loaded groups ahead: nothing is computed from it before its
-// group's turn (an operation on it at the load waits for the load: 0.36
-// against 0.18 ms a solve with the values negated on arrival).
+// The solve of the packed form by T threads, LPR lanes per row: one for real
+// rows, two for complex ones (the real and the imaginary part).  A thread has
+// up to ROWS rows of a group in registers, loaded D groups ahead (what is wider
+// than that goes through memory).  NEAR: every entry is in the ring.
+//
+// A sub-core of this chip takes one FP64 warp instruction every 64 cycles,
+// however few of its lanes are live, and all four together one every 19
+// (measured), so what counts is the number of FP64 instructions on the fullest
+// sub-core.  A warp therefore runs as many entries as its longest row has --
+// one branch to straight-line code, the shorter rows against a zero slot -- and
+// not a predicated FMA for every place of the packed form; and a complex row's
+// 16 FMAs are spread over two lanes.
+//
+// Nothing is computed from a row before its group's turn: an operation on what
+// was loaded waits for the load (0.36 against 0.18 ms a solve with the values
+// negated on arrival).
 template <class S, int K>
 struct PackedRow {
-  int32_t c[K];
+  int32_t c[K];  // positions (-1: none); of merged rows ring slots, then the count in n
+  int32_t n;
   S v[K];
-  S x;
-  __device__ __forceinline__ void load(const int32_t* off, const S* val, const S* t, int p) {
-    static_assert(K % 2 == 0, "whole 8-byte pairs of columns");
-    const int2* o = reinterpret_cast<const int2*>(off + (size_t)K * p);
-#pragma unroll
-    for (int q = 0; q < K / 2; ++q) {
-      const int2 w = __ldg(o + q);
-      c[2 * q] = w.x;
-      c[2 * q + 1] = w.y;
+  double x;
+  __device__ __forceinline__ void load(const int32_t* off, const S* val, const double* t, size_t p, int lpr, int part) {
+    if constexpr (K == kMergeEntries) {
+      const int4* o = reinterpret_cast<const int4*>(off + kMergeStride * p);
+      const int4 w0 = __ldg(o), w1 = __ldg(o + 1);
+      c[0] = w0.x; c[1] = w0.y; c[2] = w0.z; c[3] = w0.w;
+      c[4] = w1.x; c[5] = w1.y;
+      n = w1.z;
+    } else {
+      const int4 w = __ldg(reinterpret_cast<const int4*>(off + K * p));
+      c[0] = w.x; c[1] = w.y; c[2] = w.z; c[3] = w.w;
     }
     constexpr int PV = 16 / (int)sizeof(S);
-    const Pack16<S>* vv = reinterpret_cast<const Pack16<S>*>(val + (size_t)K * p);
+    const Pack16<S>* vv = reinterpret_cast<const Pack16<S>*>(val + K * p);
 #pragma unroll
     for (int q = 0; q < K / PV; ++q) {
       const Pack16<S> w = vv[q];
 #pragma unroll
       for (int u = 0; u < PV; ++u) v[q * PV + u] = w.v[u];
     }
-    x = t[p];
+    x = t[lpr * p + part];
   }
 };
 
-// The solve of the packed form by T threads; a thread has up to ROWS rows of a
-// group in registers, loaded D groups ahead (what is wider than that goes
-// through memory).  NEAR: every entry is in the ring.
 template <class S, int K, int T, int ROWS, int D, bool NEAR>
 __device__ __forceinline__ void packed_solve(int ng, const int32_t* __restrict__ ptr, const int32_t* __restrict__ off,
-                                             const S* __restrict__ val, S* t, S* tw) {
+                                             const S* __restrict__ val, double* t, double* tw) {
   constexpr int kWin = level_window<S>();
-  const int tid = (int)threadIdx.x;
+  constexpr int LPR = ScalarInfo<S>::cplx ? 2 : 1;
+  constexpr int TR = T / LPR;  // rows in step
+  constexpr bool kRingSlots = K == kMergeEntries;
+  const int tid = (int)threadIdx.x / LPR, part = LPR == 2 ? (int)threadIdx.x & 1 : 0;
+  const int wrow = ((int)threadIdx.x & ~31) / LPR;  // the warp's first row
+  const int odd = part << 31;
   PackedRow<S, K> row[D][ROWS];
   auto fetch = [&](PackedRow<S, K>(&w)[ROWS], int g) {
     const int b = ptr[g] + tid, e = ptr[g + 1];
 #pragma unroll
     for (int u = 0; u < ROWS; ++u)
-      if (b + u * T < e) w[u].load(off, val, t, b + u * T);
+      if (b + u * TR < e) w[u].load(off, val, t, b + u * TR, LPR, part);
   };
 #pragma unroll
   for (int k = 0; k < D; ++k)
@@ -595,25 +622,66 @@ __device__ __forceinline__ void packed_solve(int ng, const int32_t* __restrict__
       const int g = g0 + k;
       if (g >= ng) break;  // uniform
       const int e = ptr[g + 1];
-      auto solve = [&](const PackedRow<S, K>& w, int p) {
-        S tv[K];  // all reads of t, then the chain
+      // a warp's 32 / LPR rows from its own one on; live: the lane has a row
+      auto solve = [&](const PackedRow<S, K>& w, int p, bool live) {
+        int n = 0;
+        if constexpr (kRingSlots) {
+          if (live) n = w.n;
+        } else {
+          if (live) n = w.c[3] >= 0 ? 4 : (w.c[2] >= 0 ? 3 : (w.c[1] >= 0 ? 2 : (w.c[0] >= 0 ? 1 : 0)));
+        }
+        const int nw = __reduce_max_sync(DIAF_FULL, n);
+        double acc = w.x;
+        auto run = [&](auto count) {
+          constexpr int Q = decltype(count)::value;
+          const double* src[Q];
 #pragma unroll
-        for (int q = 0; q < K; ++q)
-          if (w.c[q] >= 0) tv[q] = NEAR || w.c[q] >= e - kWin ? tw[w.c[q] & (kWin - 1)] : t[w.c[q]];
-        S acc = w.x;
+          for (int q = 0; q < Q; ++q) {
+            const bool has = q < n;
+            if (kRingSlots) src[q] = tw + (has ? w.c[q] : kWin);
+            else if (NEAR) src[q] = tw + LPR * (has ? w.c[q] & (kWin - 1) : kWin);
+            else src[q] = !has || w.c[q] >= e - kWin ? tw + LPR * (has ? w.c[q] & (kWin - 1) : kWin)
+                                                     : t + (size_t)LPR * w.c[q];
+          }
+          if constexpr (LPR == 1) {
+            double tv[Q];
 #pragma unroll
-        for (int q = 0; q < K; ++q)
-          if (w.c[q] >= 0) acc = sc_msub(acc, w.v[q], tv[q]);
-        t[p] = acc;
-        tw[p & (kWin - 1)] = acc;
+            for (int q = 0; q < Q; ++q) tv[q] = *src[q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) acc = fma(-w.v[q], tv[q], acc);
+          } else {  // re: (acc - v.re t.re) + v.im t.im; im: (acc - v.re t.im) - v.im t.re
+            double t0[Q], t1[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+              t0[q] = src[q][part];
+              t1[q] = src[q][1 - part];
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+              const double im = __hiloint2double(__double2hiint(w.v[q].im) ^ odd, __double2loint(w.v[q].im));
+              acc = fma(im, t1[q], fma(-w.v[q].re, t0[q], acc));
+            }
+          }
+        };
+        if (nw == 2) run(std::integral_constant<int, 2>());
+        else if (nw == 3) run(std::integral_constant<int, 3>());
+        else if (nw == 4) run(std::integral_constant<int, 4>());
+        else if (nw == 1) run(std::integral_constant<int, 1>());
+        else if (K > 4 && nw == 5) run(std::integral_constant<int, K < 5 ? K : 5>());
+        else if (K > 4 && nw == 6) run(std::integral_constant<int, K < 6 ? K : 6>());
+        if (live) {
+          t[(size_t)LPR * p + part] = acc;
+          tw[LPR * (p & (kWin - 1)) + part] = acc;
+        }
       };
 #pragma unroll
       for (int u = 0; u < ROWS; ++u)
-        if (b + tid + u * T < e) solve(row[k][u], b + tid + u * T);
-      for (int p = b + tid + ROWS * T; p < e; p += T) {
+        if (b + wrow + u * TR < e) solve(row[k][u], b + tid + u * TR, b + tid + u * TR < e);
+      for (int p0 = b + wrow + ROWS * TR; p0 < e; p0 += TR) {
+        const int p = p0 + tid - wrow;
         PackedRow<S, K> w;
-        w.load(off, val, t, p);
-        solve(w, p);
+        if (p < e) w.load(off, val, t, p, LPR, part);
+        solve(w, p, p < e);
       }
       if (g + D < ng) fetch(row[k], g + D);
       b = e;
@@ -628,9 +696,10 @@ template <class S, int T, int ROWS, int D, bool MERGED>
 __global__ void __launch_bounds__(T, 1)
     trsv_packed_kernel(int nlev, int r, const int32_t* __restrict__ lvlptr, const int32_t* __restrict__ poff,
                        const S* __restrict__ pval, const int32_t* __restrict__ moff, const double* __restrict__ mval,
-                       const uint32_t* __restrict__ pflags, S* t) {
+                       const uint32_t* __restrict__ pflags, double* t) {
   extern __shared__ __align__(16) unsigned char level_ring[];
-  S* tw = reinterpret_cast<S*>(level_ring);
+  double* tw = reinterpret_cast<double*>(level_ring);
+  if (threadIdx.x < 2) tw[level_window<double>() + threadIdx.x] = 0.0;  // the zero slot
   __shared__ int32_t sptr[kLevelPtrSmem + 1];
   const uint32_t fl = *pflags;
   const bool merged = MERGED && !fl;
@@ -678,7 +747,7 @@ cudaError_t level_place(int n, bool cplx, const int32_t* lev, const int32_t* ran
   int32_t* bs = work + n;
   const bool rows = L.r == 0 || cplx;  // the rows' pointers are needed
   level_place_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, lev, rank, rcnt, L.lvlptr, pos, L.xrow, len,
-                                                      rows ? nullptr : L.poff);
+                                                      rows ? nullptr : L.poff, (double*)L.pval);
   DIAF_COUNT_LAUNCH();
   return rows ? exclusive_scan_i32(len, L.rowptr, n, bs, s) : cudaGetLastError();
 }
@@ -707,8 +776,8 @@ cudaError_t level_fill(int n, bool cplx, const int32_t* cp, const int32_t* ri, c
                                               L.poff, (double*)L.pval, (double*)L.dinv, zflag, L.pflags);
     DIAF_COUNT_LAUNCH();
     if (L.r > 1) {
-      merge_kernel<<<ceil_div(L.nlev, L.r), 256, 0, s>>>(L.nlev, L.r, L.lvlptr, L.poff, (const double*)L.pval, L.moff,
-                                                         L.mval, L.pflags);
+      merge_kernel<<<ceil_div(L.nlev, L.r), 256, 0, s>>>(L.nlev, L.r, L.lvlptr, L.poff, (const double*)L.pval, L.mpos,
+                                                         L.moff, L.mval, L.pflags);
       DIAF_COUNT_LAUNCH();
     }
   } else {
@@ -730,7 +799,7 @@ cudaError_t remap_columns(int64_t nnz, const int32_t* pos, const int32_t* cin, i
 
 template <class S, int T, int ROWS, int D, bool MERGED>
 static cudaError_t trsv_packed_t(const LevelCsr& L, void* t, cudaStream_t s) {
-  constexpr size_t ring = sizeof(S) * level_window<S>();
+  constexpr size_t ring = sizeof(S) * level_window<S>() + 16;  // and the zero slot
   static std::atomic<uint64_t> configured{0};  // the attribute is per device: one bit each
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -743,7 +812,7 @@ static cudaError_t trsv_packed_t(const LevelCsr& L, void* t, cudaStream_t s) {
     configured.fetch_or(bit);
   }
   trsv_packed_kernel<S, T, ROWS, D, MERGED><<<1, T, ring, s>>>(L.nlev, L.r, L.lvlptr, L.poff, (const S*)L.pval, L.moff,
-                                                         L.mval, L.pflags, (S*)t);
+                                                         L.mval, L.pflags, (double*)t);
   DIAF_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -758,9 +827,15 @@ static cudaError_t trsv_packed(const LevelCsr& L, const void* x, void* t, cudaSt
     scale_rhs_kernel<S><<<ceil_div(L.n, 256), 256, 0, s>>>(L.n, (const S*)L.dinv, L.xrow, (const S*)x, (S*)t);
   DIAF_COUNT_LAUNCH();
   // (64 registers a thread, as 1,024 threads would have, spill: more rows each instead)
-  if (L.maxg <= 256) return trsv_packed_t<S, 256, 1, 4, MERGED>(L, t, s);
-  if (L.maxg <= 512) return trsv_packed_t<S, 512, 1, 2, MERGED>(L, t, s);
-  return trsv_packed_t<S, 512, 2, sizeof(S) == 8 ? 2 : 1, MERGED>(L, t, s);
+  if constexpr (ScalarInfo<S>::cplx) {
+    if (L.maxg <= 128) return trsv_packed_t<S, 256, 1, 4, MERGED>(L, t, s);
+    if (L.maxg <= 256) return trsv_packed_t<S, 512, 1, 2, MERGED>(L, t, s);
+    return trsv_packed_t<S, 512, 2, 1, MERGED>(L, t, s);
+  } else {
+    if (L.maxg <= 256) return trsv_packed_t<S, 256, 1, 4, MERGED>(L, t, s);
+    if (L.maxg <= 512) return trsv_packed_t<S, 512, 1, 2, MERGED>(L, t, s);
+    return trsv_packed_t<S, 512, 2, 2, MERGED>(L, t, s);
+  }
 }
 
 template <class S>

@@ -49,12 +49,14 @@ struct LevelCsr {
   int maxg = 0;                 // rows of the widest group
   int32_t* poff = nullptr;      // kPackEntries n
   void* pval = nullptr;         // kPackEntries n
-  int32_t* moff = nullptr;      // kMergeEntries n (r > 1)
+  int32_t* mpos = nullptr;      // kMergeEntries n (r > 1): the merged entries' column positions
+  int32_t* moff = nullptr;      // kMergeStride n: their slots in the solve's window, then their number
   double* mval = nullptr;       // kMergeEntries n (r > 1)
   uint32_t* pflags = nullptr;   // device: what the solve has to know of the entries (kPackMergeFull, kPackFar)
 };
 constexpr int kPackEntries = 4;
 constexpr int kMergeEntries = 6;
+constexpr int kMergeStride = 8;
 constexpr int kGroupRows = 1024;  // rows of a group of levels: one thread each
 enum : uint32_t {
   kPackMergeFull = 1u,  // a merged row has more than kMergeEntries entries: the solve goes level by level
