@@ -415,6 +415,18 @@ diaf_status diaf_sparsified_count(const diaf_csc* A, int32_t k, int32_t p_l, int
 diaf_status diaf_sparsified_fill(const diaf_csc* A, int32_t k, int32_t p_l, int32_t keep, const int32_t* colptr,
                                  int32_t* rowidx, void* stream);
 
+/* The same pattern in one pass where `keep` (>= 1) bounds the entries of a
+ * column (Sec. 4.1): diaf_sparsified_rows writes the sorted rows of column j
+ * to d_rows[keep j ..] (device, n keep), colptr (device, n + 1) and the entry
+ * count, and synchronises the stream; diaf_sparsified_pack then writes rowidx
+ * (device, nnz) from them.  Errors as diaf_sparsified_count. */
+diaf_status diaf_sparsified_rows(const diaf_csc* A, int32_t k, int32_t p_l, int32_t keep, int32_t* d_rows,
+                                 int32_t* colptr, int64_t* nnz, void* stream);
+/* Second step of the one-pass pattern (Sec. 4.1): d_rows and colptr of
+ * diaf_sparsified_rows to rowidx; stream work only. */
+diaf_status diaf_sparsified_pack(int32_t n, int32_t keep, const int32_t* d_rows, const int32_t* colptr,
+                                 int32_t* rowidx, void* stream);
+
 /* ---- Learned proposal of the W pattern J_j ----------------------------------
  * Not in the paper: Sec. 4 chooses J_j by fixed rules (pattern(A), powers of
  * A, dropping by position).  Here a small network scores every candidate row

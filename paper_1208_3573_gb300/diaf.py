@@ -157,6 +157,9 @@ def lib() -> ctypes.CDLL:
                                             vp, ctypes.POINTER(ctypes.c_int64), vp]
         L.diaf_sparsified_fill.argtypes = [ctypes.POINTER(CSC_t), ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
                                            vp, vp, vp]
+        L.diaf_sparsified_rows.argtypes = [ctypes.POINTER(CSC_t), ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
+                                           vp, vp, ctypes.POINTER(ctypes.c_int64), vp]
+        L.diaf_sparsified_pack.argtypes = [ctypes.c_int32, ctypes.c_int32, vp, vp, vp, vp]
         L.diaf_level_schedule.argtypes = [ctypes.c_int32, vp, vp, vp, ctypes.POINTER(ctypes.c_int32),
                                           ctypes.POINTER(ctypes.c_int32)]
         L.diaf_status_string.argtypes = [ctypes.c_int]
@@ -524,16 +527,32 @@ def toggle_targets(CAND: DeviceCSC, in_base: torch.Tensor, r0: torch.Tensor, rt:
     return value
 
 
+# the one-pass form holds n x keep rows; beyond this many the two-pass one is as good and holds fewer
+ONE_PASS_KEEP = 64
+
+
 def sparsified_powers(A: DeviceCSC, k: int = 2, p_l: int = 0, keep: int = 0, stream=None) -> DeviceCSC:
-    """W pattern by sparsified powers (diaf_sparsified_count / _fill)."""
+    """W pattern by sparsified powers (diaf_sparsified_rows / _pack when at most
+    ONE_PASS_KEEP entries per column are kept, else diaf_sparsified_count / _fill)."""
     L = lib()
     a = A.csc_t()
     s = _stream(stream)
-    colptr = torch.empty(A.n + 1, dtype=torch.int32, device=A.colptr.device)
+    dev = A.colptr.device
+    colptr = torch.empty(A.n + 1, dtype=torch.int32, device=dev)
     nnz = ctypes.c_int64()
-    _check(L.diaf_sparsified_count(ctypes.byref(a), k, p_l, keep, _ptr(colptr), ctypes.byref(nnz), s))
-    rowidx = torch.empty(max(int(nnz.value), 1), dtype=torch.int32, device=A.colptr.device)
-    _check(L.diaf_sparsified_fill(ctypes.byref(a), k, p_l, keep, _ptr(colptr), _ptr(rowidx), s))
+    one_pass = 1 <= keep <= ONE_PASS_KEEP
+    if one_pass:
+        rows = torch.empty(max(A.n * keep, 1), dtype=torch.int32, device=dev)
+        _check(L.diaf_sparsified_rows(ctypes.byref(a), k, p_l, keep, _ptr(rows), _ptr(colptr), ctypes.byref(nnz), s))
+    else:
+        _check(L.diaf_sparsified_count(ctypes.byref(a), k, p_l, keep, _ptr(colptr), ctypes.byref(nnz), s))
+    rowidx = torch.empty(max(int(nnz.value), 1), dtype=torch.int32, device=dev)
+    if one_pass:
+        _check(L.diaf_sparsified_pack(A.n, keep, _ptr(rows), _ptr(colptr), _ptr(rowidx), s))
+        if s != torch.cuda.current_stream(dev).cuda_stream:  # rows goes back to its own stream's pool
+            rows.record_stream(torch.cuda.ExternalStream(s, device=dev))
+    else:
+        _check(L.diaf_sparsified_fill(ctypes.byref(a), k, p_l, keep, _ptr(colptr), _ptr(rowidx), s))
     return DeviceCSC(A.n, colptr, rowidx[:int(nnz.value)])
 
 

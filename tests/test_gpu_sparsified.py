@@ -90,3 +90,25 @@ def test_sparsified_rejects_zero_diagonal_and_overflow(D):
     with pytest.raises(D.DiafError) as e:
         D.sparsified_powers(Az, 2, 0, 0)
     assert e.value.status == D.DIAF_EINVAL
+
+
+@pytest.mark.parametrize("k", [1, 2])
+@pytest.mark.parametrize("half", [(3, 4), (4, 4), (16, 16), (16, 17), (31, 32), (32, 32)])
+def test_sparsified_list_lengths(D, half, k):
+    """Columns of 8, 9, 33, 34, 64 and 65 entries: at and beyond the short
+    lists' 32 entries of t and 64 products, with every way of keeping entries."""
+    lo, hi = half
+    rng = np.random.default_rng(lo + hi)
+    n = 150
+    import scipy.sparse as sp
+    from workloads import CSC
+    M = sp.diags([rng.standard_normal(n - abs(d)) * (1.0 if d else 0.0) + (8.0 if d == 0 else 0.0)
+                  for d in range(-lo, hi + 1)], range(-lo, hi + 1))
+    A = CSC.from_scipy(M.tocsc())
+    p_l = 7 if k > 1 and lo + hi > 15 else 0
+    for keep in (0, 1, 5, 64, 65):
+        P = D.sparsified_powers(D.DeviceCSC.from_host(A), k, p_l, keep)
+        o = oracle_sp(A, k, p_l, keep)
+        cp, ri = _host(P)
+        np.testing.assert_array_equal(cp, o.colptr)
+        np.testing.assert_array_equal(ri, o.rowidx)
