@@ -5,6 +5,7 @@
 // scoring the candidate, and the selection of the diagonal plus the best
 // keep-1 candidates.  Training: mean squared error of the score against a
 // per-candidate target, backward pass, Adam.
+#include <algorithm>
 #include <string>
 
 #include "factors.cuh"
@@ -32,12 +33,33 @@ __device__ __forceinline__ int find_sorted(const int32_t* a, int n, int key) {
   return -1;
 }
 
+// |v|, the root of |v|^2 (for a real value that is |v| itself: no root)
+__device__ __forceinline__ double modulus(double v) { return fabs(v); }
+__device__ __forceinline__ double modulus(Cx<double> v) { return sqrt(sc_abs2(v)); }
+
 // |value| of the entry (row, col) of A, 0 when absent (binary search in the column)
 template <class S>
 __device__ __forceinline__ double entry_abs(const int32_t* Acp, const int32_t* Ari, const S* Av, int row, int col) {
   const int a0 = Acp[col];
   const int pos = find_sorted(Ari + a0, Acp[col + 1] - a0, row);
-  return pos >= 0 ? sqrt((double)sc_abs2(Av[a0 + pos])) : 0.0;
+  return pos >= 0 ? modulus(Av[a0 + pos]) : 0.0;
+}
+
+// |a_jj| and its logarithm per column: every candidate's f4 would otherwise
+// search, divide and take a logarithm for itself.
+template <class S>
+__global__ void diag_log_kernel(int n, const int32_t* __restrict__ Acp, const int32_t* __restrict__ Ari,
+                                const S* __restrict__ Av, double2* __restrict__ dlog) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const double d = entry_abs(Acp, Ari, Av, j, j);
+  dlog[j] = make_double2(d, d > 0.0 ? log(d) : 0.0);
+}
+
+// x / d (0 for d = 0) by d's reciprocal r; a divisor whose reciprocal is not
+// a normal number divides
+__device__ __forceinline__ float scaled(double x, double r, double d) {
+  return d > 0.0 ? (float)(r > 1e-300 && r < 1e300 ? x * r : x / d) : 0.0f;
 }
 
 // Features of candidate c of column j (one warp per column; lane l takes the
@@ -47,11 +69,16 @@ __device__ __forceinline__ double entry_abs(const int32_t* Acp, const int32_t* A
 //   f4 log(|a_cc| / |a_jj|) in [-10, 10]
 //   f5 |A_jc| / |a_jj|              f6 nnz(A(:,c)) / nnz(A(:,j))
 //   f7 +1 for c < j, -1 for c > j, 0 on the diagonal
+// What bounded it was the one FP64 pipe (an instruction per 64 cycles and
+// sub-core): square roots of squares, three divisions and a logarithm per
+// candidate.  Moduli are taken directly, the divisors' reciprocals once per
+// column, the logarithms once per row of A (f4 as their difference):
+// lognormal 40^3 (64,000 columns of 25 candidates) 0.93 -> 0.42 ms.
 template <class S>
 __global__ void __launch_bounds__(kFeatWarps * 32)
     features_kernel(int n, const int32_t* __restrict__ Acp, const int32_t* __restrict__ Ari, const S* __restrict__ Av,
-                    const int32_t* __restrict__ Ccp, const int32_t* __restrict__ Cri, float* __restrict__ feat,
-                    uint32_t* status) {
+                    const int32_t* __restrict__ Ccp, const int32_t* __restrict__ Cri,
+                    const double2* __restrict__ dlog, float* __restrict__ feat, uint32_t* status) {
   __shared__ int32_t cand[kFeatWarps][kCandMax];
   __shared__ S acc[kFeatWarps][kCandMax];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -81,15 +108,16 @@ __global__ void __launch_bounds__(kFeatWarps * 32)
   }
   __syncwarp();
   const int a0 = Acp[j], na = Acp[j + 1] - a0;
-  double aj_max = 0.0, ajj = 0.0;
+  double aj_max = 0.0;
+  const double2 dj = dlog[j];
+  const double ajj = dj.x;
   double acj[kCandPerLane];
 #pragma unroll
   for (int u = 0; u < kCandPerLane; ++u) acj[u] = 0.0;
   for (int p = 0; p < na; ++p) {
     const int r = Ari[a0 + p];
-    const double v = sqrt((double)sc_abs2(Av[a0 + p]));
+    const double v = modulus(Av[a0 + p]);
     aj_max = v > aj_max ? v : aj_max;
-    if (r == j) ajj = v;
 #pragma unroll
     for (int u = 0; u < kCandPerLane; ++u)
       if (r == cl[u]) acj[u] = v;
@@ -115,68 +143,108 @@ __global__ void __launch_bounds__(kFeatWarps * 32)
 #pragma unroll
   for (int u = 0; u < kCandPerLane; ++u) {
     const int i = lane + 32 * u;
-    a2c[u] = i < nc ? sqrt((double)sc_abs2(acc[wib][i])) : 0.0;
+    a2c[u] = i < nc ? modulus(acc[wib][i]) : 0.0;
     a2m = a2c[u] > a2m ? a2c[u] : a2m;
   }
   const double a2max = warp_max(a2m);
+  const double raj = aj_max > 0.0 ? 1.0 / aj_max : 0.0, ra2 = a2max > 0.0 ? 1.0 / a2max : 0.0,
+               rjj = ajj > 0.0 ? 1.0 / ajj : 0.0;
 #pragma unroll
   for (int u = 0; u < kCandPerLane; ++u) {
     const int i = lane + 32 * u;
     if (i >= nc) continue;
     const int c = cl[u];
-    const double acc_diag = entry_abs(Acp, Ari, Av, c, c);
+    const double2 dc = dlog[c];
     const double ajc = entry_abs(Acp, Ari, Av, j, c);
     float* f = feat + (size_t)(c0 + i) * F;
     f[0] = c == j ? 1.0f : 0.0f;
     f[1] = acj[u] > 0.0 ? 1.0f : 0.0f;
-    f[2] = aj_max > 0.0 ? (float)(acj[u] / aj_max) : 0.0f;
-    f[3] = a2max > 0.0 ? (float)(a2c[u] / a2max) : 0.0f;
-    double lr = (acc_diag > 0.0 && ajj > 0.0) ? log(acc_diag / ajj) : 0.0;
+    f[2] = scaled(acj[u], raj, aj_max);
+    f[3] = scaled(a2c[u], ra2, a2max);
+    const double lr = (dc.x > 0.0 && ajj > 0.0) ? dc.y - dj.y : 0.0;
     f[4] = (float)(lr > 10.0 ? 10.0 : (lr < -10.0 ? -10.0 : lr));
-    f[5] = ajj > 0.0 ? (float)(ajc / ajj) : 0.0f;
+    f[5] = scaled(ajc, rjj, ajj);
     f[6] = na > 0 ? (float)(Acp[c + 1] - Acp[c]) / (float)na : 0.0f;
     f[7] = c < j ? 1.0f : (c > j ? -1.0f : 0.0f);
   }
 }
 
 // ---------------------------------------------------------------- MLP
-struct Fwd {
-  float h1[H], h2[H], y;
-};
+// kFwdRows rows per thread: a weight read from shared memory (16 bytes at a
+// time, broadcast) serves that many multiply-adds, which otherwise wait for
+// one read each.  Every row's sums keep their order.  1.5 M rows: 0.60 -> 0.096 ms (43 TFLOP/s).
+constexpr int kFwdRows = 4;
+constexpr int kFwdThreads = 128;
 
-__device__ __forceinline__ void mlp_fwd(const float* P, const float* f, Fwd& o) {
+template <int N>
+__device__ __forceinline__ void load4(const float* p, float (&w)[N]) {
 #pragma unroll
-  for (int h = 0; h < H; ++h) {
-    float s = P[OFF_B1 + h];
-#pragma unroll
-    for (int i = 0; i < F; ++i) s = fmaf(P[OFF_W1 + h * F + i], f[i], s);
-    o.h1[h] = s > 0.0f ? s : 0.0f;
+  for (int i = 0; i < N; i += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(p + i);
+    w[i] = v.x;
+    w[i + 1] = v.y;
+    w[i + 2] = v.z;
+    w[i + 3] = v.w;
   }
-#pragma unroll 4
-  for (int h = 0; h < H; ++h) {
-    float s = P[OFF_B2 + h];
-#pragma unroll
-    for (int g = 0; g < H; ++g) s = fmaf(P[OFF_W2 + h * H + g], o.h1[g], s);
-    o.h2[h] = s > 0.0f ? s : 0.0f;
-  }
-  float y = P[OFF_B3];
-#pragma unroll
-  for (int h = 0; h < H; ++h) y = fmaf(P[OFF_W3 + h], o.h2[h], y);
-  o.y = y;
 }
 
-__global__ void mlp_forward_kernel(const float* __restrict__ params, const float* __restrict__ feat, int64_t nrows,
-                                   float* __restrict__ out) {
-  __shared__ float P[NPARAM];
+__global__ void __launch_bounds__(kFwdThreads)
+    mlp_forward_kernel(const float* __restrict__ params, const float* __restrict__ feat, int64_t nrows,
+                       float* __restrict__ out) {
+  static_assert(OFF_W1 % 4 == 0 && OFF_W2 % 4 == 0 && F % 4 == 0 && H % 4 == 0, "16-byte rows of weights");
+  __shared__ __align__(16) float P[(NPARAM + 3) / 4 * 4];
   for (int i = threadIdx.x; i < NPARAM; i += blockDim.x) P[i] = params[i];
   __syncthreads();
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nrows; s += (int64_t)gridDim.x * blockDim.x) {
-    float f[F];
+  const int64_t per_block = (int64_t)kFwdThreads * kFwdRows;
+  for (int64_t base = blockIdx.x * per_block; base < nrows; base += gridDim.x * per_block) {
+    float h1[kFwdRows][H], y[kFwdRows];
+    {
+      float f[kFwdRows][F];
 #pragma unroll
-    for (int i = 0; i < F; ++i) f[i] = feat[s * F + i];
-    Fwd o;
-    mlp_fwd(P, f, o);
-    out[s] = o.y;
+      for (int u = 0; u < kFwdRows; ++u) {
+        const int64_t s = base + threadIdx.x + (int64_t)u * kFwdThreads;
+#pragma unroll
+        for (int i = 0; i < F; ++i) f[u][i] = s < nrows ? feat[s * F + i] : 0.0f;
+      }
+#pragma unroll
+      for (int h = 0; h < H; ++h) {
+        float w[F];
+        load4(P + OFF_W1 + h * F, w);
+        const float b = P[OFF_B1 + h];
+#pragma unroll
+        for (int u = 0; u < kFwdRows; ++u) {
+          float s = b;
+#pragma unroll
+          for (int i = 0; i < F; ++i) s = fmaf(w[i], f[u][i], s);
+          h1[u][h] = s > 0.0f ? s : 0.0f;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kFwdRows; ++u) y[u] = P[OFF_B3];
+#pragma unroll 1
+    for (int h = 0; h < H; ++h) {
+      float s[kFwdRows];
+#pragma unroll
+      for (int u = 0; u < kFwdRows; ++u) s[u] = P[OFF_B2 + h];
+#pragma unroll
+      for (int g = 0; g < H; g += 4) {
+        float w[4];
+        load4(P + OFF_W2 + h * H + g, w);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+          for (int u = 0; u < kFwdRows; ++u) s[u] = fmaf(w[e], h1[u][g + e], s[u]);
+      }
+      const float w3 = P[OFF_W3 + h];
+#pragma unroll
+      for (int u = 0; u < kFwdRows; ++u) y[u] = fmaf(w3, s[u] > 0.0f ? s[u] : 0.0f, y[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kFwdRows; ++u) {
+      const int64_t s = base + threadIdx.x + (int64_t)u * kFwdThreads;
+      if (s < nrows) out[s] = y[u];
+    }
   }
 }
 
@@ -185,80 +253,150 @@ __global__ void mlp_forward_kernel(const float* __restrict__ params, const float
 // gradient as a sum over the block's samples, written to the block's row of
 // `part` (NPARAM + 1 floats: the gradient, then the loss); the blocks' rows
 // are summed in block order afterwards, so the result is reproducible.
+//
+// A sample's values lie kRowLd floats apart, one row of shared memory per
+// value: a warp stores 32 samples to 32 banks, and the sums read four samples
+// at a time (16 bytes); the 32 x 32 sums of W2 go in tiles of 2 x 4 per thread,
+// the 32 x 8 of W1 in 1 x 2, so that a read serves several of them.  (With a
+// sample's values side by side every store was a 32-way bank conflict and every
+// multiply-add waited for two reads: 8,192 rows, kernel 28.7 -> 17.4 us.)
 constexpr int kGradRows = 128;
 constexpr int kPartLd = NPARAM + 1;
+constexpr int kParamLd = (NPARAM + 3) / 4 * 4;
+constexpr int kRowLd = kGradRows + 4;
+constexpr int kGradFloats = kParamLd + kRowLd * (F + 4 * H + 1);
+
+__device__ __forceinline__ float dot4(float g, float4 a, float4 b) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, g))));
+}
+__device__ __forceinline__ float add4(float g, float4 a) { return (((g + a.x) + a.y) + a.z) + a.w; }
 
 __global__ void __launch_bounds__(kGradRows)
     mlp_grad_kernel(const float* __restrict__ params, const float* __restrict__ feat, const float* __restrict__ target,
                     int64_t nrows, float* __restrict__ part) {
-  extern __shared__ float sm[];
-  float* P = sm;                        // NPARAM
-  float* sF = P + NPARAM;               // [kGradRows][F]
-  float* sH1 = sF + kGradRows * F;      // [kGradRows][H]
-  float* sH2 = sH1 + kGradRows * H;     // [kGradRows][H]
-  float* sD1 = sH2 + kGradRows * H;     // dL/d(pre-activation 1)
-  float* sD2 = sD1 + kGradRows * H;     // dL/d(pre-activation 2)
-  float* sDy = sD2 + kGradRows * H;     // [kGradRows]
+  static_assert(kGradRows == 128 && H == 32 && F == 8, "the threads' tiles of the gradient");
+  extern __shared__ __align__(16) float sm[];
+  float* P = sm;                  // NPARAM, to 16 bytes
+  float* sF = P + kParamLd;       // [F][kRowLd]
+  float* sH1 = sF + F * kRowLd;   // [H][kRowLd]
+  float* sH2 = sH1 + H * kRowLd;  // [H][kRowLd]
+  float* sD1 = sH2 + H * kRowLd;  // dL/d(pre-activation 1)
+  float* sD2 = sD1 + H * kRowLd;  // dL/d(pre-activation 2)
+  float* sDy = sD2 + H * kRowLd;  // [kRowLd]
   for (int i = threadIdx.x; i < NPARAM; i += blockDim.x) P[i] = params[i];
   __syncthreads();
   const int64_t s = blockIdx.x * (int64_t)kGradRows + threadIdx.x;
   const int t = threadIdx.x;
   float l2 = 0.0f;
   if (s < nrows) {
-    float f[F];
+    float h1[H];
+    {
+      float f[F];
 #pragma unroll
-    for (int i = 0; i < F; ++i) f[i] = sF[t * F + i] = feat[s * F + i];
-    Fwd o;
-    mlp_fwd(P, f, o);
-    const float e = o.y - target[s];
+      for (int i = 0; i < F; ++i) f[i] = sF[i * kRowLd + t] = feat[s * F + i];
+#pragma unroll
+      for (int h = 0; h < H; ++h) {
+        float w[F];
+        load4(P + OFF_W1 + h * F, w);
+        float v = P[OFF_B1 + h];
+#pragma unroll
+        for (int i = 0; i < F; ++i) v = fmaf(w[i], f[i], v);
+        h1[h] = v > 0.0f ? v : 0.0f;
+        sH1[h * kRowLd + t] = h1[h];
+      }
+    }
+    float y = P[OFF_B3];
+#pragma unroll 2
+    for (int h = 0; h < H; ++h) {
+      float v = P[OFF_B2 + h];
+#pragma unroll
+      for (int g = 0; g < H; g += 4) {
+        float w[4];
+        load4(P + OFF_W2 + h * H + g, w);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v = fmaf(w[e], h1[g + e], v);
+      }
+      v = v > 0.0f ? v : 0.0f;
+      sH2[h * kRowLd + t] = v;
+      y = fmaf(P[OFF_W3 + h], v, y);
+    }
+    const float e = y - target[s];
     l2 = e * e;
     const float dy = 2.0f * e / (float)nrows;
     sDy[t] = dy;
     float d2[H];
 #pragma unroll
     for (int h = 0; h < H; ++h) {
-      d2[h] = o.h2[h] > 0.0f ? dy * P[OFF_W3 + h] : 0.0f;
-      sH1[t * H + h] = o.h1[h];
-      sH2[t * H + h] = o.h2[h];
-      sD2[t * H + h] = d2[h];
+      d2[h] = sH2[h * kRowLd + t] > 0.0f ? dy * P[OFF_W3 + h] : 0.0f;
+      sD2[h * kRowLd + t] = d2[h];
     }
-#pragma unroll 4
-    for (int g = 0; g < H; ++g) {
-      float sacc = 0.0f;
+#pragma unroll 1
+    for (int g = 0; g < H; g += 4) {
+      float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int h = 0; h < H; ++h) sacc = fmaf(P[OFF_W2 + h * H + g], d2[h], sacc);
-      sD1[t * H + g] = o.h1[g] > 0.0f ? sacc : 0.0f;
+      for (int h = 0; h < H; ++h) {
+        float w[4];
+        load4(P + OFF_W2 + h * H + g, w);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = fmaf(w[q], d2[h], acc[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        sD1[(g + q) * kRowLd + t] = sH1[(g + q) * kRowLd + t] > 0.0f ? acc[q] : 0.0f;
     }
   } else {
     sDy[t] = 0.0f;
-#pragma unroll
-    for (int i = 0; i < F; ++i) sF[t * F + i] = 0.0f;
-    for (int h = 0; h < H; ++h) sH1[t * H + h] = sH2[t * H + h] = sD1[t * H + h] = sD2[t * H + h] = 0.0f;
+    for (int i = 0; i < F; ++i) sF[i * kRowLd + t] = 0.0f;
+    for (int h = 0; h < H; ++h)
+      sH1[h * kRowLd + t] = sH2[h * kRowLd + t] = sD1[h * kRowLd + t] = sD2[h * kRowLd + t] = 0.0f;
   }
   __syncthreads();
-  const int rows = (int)((nrows - blockIdx.x * (int64_t)kGradRows) < kGradRows ? (nrows - blockIdx.x * (int64_t)kGradRows)
-                                                                              : kGradRows);
-  for (int p = threadIdx.x; p < NPARAM; p += blockDim.x) {
-    float g = 0.0f;
-    if (p < OFF_B1) {  // W1[h][i] = sum_s d1[s][h] f[s][i]
-      const int h = p / F, i = p % F;
-      for (int r = 0; r < rows; ++r) g = fmaf(sD1[r * H + h], sF[r * F + i], g);
-    } else if (p < OFF_W2) {
-      const int h = p - OFF_B1;
-      for (int r = 0; r < rows; ++r) g += sD1[r * H + h];
-    } else if (p < OFF_B2) {  // W2[h][q] = sum_s d2[s][h] h1[s][q]
-      const int h = (p - OFF_W2) / H, q = (p - OFF_W2) % H;
-      for (int r = 0; r < rows; ++r) g = fmaf(sD2[r * H + h], sH1[r * H + q], g);
-    } else if (p < OFF_W3) {
-      const int h = p - OFF_B2;
-      for (int r = 0; r < rows; ++r) g += sD2[r * H + h];
-    } else if (p < OFF_B3) {  // w3[h] = sum_s dy[s] h2[s][h]
-      const int h = p - OFF_W3;
-      for (int r = 0; r < rows; ++r) g = fmaf(sDy[r], sH2[r * H + h], g);
-    } else {
-      for (int r = 0; r < rows; ++r) g += sDy[r];
+  // every parameter's sum over the samples, in their order (the zeros of
+  // missing ones add nothing)
+  float* const out = part + (size_t)blockIdx.x * kPartLd;
+  auto at = [&](const float* v, int row, int r) { return *reinterpret_cast<const float4*>(v + row * kRowLd + r); };
+  {
+    const int h = 2 * (t >> 3), q = t & 7;  // rows h, h + 1 and columns q, q + 8, q + 16, q + 24 of W2
+    float g[2][4] = {};
+    for (int r = 0; r < kGradRows; r += 4) {
+      const float4 d0 = at(sD2, h, r), d1 = at(sD2, h + 1, r);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const float4 x = at(sH1, q + 8 * b, r);
+        g[0][b] = dot4(g[0][b], d0, x);
+        g[1][b] = dot4(g[1][b], d1, x);
+      }
     }
-    part[(size_t)blockIdx.x * kPartLd + p] = g;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) out[OFF_W2 + (h + a) * H + q + 8 * b] = g[a][b];
+  }
+  {
+    const int h = t >> 2, i = t & 3;  // columns i, i + 4 of row h of W1
+    float g0 = 0.0f, g1 = 0.0f;
+    for (int r = 0; r < kGradRows; r += 4) {
+      const float4 d = at(sD1, h, r);
+      g0 = dot4(g0, d, at(sF, i, r));
+      g1 = dot4(g1, d, at(sF, i + 4, r));
+    }
+    out[OFF_W1 + h * F + i] = g0;
+    out[OFF_W1 + h * F + i + 4] = g1;
+  }
+  if (t < 3 * H + 1) {  // the biases, w3 and b3
+    float g = 0.0f;
+    const int h = t & (H - 1);
+    if (t < 2 * H) {
+      const float* v = t < H ? sD1 : sD2;
+      for (int r = 0; r < kGradRows; r += 4) g = add4(g, at(v, h, r));
+      out[(t < H ? OFF_B1 : OFF_B2) + h] = g;
+    } else if (t < 3 * H) {
+      for (int r = 0; r < kGradRows; r += 4) g = dot4(g, at(sDy, 0, r), at(sH2, h, r));
+      out[OFF_W3 + h] = g;
+    } else {
+      for (int r = 0; r < kGradRows; r += 4) g = add4(g, at(sDy, 0, r));
+      out[OFF_B3] = g;
+    }
   }
   l2 = warp_sum(l2);
   __shared__ float red[kGradRows / 32];
@@ -426,18 +564,29 @@ diaf_status diaf_propose_features(const diaf_csc* A, const diaf_pattern* CAND, f
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint32_t* st = nullptr;
   if (cudaMallocAsync(&st, sizeof(uint32_t), s) != cudaSuccess) return DIAF_ENOMEM;
+  double2* dlog = nullptr;
+  if (cudaMallocAsync(&dlog, sizeof(double2) * n, s) != cudaSuccess) {
+    cudaFreeAsync(st, s);
+    return DIAF_ENOMEM;
+  }
   cudaMemsetAsync(st, 0, sizeof(uint32_t), s);
   const int blocks = ceil_div(n, kFeatWarps);
   if (A->dtype == DIAF_C128)
+    diag_log_kernel<Cx<double>><<<ceil_div(n, 256), 256, 0, s>>>(n, A->colptr, A->rowidx, (const Cx<double>*)A->vals, dlog);
+  else
+    diag_log_kernel<double><<<ceil_div(n, 256), 256, 0, s>>>(n, A->colptr, A->rowidx, (const double*)A->vals, dlog);
+  DIAF_COUNT_LAUNCH();
+  if (A->dtype == DIAF_C128)
     features_kernel<Cx<double>><<<blocks, kFeatWarps * 32, 0, s>>>(n, A->colptr, A->rowidx, (const Cx<double>*)A->vals,
-                                                                 CAND->colptr, CAND->rowidx, d_feat, st);
+                                                                 CAND->colptr, CAND->rowidx, dlog, d_feat, st);
   else
     features_kernel<double><<<blocks, kFeatWarps * 32, 0, s>>>(n, A->colptr, A->rowidx, (const double*)A->vals,
-                                                             CAND->colptr, CAND->rowidx, d_feat, st);
+                                                             CAND->colptr, CAND->rowidx, dlog, d_feat, st);
   DIAF_COUNT_LAUNCH();
   uint32_t h = 0;
   cudaMemcpyAsync(&h, st, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
   cudaFreeAsync(st, s);
+  cudaFreeAsync(dlog, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return DIAF_ECUDA;
   if (h & DEV_ST_BAD_INPUT) {
     diaf_set_last_error("a row index of A or CAND is out of range");
@@ -453,9 +602,9 @@ diaf_status diaf_propose_features(const diaf_csc* A, const diaf_pattern* CAND, f
 diaf_status diaf_mlp_forward(const float* d_params, const float* d_feat, int64_t nrows, float* d_out, void* stream) {
   if (nrows < 0 || (nrows > 0 && (!d_params || !d_feat || !d_out))) return DIAF_EINVAL;
   if (nrows == 0) return DIAF_OK;
-  int blocks = (int)((nrows + 255) / 256);
-  if (blocks > 4096) blocks = 4096;
-  mlp_forward_kernel<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(d_params, d_feat, nrows, d_out);
+  const int64_t per_block = (int64_t)kFwdThreads * kFwdRows;
+  int blocks = (int)std::min<int64_t>((nrows + per_block - 1) / per_block, 4096);
+  mlp_forward_kernel<<<blocks, kFwdThreads, 0, static_cast<cudaStream_t>(stream)>>>(d_params, d_feat, nrows, d_out);
   DIAF_COUNT_LAUNCH();
   return cudaGetLastError() == cudaSuccess ? DIAF_OK : DIAF_ECUDA;
 }
@@ -464,7 +613,7 @@ diaf_status diaf_mlp_grad(const float* d_params, const float* d_feat, const floa
                           float* d_grad, float* d_loss, void* stream) {
   if (nrows <= 0 || !d_params || !d_feat || !d_target || !d_grad || !d_loss) return DIAF_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const size_t smem = sizeof(float) * (NPARAM + kGradRows * (F + 4 * H + 1));
+  const size_t smem = sizeof(float) * kGradFloats;
   static bool configured = false;
   if (!configured) {
     if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
