@@ -1,10 +1,12 @@
 // Right-preconditioned BiCGSTAB (the evaluation solver of Sec. 5) with the
 // scalars kept on the device: one device-to-host read per iteration.
+#include <atomic>
 #include <string>
 #include <vector>
 
 #include "plan.cuh"
 #include "sparse.cuh"
+#include "warp_la.cuh"
 
 extern "C" diaf_status diaf_apply(diaf_factors* F, const void* x, void* y, void* stream);
 
@@ -297,22 +299,36 @@ struct GState {
   double hnext;                      // H(j+1, j) (read together with resid)
 };
 
-// part[i * nb + block] = partial sum of conj(V_i) w over the block's elements
+// part[i * nb + block] = partial sum of conj(V_i) w over the block's elements.
+// kDotBatch vectors at a time: their 32-lane sums go through one reduce-scatter
+// (the same pairs of lanes as a butterfly per vector, so the same rounding) and
+// eight lanes add the warps' parts of eight vectors side by side.  An FP64 add
+// takes a sub-core 64 cycles, and one vector after the other spent them on
+// butterflies and on one thread's sum (complex, n = 1,600, 25 vectors:
+// 65 -> 26 us).
+constexpr int kDotBatch = 8;
 template <class S>
 __global__ void k_mdot_partial(int n, const S* __restrict__ V, int cnt, const S* __restrict__ w, S* part) {
-  __shared__ S sh[kRedThreads / 32];
-  for (int i = 0; i < cnt; ++i) {
-    const S* vi = V + (size_t)i * n;
-    S acc = sc_zero<S>();
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x)
-      acc += sc_cmul(vi[e], w[e]);
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  static_assert(kRedThreads / 32 == kDotBatch, "eight warps");
+  __shared__ S sh[kDotBatch][kRedThreads / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i0 = 0; i0 < cnt; i0 += kDotBatch) {
+    S acc[kDotBatch];
+#pragma unroll
+    for (int u = 0; u < kDotBatch; ++u) acc[u] = sc_zero<S>();
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+      const S we = w[e];
+#pragma unroll
+      for (int u = 0; u < kDotBatch; ++u)
+        if (i0 + u < cnt) acc[u] += sc_cmul(V[(size_t)(i0 + u) * n + e], we);
+    }
+    const S tot = warp_reduce_scatter<S, kDotBatch>(acc, lane);  // lane 4u: vector u
+    if ((lane & 3) == 0) sh[lane >> 2][warp] = tot;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if ((int)threadIdx.x < kDotBatch && i0 + (int)threadIdx.x < cnt) {
       S t = sc_zero<S>();
-      for (int k = 0; k < kRedThreads / 32; ++k) t += sh[k];
-      part[(size_t)i * gridDim.x + blockIdx.x] = t;
+      for (int k = 0; k < kRedThreads / 32; ++k) t += sh[threadIdx.x][k];
+      part[(size_t)(i0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
     }
     __syncthreads();
   }
@@ -335,11 +351,18 @@ __global__ void k_mdot_final(const S* part, int nb, S* out, int accumulate) {
   }
 }
 
+// Elementwise work of many FP64 operations per element: blocks of two warps,
+// so that a vector spreads over the sub-cores of all SMs (64 cycles per FP64
+// instruction and sub-core).
+constexpr int kElemThreads = 64;
+static int elem_blocks(int n) { return n < 1 ? 1 : (n > 152 * 32 * kElemThreads ? 152 * 32 : ceil_div(n, kElemThreads)); }
+
 // w -= sum_i c[i] V_i
 template <class S>
 __global__ void k_mupdate(int n, const S* __restrict__ V, int cnt, const S* __restrict__ c, S* w) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
     S acc = sc_zero<S>();
+#pragma unroll 8
     for (int i = 0; i < cnt; ++i) acc += c[i] * V[(size_t)i * n + e];
     w[e] -= acc;
   }
@@ -350,6 +373,7 @@ template <class S>
 __global__ void k_combine(int n, const S* __restrict__ V, int cnt, const S* __restrict__ c, S* u) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
     S acc = sc_zero<S>();
+#pragma unroll 8
     for (int i = 0; i < cnt; ++i) acc += c[i] * V[(size_t)i * n + e];
     u[e] = acc;
   }
@@ -364,52 +388,81 @@ __global__ void k_normalize(int n, GState<S>* st, int j, const S* w, S* v) {
   if (blockIdx.x == 0 && threadIdx.x == 0) st->hnext = nrm;
 }
 
-// column j of H from h and hnext; old rotations, a new one, g updated
+// column j of H from h (plus the second Gram-Schmidt pass's part, in y) and
+// hnext; old rotations, a new one, g updated.  The rotations are one thread's
+// chain; what it reads is staged in shared memory by all (each step waited for
+// three reads of global memory before: 21 -> 15 us at 25 rotations).
 template <class S>
 __global__ void k_givens(GState<S>* st, int j) {
   constexpr int LD = kGmresMax + 1;
-  S* col = st->H + (size_t)j * LD;
-  for (int i = 0; i <= j; ++i) col[i] = st->h[i];
-  col[j + 1] = sc_real_s<S>(st->hnext);
-  for (int i = 0; i < j; ++i) {
-    const S a = col[i], b = col[i + 1];
-    col[i] = st->cs[i] * a + st->sn[i] * b;
-    col[i + 1] = st->cs[i] * b - sc_conj(st->sn[i]) * a;
+  __shared__ S col[kGmresMax + 1], sn[kGmresMax];
+  __shared__ double cs[kGmresMax];
+  const int t0 = threadIdx.x;
+  if (t0 <= j) {
+    const S h = st->h[t0] + st->y[t0];
+    st->h[t0] = h;
+    col[t0] = h;
   }
-  const S a = col[j];
-  const double bb = sc_real(col[j + 1]);  // a norm: real, >= 0
-  const double aa = sqrt((double)sc_abs2(a));
-  const double t = sqrt(aa * aa + bb * bb);
-  double c;
-  S sv;
-  if (t == 0.0) {
-    c = 1.0; sv = sc_zero<S>();
-  } else if (aa == 0.0) {
-    c = 0.0; sv = sc_real_s<S>(1.0);
-  } else {
-    c = aa / t;
-    sv = (bb / (aa * t)) * a;  // (a / |a|) (b / t)
+  if (t0 < j) {
+    cs[t0] = st->cs[t0];
+    sn[t0] = st->sn[t0];
   }
-  st->cs[j] = c;
-  st->sn[j] = sv;
-  col[j] = c * a + sv * col[j + 1];
-  col[j + 1] = sc_zero<S>();
-  const S gj = st->g[j];
-  st->g[j + 1] = -(sc_conj(sv) * gj);
-  st->g[j] = c * gj;
-  st->resid = sqrt((double)sc_abs2(st->g[j + 1]));
+  __syncthreads();
+  if (t0 == 0) {
+    col[j + 1] = sc_real_s<S>(st->hnext);
+    for (int i = 0; i < j; ++i) {
+      const S a = col[i], b = col[i + 1];
+      col[i] = cs[i] * a + sn[i] * b;
+      col[i + 1] = cs[i] * b - sc_conj(sn[i]) * a;
+    }
+    const S a = col[j];
+    const double bb = sc_real(col[j + 1]);  // a norm: real, >= 0
+    const double aa = sqrt((double)sc_abs2(a));
+    const double t = sqrt(aa * aa + bb * bb);
+    double c;
+    S sv;
+    if (t == 0.0) {
+      c = 1.0; sv = sc_zero<S>();
+    } else if (aa == 0.0) {
+      c = 0.0; sv = sc_real_s<S>(1.0);
+    } else {
+      c = aa / t;
+      sv = (bb / (aa * t)) * a;  // (a / |a|) (b / t)
+    }
+    st->cs[j] = c;
+    st->sn[j] = sv;
+    col[j] = c * a + sv * col[j + 1];
+    col[j + 1] = sc_zero<S>();
+    const S gj = st->g[j];
+    st->g[j + 1] = -(sc_conj(sv) * gj);
+    st->g[j] = c * gj;
+    st->resid = sqrt((double)sc_abs2(st->g[j + 1]));
+  }
+  __syncthreads();
+  if (t0 <= j + 1) st->H[(size_t)j * LD + t0] = col[t0];
 }
 
 // y = R^-1 g for the rotated k x k upper triangle; zero pivots give 0
+// (one chain; H, g and y staged in shared memory)
 template <class S>
 __global__ void k_backsolve(GState<S>* st, int k) {
   constexpr int LD = kGmresMax + 1;
-  for (int i = k - 1; i >= 0; --i) {
-    S acc = st->g[i];
-    for (int t = i + 1; t < k; ++t) acc -= st->H[i + (size_t)t * LD] * st->y[t];
-    const S d = st->H[i + (size_t)i * LD];
-    st->y[i] = sc_abs2(d) > 0.0 ? sdiv(acc, d) : sc_zero<S>();
-  }
+  extern __shared__ __align__(16) unsigned char bs_smem[];
+  S* Hs = reinterpret_cast<S*>(bs_smem);  // k x k, column-major
+  S* g = Hs + k * k;
+  S* y = g + k;
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) Hs[e] = st->H[(e % k) + (size_t)(e / k) * LD];
+  for (int e = threadIdx.x; e < k; e += blockDim.x) g[e] = st->g[e];
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int i = k - 1; i >= 0; --i) {
+      S acc = g[i];
+      for (int t = i + 1; t < k; ++t) acc -= Hs[i + t * k] * y[t];
+      const S d = Hs[i + i * k];
+      y[i] = sc_abs2(d) > 0.0 ? sdiv(acc, d) : sc_zero<S>();
+    }
+  __syncthreads();
+  for (int e = threadIdx.x; e < k; e += blockDim.x) st->y[e] = y[e];
 }
 
 // start of a cycle: g = (beta, 0, ...), v_0 = r / beta (beta from st->dot)
@@ -423,11 +476,6 @@ __global__ void k_cycle_start(int n, GState<S>* st, const S* r, S* v0) {
     st->g[0] = sc_real_s<S>(beta);
     st->resid = beta;
   }
-}
-
-template <class S>
-__global__ void k_add_small(int cnt, const S* a, S* h) {  // h += a (cnt <= blockDim)
-  if ((int)threadIdx.x < cnt) h[threadIdx.x] += a[threadIdx.x];
 }
 
 template <class S>
@@ -459,6 +507,16 @@ diaf_status gmres_t(diaf_solver* SV, diaf_factors* F, const S* b, S* xout, doubl
   };
   S *V, *w, *x, *r, *u, *z, *part;
   GState<S>* st;
+  // the back substitution stages up to m (m + 2) values (66 KB): beyond 48 KB by attribute, per device
+  static std::atomic<uint64_t> configured{0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return DIAF_ECUDA;
+  if (dev > 63 || !(configured.load() >> dev & 1)) {
+    if (cudaFuncSetAttribute(k_backsolve<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(sizeof(S) * kGmresMax * (kGmresMax + 2))) != cudaSuccess)
+      return DIAF_ECUDA;
+    if (dev <= 63) configured.fetch_or(1ull << dev);
+  }
   const size_t nv = sizeof(S) * (size_t)(n > 0 ? n : 1);
   if (!get((void**)&V, nv * (m + 1)) || !get((void**)&w, nv) || !get((void**)&x, nv) || !get((void**)&r, nv) ||
       !get((void**)&u, nv) || !get((void**)&z, nv) ||
@@ -511,20 +569,18 @@ diaf_status gmres_t(diaf_solver* SV, diaf_factors* F, const S* b, S* xout, doubl
       DIAF_COUNT_LAUNCH();
       k_mdot_final<S><<<j + 1, kRedThreads, 0, s>>>(part, kRedBlocks, st->h, 0);
       DIAF_COUNT_LAUNCH();
-      k_mupdate<S><<<vb, vt, 0, s>>>(n, V, j + 1, st->h, w);
+      k_mupdate<S><<<elem_blocks(n), kElemThreads, 0, s>>>(n, V, j + 1, st->h, w);
       DIAF_COUNT_LAUNCH();
       k_mdot_partial<S><<<kRedBlocks, kRedThreads, 0, s>>>(n, V, j + 1, w, part);
       DIAF_COUNT_LAUNCH();
       k_mdot_final<S><<<j + 1, kRedThreads, 0, s>>>(part, kRedBlocks, st->y, 0);  // y: scratch until the cycle ends
       DIAF_COUNT_LAUNCH();
-      k_mupdate<S><<<vb, vt, 0, s>>>(n, V, j + 1, st->y, w);
-      DIAF_COUNT_LAUNCH();
-      k_add_small<S><<<1, kGmresMax, 0, s>>>(j + 1, st->y, st->h);
+      k_mupdate<S><<<elem_blocks(n), kElemThreads, 0, s>>>(n, V, j + 1, st->y, w);
       DIAF_COUNT_LAUNCH();
       norm2_to_dot(w);
       k_normalize<S><<<vb, vt, 0, s>>>(n, st, j, w, V + (size_t)(j + 1) * n);
       DIAF_COUNT_LAUNCH();
-      k_givens<S><<<1, 1, 0, s>>>(st, j);
+      k_givens<S><<<1, kGmresMax + 1, 0, s>>>(st, j);
       DIAF_COUNT_LAUNCH();
       ++its;
       kdone = j + 1;
@@ -536,9 +592,9 @@ diaf_status gmres_t(diaf_solver* SV, diaf_factors* F, const S* b, S* xout, doubl
       if (rel <= tol || rh[1] == 0.0) { happy = rh[1] == 0.0; break; }
     }
     if (info->breakdown) break;
-    k_backsolve<S><<<1, 1, 0, s>>>(st, kdone);
+    k_backsolve<S><<<1, 256, sizeof(S) * (size_t)(kdone * kdone + 2 * kdone), s>>>(st, kdone);
     DIAF_COUNT_LAUNCH();
-    k_combine<S><<<vb, vt, 0, s>>>(n, V, kdone, st->y, u);
+    k_combine<S><<<elem_blocks(n), kElemThreads, 0, s>>>(n, V, kdone, st->y, u);
     DIAF_COUNT_LAUNCH();
     diaf_status ms = M(u, z);
     if (ms != DIAF_OK) return ms;
