@@ -239,11 +239,12 @@ __device__ inline int build_I(const ColArgs& a, int j, int m, int l, const Colum
 }
 
 // Phase (v_jj real >= 0, else the largest |w_q| real), residual
-// ||A_j w - v||, finiteness, and the scatter of column j.
+// ||A_j w - v|| (r2_known >= 0: its square, known to the caller), finiteness,
+// and the scatter of column j.
 template <class SD, int LDT>
 __device__ void finish_column(const ColArgs& a, int j, int k, int m, int l, int jpos, const SD* Ts, SD* wv, SD* vv,
                               const ColumnIdx& ix, uint32_t flags, bool do_phase, int lane,
-                              double rank_thr = -1.0) {
+                              double rank_thr = -1.0, double r2_known = -1.0) {
   using R = RealOf<SD>;
   if (do_phase) {
     SD ph = sc_real_s<SD>(R(1));
@@ -270,16 +271,19 @@ __device__ void finish_column(const ColArgs& a, int j, int k, int m, int l, int 
     for (int t = lane; t < l; t += DIAF_WARP) vv[t] = ph * vv[t];
     __syncwarp();
   }
-  R r2 = R(0);
-  for (int r = lane; r < m; r += DIAF_WARP) {
-    SD s = sc_zero<SD>();
-    for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
-    if (ix.inI[r] >= 0) s -= vv[ix.inI[r]];
-    r2 += sc_abs2(s);
+  R r2 = R(r2_known);
+  if (r2_known < 0.0) {
+    r2 = R(0);
+    for (int r = lane; r < m; r += DIAF_WARP) {
+      SD s = sc_zero<SD>();
+      for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
+      if (ix.inI[r] >= 0) s -= vv[ix.inI[r]];
+      r2 += sc_abs2(s);
+    }
+    for (int t = lane; t < l; t += DIAF_WARP)
+      if (ix.Iloc[t] < 0) r2 += sc_abs2(vv[t]);
+    r2 = warp_sum(r2);
   }
-  for (int t = lane; t < l; t += DIAF_WARP)
-    if (ix.Iloc[t] < 0) r2 += sc_abs2(vv[t]);
-  r2 = warp_sum(r2);
   const double resj = sqrt((double)r2);
   if (resj <= rank_thr) flags |= DIAF_FLAG_RANK_DEFICIENT;  // DIAF-S: res = ||A-hat w|| = sigma_min
   bool finite = isfinite(resj);
@@ -467,27 +471,24 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
     }
     __syncwarp();
   } else if (ALG == DIAF_ALG_S) {
-    // ---- DIAF-S: QR of the tile without the I_j rows, Jacobi SVD of R-hat
+    // ---- DIAF-S: the smallest singular vector of the tile without the I_j
+    // rows, directly, or by its QR and the Jacobi SVD of R-hat
+    S xw = sc_zero<S>();
+    bool direct = false;
+    uint32_t rowmask[MMAX / DIAF_WARP];
+    if constexpr (kSmallestFits<S, KMAX>) {
+      copy_tile<S, S, KMAX, MMAX, LDT>(Ts, ix.inI, Tw, m, k, lane, rowmask);
+      direct = warp_smallest_vector<S, S, KMAX, MMAX, LDT, KP>(Ts, ix.inI, Tw, rowmask, wv, vv, m, k, lane, &xw);
+    }
+    __syncwarp();
+    if (direct) {
+      if (lane < k) wv[lane] = xw;
+    } else {
     for (int i = lane; i < me * k; i += DIAF_WARP) {
       int r = i % me, c = i / me;
       Tw[r + c * LDT] = (r < m && ix.inI[r] >= 0) ? sc_zero<S>() : Ts[r + c * LDT];
     }
     __syncwarp();
-    S xw = sc_zero<S>();
-    bool direct = false;
-    if constexpr (kSmallestFits<S, KMAX>)
-      direct = warp_smallest_vector<S, S, KMAX, LDT, KP>(Ts, ix.inI, Tw, wv, vv, m, k, lane, &xw);
-    __syncwarp();
-    if (direct) {
-      if (lane < k) wv[lane] = xw;
-    } else {
-    if constexpr (kSmallestFits<S, KMAX>) {  // the attempt overwrote the working tile
-      for (int i = lane; i < me * k; i += DIAF_WARP) {
-        int r = i % me, c = i / me;
-        Tw[r + c * LDT] = (r < m && ix.inI[r] >= 0) ? sc_zero<S>() : Ts[r + c * LDT];
-      }
-      __syncwarp();
-    }
     warp_householder_qr_rs<S, LDT, KMAX, MMAX / DIAF_WARP>(Tw, me, k, lane);
     for (int i = lane; i < k * k; i += DIAF_WARP) {
       int r = i % k, c = i / k;

@@ -107,6 +107,61 @@ __device__ bool warp_gram_cholesky(const float* W, int m, int k, float* Rs, doub
   return true;
 }
 
+// FP32 leverage keys of the real m x k tile W (m >= k; leading dimension LDT;
+// rowmask: the columns that the lane's rows have) from its Gram matrix's
+// inverse: hk[r] = w_r^T (W^T W)^-1 w_r.  Ms: KP x KMAX scratch, buf: 2 KMAX,
+// 16-byte aligned.  False (uniformly) unless the column-scaled kappa is at
+// most kGramKappaMax; *kap2 receives its square.
+template <int KMAX, int MMAX, int LDT, int KP>
+__device__ bool warp_gram_keys(const float* W, const uint32_t (&rowmask)[MMAX / DIAF_WARP], float* Ms, float* buf,
+                               float* hk, int m, int k, int lane, float* kap2) {
+  float acc[KMAX];
+  {
+    uint32_t colmask[MMAX / DIAF_WARP];
+    tile_gram<float, KMAX, MMAX, LDT>(W, m, k, lane, acc, colmask);
+  }
+  float hqq = 0.0f;
+  if (lane < k) {
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p)
+      if (p < k) {
+        Ms[p + lane * KP] = acc[p];
+        if (p == lane) hqq = acc[p];
+      }
+  }
+  __syncwarp();
+  float piv = 1.0f, scale = 1.0f;
+  warp_sweep_inverse<float, KMAX, KP>(Ms, 0.0f, k, acc, buf, lane, &piv, &scale);
+  const float k2 = warp_max(lane < k ? (piv > 0.0f ? hqq / piv : INFINITY) : 0.0f);
+  if (!(k2 <= kGramKappaMax * kGramKappaMax)) return false;
+  *kap2 = k2;
+  if (lane < k) {
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i)
+      if (i >= KMAX - k) Ms[i - (KMAX - k) + lane * KP] = -scale * acc[i];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < MMAX / DIAF_WARP; ++u) {
+    const int r = lane + DIAF_WARP * u;
+    if (r >= m) continue;
+    float h = 0.0f;
+    for (uint32_t b = rowmask[u]; b; b &= b - 1) {
+      const int p = __ffs(b) - 1;
+      const float tp = W[r + p * LDT];
+      float y = 0.5f * Ms[p + p * KP] * tp;
+      for (uint32_t c = b & (b - 1); c; c &= c - 1) {
+        const int q = __ffs(c) - 1;
+        y = fmaf(Ms[q + p * KP], W[r + q * LDT], y);
+      }
+      h = fmaf(2.0f * tp, y, h);
+    }
+    hk[r] = h;
+  }
+  __syncwarp();
+  return true;
+}
+
 template <class S, int KMAX, int MMAX, int ALG>
 struct MixedLayout {
   using SD = typename DoubleOf<S>::T;
@@ -199,6 +254,30 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
   gather_tile<SD, KMAX, MMAX, LDT>(a, j, k, m, me, Ts, ix, lane);
   DIAF_PHASE(0);
 
+  // ---- the keys of wide real tiles from the inverse of T's Gram matrix: h_r =
+  // t_r^T (T^T T)^-1 t_r, all of it independent multiply-adds over a row's
+  // nonzeros, where the Householder QR is a chain of k reflectors with a
+  // reduce-scatter each (lognormal 64^3: QR and row solves 47 % of the cycles).
+  // The Gram matrix squares the conditioning, so the key bound carries
+  // kappa^2; what it cannot decide goes on to the QR, whose bound carries kappa.
+  bool keyed = false;
+  float kap = 0.0f;
+  if constexpr (!L::kRegQR && !ScalarInfo<S>::cplx && ALG == DIAF_ALG_S) {
+    if (m >= k) {
+      uint32_t rowmask[MMAX / DIAF_WARP];
+      copy_tile<S, SD, KMAX, MMAX, LDT>(Ts, nullptr, Tw, m, k, lane, rowmask);
+      DIAF_PHASE(1);
+      float kap2 = 0.0f;
+      if (warp_gram_keys<KMAX, MMAX, LDT, KP>(Tw, rowmask, Rs, reinterpret_cast<float*>(wv), hk, m, k, lane, &kap2)) {
+        keyed = a.rule == DIAF_RULE_FIXED;
+        if (!keyed) {
+          const double margin = select_rows_greedy(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
+          keyed = l <= 1 || margin > 2.0 * kMixedDeltaScale * (m + k) * (double)FLT_EPSILON * (double)kap2;
+        }
+      }
+    }
+  }
+  if (!keyed) {
   // ---- FP32 QR of T and the keys
   if constexpr (L::kRegQR) {
     // the tile in registers, one row per lane: R and the column norms directly
@@ -225,7 +304,6 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     __syncwarp();
   }
   DIAF_PHASE(2);
-  float kap = 0.0f;
   for (int c = lane; c < k; c += DIAF_WARP) {
     float d = (float)sc_abs(Rs[c + c * KP]);
     kap = fmaxf(kap, d > 0.0f ? (float)cn[c] / d : INFINITY);
@@ -266,8 +344,9 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
 #endif
     }
   }
+  }
   const int jpos = build_I(a, j, m, l, ix, lane);
-  double rank_thr = -1.0;
+  double rank_thr = -1.0, r2_known = -1.0;
   for (int t = lane; t < l; t += DIAF_WARP) vv[t] = sc_zero<SD>();
   __syncwarp();
   DIAF_PHASE(4);
@@ -276,12 +355,11 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     // ---- A-hat (I_j rows zeroed) in FP32, its smallest singular vector by
     // inverse iteration; the columns that form cannot take go on to the FP32
     // QR of A-hat and the Jacobi SVD of R-hat
-    for (int c = 0; c < k; ++c)
-      for (int r = lane; r < m; r += DIAF_WARP)
-        Tw[r + c * LDT] = ix.inI[r] >= 0 ? sc_zero<S>() : sc_cast<S>(Ts[r + c * LDT]);
-    __syncwarp();
+    uint32_t rowmask[MMAX / DIAF_WARP];
+    copy_tile<S, SD, KMAX, MMAX, LDT>(Ts, ix.inI, Tw, m, k, lane, rowmask);
     SD xw = sc_zero<SD>();
-    const bool direct = warp_smallest_vector<S, SD, KMAX, LDT, KP>(Ts, ix.inI, Tw, gg, zz, m, k, lane, &xw);
+    const bool direct =
+        warp_smallest_vector<S, SD, KMAX, MMAX, LDT, KP>(Ts, ix.inI, Tw, rowmask, gg, zz, m, k, lane, &xw);
 #ifdef DIAF_PHASE_TIMING
     if (lane == 0 && a.phase && !direct) atomicAdd(&a.phase[24 + 5], 1ull);
 #endif
@@ -289,6 +367,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     if (direct) {
       if (lane < k) wv[lane] = xw;
       __syncwarp();
+      r2_known = split_rows<SD, MMAX, LDT>(Ts, ix.inI, rowmask, wv, vv, m, lane);
       DIAF_PHASE(8);
     } else {
     // ---- FP32 QR of A-hat (I_j rows zeroed) into Rs; then the Jacobi SVD of R-hat
@@ -413,13 +492,14 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     rank_thr = 1e-14 * smax;  // tested on res = ||A-hat w|| in finish_column
     }
     // v = T(I_j,:) w and the rank test on the FP64 value of ||A-hat w||
-    for (int t = lane; t < l; t += DIAF_WARP) {
-      SD s = sc_zero<SD>();
-      int r = ix.Iloc[t];
-      if (r >= 0)
-        for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
-      vv[t] = s;
-    }
+    if (!direct)
+      for (int t = lane; t < l; t += DIAF_WARP) {
+        SD s = sc_zero<SD>();
+        int r = ix.Iloc[t];
+        if (r >= 0)
+          for (int q = 0; q < k; ++q) s = sc_madd(s, Ts[r + q * LDT], wv[q]);
+        vv[t] = s;
+      }
     __syncwarp();
   } else {
     // ---- eigenpairs of C = Q_I Q_I^* by an FP32 one-sided Jacobi (the rows of
@@ -590,7 +670,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     }
   }
   DIAF_PHASE(9);
-  finish_column<SD, LDT>(a, j, k, m, l, jpos, Ts, wv, vv, ix, flags, true, lane, rank_thr);
+  finish_column<SD, LDT>(a, j, k, m, l, jpos, Ts, wv, vv, ix, flags, true, lane, rank_thr, r2_known);
   DIAF_PHASE(10);
 }
 

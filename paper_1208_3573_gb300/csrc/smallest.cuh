@@ -49,8 +49,8 @@ constexpr bool kSmallestFits = !(ScalarInfo<S>::cplx && sizeof(S) == 16);
 constexpr int kInverseItMax = 16;
 constexpr int kCorrectMax = 8;
 
-// The tile product (T^* z)_c of lane c (defined with the mixed kernel's other
-// tile helpers below): rows split between the half-warps for up to 16 columns.
+// (T^* z)_c of lane c in FP64 over the m tile rows; tiles of up to 16 columns
+// split the rows between the half-warps.
 template <class SD, int LDT, int KMAX>
 __device__ __forceinline__ SD tile_adj_mul(const SD* Ts, const SD* zz, int m, int k, int lane) {
   SD g = sc_zero<SD>();
@@ -64,6 +64,70 @@ __device__ __forceinline__ SD tile_adj_mul(const SD* Ts, const SD* zz, int m, in
       for (int r = 0; r < m; ++r) g = sc_cmadd(g, Ts[r + lane * LDT], zz[r]);
   }
   return g;
+}
+
+// Copies the tile to the working type (rows in I_j as zeros when inI is given)
+// and notes which columns each of the lane's rows (lane + 32u) has, all of
+// them, I_j's too.
+template <class S, class SD, int KMAX, int MMAX, int LDT>
+__device__ __forceinline__ void copy_tile(const SD* Ts, const int32_t* inI, S* Tw, int m, int k, int lane,
+                                          uint32_t (&rowmask)[MMAX / DIAF_WARP]) {
+#pragma unroll
+  for (int u = 0; u < MMAX / DIAF_WARP; ++u) {
+    rowmask[u] = 0;
+    const int r = lane + DIAF_WARP * u;
+    if (r < m) {
+      const bool out = inI && inI[r] >= 0;
+      for (int c = 0; c < k; ++c) {
+        const S v = sc_cast<S>(Ts[r + c * LDT]);
+        if (sc_real(v) != RealOf<S>(0) || sc_imag(v) != RealOf<S>(0)) rowmask[u] |= 1u << c;
+        Tw[r + c * LDT] = out ? sc_zero<S>() : v;
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// Column `lane` of W^* W in acc (two lanes per column, alternate rows, for up
+// to 16 columns; both end with the whole) and the rows of the lane's share
+// with a nonzero in that column.
+template <class S, int KMAX, int MMAX, int LDT>
+__device__ __forceinline__ void tile_gram(const S* W, int m, int k, int lane, S (&acc)[KMAX],
+                                          uint32_t (&colmask)[MMAX / DIAF_WARP]) {
+  constexpr bool kHalf = KMAX <= 16;
+#pragma unroll
+  for (int p = 0; p < KMAX; ++p) acc[p] = sc_zero<S>();
+#pragma unroll
+  for (int u = 0; u < MMAX / DIAF_WARP; ++u) colmask[u] = 0;
+  const int q = kHalf ? lane & 15 : lane;
+  if (q < k) {
+    const S* wq = W + q * LDT;
+#pragma unroll
+    for (int u = 0; u < MMAX / DIAF_WARP; ++u)
+      for (int r = DIAF_WARP * u + (kHalf ? lane >> 4 : 0); r < m && r < DIAF_WARP * (u + 1); r += kHalf ? 2 : 1) {
+        const S x = wq[r];
+        if (sc_real(x) != RealOf<S>(0) || sc_imag(x) != RealOf<S>(0)) colmask[u] |= 1u << (r & 31);
+#pragma unroll
+        for (int p = 0; p < KMAX; ++p)
+          if (p < k) acc[p] = sc_cmadd(acc[p], W[r + p * LDT], x);
+      }
+  }
+  if constexpr (kHalf) {
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p) acc[p] += shfl_xor(acc[p], 16);
+  }
+}
+
+// Warp-wide sums of two values at once: the halves of the warp take one each
+// after the first step (five FP64 additions instead of ten).
+template <class T>
+__device__ __forceinline__ void warp_sum2(T& a, T& b, int lane) {
+  const bool up = lane >= 16;
+  T v = up ? b : a;
+  v += shfl_xor(up ? a : b, 16);
+  v = group_sum<16>(v);
+  a = shfl_idx(v, 0);
+  b = shfl_idx(v, 16);
 }
 
 // Inverse of H - shift I for the Hermitian k x k matrix Hs (leading dimension
@@ -147,36 +211,22 @@ __device__ __forceinline__ S warp_inverse_mul(const S (&a)[KMAX], RealOf<S> scal
 }
 
 // Ts: the tile (type SD, leading dimension LDT), Tw: a copy of it in the
-// working type with the I_j rows zeroed (overwritten), inI: its rows in I_j
-// (>= 0), gg / zz: KMAX / m scratch in SD.  On success
-// returns true and lane q < k has entry q of the unit vector in *x_out.
-template <class S, class SD, int KMAX, int LDT, int KP>
-__device__ bool warp_smallest_vector(const SD* Ts, const int32_t* inI, S* Tw, SD* gg, SD* zz, int m, int k,
+// working type with the I_j rows zeroed (overwritten), rowmask: the columns
+// that the lane's rows have (copy_tile), inI: the rows in I_j (>= 0), gg / zz:
+// KMAX / m scratch in SD.  The FP64 products run over the tile's nonzeros only
+// (stencil tiles are 10 to 40 % full, and an FP64 instruction holds a sub-core
+// for 64 cycles).  On success returns true and lane q < k has entry q of the
+// unit vector in *x_out.
+template <class S, class SD, int KMAX, int MMAX, int LDT, int KP>
+__device__ bool warp_smallest_vector(const SD* Ts, const int32_t* inI, S* Tw,
+                                     const uint32_t (&rowmask)[MMAX / DIAF_WARP], SD* gg, SD* zz, int m, int k,
                                      int lane, SD* x_out) {
   using R = RealOf<S>;
   static_assert(KP + 3 <= LDT && (KP * KMAX * sizeof(S)) % 16 == 0, "H, the pivot columns and x fit the tile");
   if (k < 2 || m < k) return false;
-  // ---- H: lane q forms column q (two lanes per column, alternate rows, for up to 16 columns)
   S acc[KMAX];
-#pragma unroll
-  for (int p = 0; p < KMAX; ++p) acc[p] = sc_zero<S>();
-  {
-    constexpr bool kHalf = KMAX <= 16;
-    const int q = kHalf ? lane & 15 : lane;
-    if (q < k) {
-      const S* wq = Tw + q * LDT;
-      for (int r = kHalf ? lane >> 4 : 0; r < m; r += kHalf ? 2 : 1) {
-        const S x = wq[r];
-#pragma unroll
-        for (int p = 0; p < KMAX; ++p)
-          if (p < k) acc[p] = sc_cmadd(acc[p], Tw[r + p * LDT], x);
-      }
-    }
-    if constexpr (kHalf) {
-#pragma unroll
-      for (int p = 0; p < KMAX; ++p) acc[p] += shfl_xor(acc[p], 16);
-    }
-  }
+  uint32_t colmask[MMAX / DIAF_WARP];
+  tile_gram<S, KMAX, MMAX, LDT>(Tw, m, k, lane, acc, colmask);
   __syncwarp();  // the tile has been read
   S* Hs = Tw;
   S* buf = Hs + KP * KMAX;
@@ -259,37 +309,83 @@ __device__ bool warp_smallest_vector(const SD* Ts, const int32_t* inI, S* Tw, SD
   // ---- corrections against the FP64 tile
   using RD = RealOf<SD>;
   SD y = lane < k ? sc_cast<SD>(x) : sc_zero<SD>();
-  double before = (double)last;
+  float before = (float)last;
   bool done = false;
 #pragma unroll 1
   for (int it = 0; it < kCorrectMax && !done; ++it) {
     if (lane < k) gg[lane] = y;
     __syncwarp();
-    for (int r = lane; r < m; r += DIAF_WARP) {
-      SD z = sc_zero<SD>();
-      if (inI[r] < 0)
-        for (int q = 0; q < k; ++q) z = sc_madd(z, Ts[r + q * LDT], gg[q]);
-      zz[r] = z;
+#pragma unroll
+    for (int u = 0; u < MMAX / DIAF_WARP; ++u) {
+      const int r = lane + DIAF_WARP * u;
+      if (r < m) {
+        SD z = sc_zero<SD>();
+        for (uint32_t b = inI[r] < 0 ? rowmask[u] : 0u; b; b &= b - 1) {
+          const int q = __ffs(b) - 1;
+          z = sc_madd(z, Ts[r + q * LDT], gg[q]);
+        }
+        zz[r] = z;
+      }
     }
     __syncwarp();
-    const SD g = tile_adj_mul<SD, LDT, KMAX>(Ts, zz, m, k, lane);
-    const RD yg = warp_sum(lane < k ? (RD)sc_real(sc_cmul(y, g)) : RD(0));
-    const RD yy = warp_sum(lane < k ? (RD)sc_abs2(y) : RD(0));
-    const RD dd = yg / yy;
-    const double room = (double)s - (double)dd;  // at most the gap to the next eigenvalue
-    if (!(room >= 1.05e-5 * (double)hinf && (double)dd > 1e-24 * (double)hinf)) return false;
+    SD g = sc_zero<SD>();
+    {
+      const int q = KMAX <= 16 ? lane & 15 : lane;
+#pragma unroll
+      for (int u = 0; u < MMAX / DIAF_WARP; ++u)
+        for (uint32_t b = colmask[u]; b; b &= b - 1) {
+          const int r = DIAF_WARP * u + __ffs(b) - 1;
+          g = sc_cmadd(g, Ts[r + q * LDT], zz[r]);
+        }
+      if constexpr (KMAX <= 16) g += shfl_xor(g, 16);
+    }
+    RD yg = lane < k ? (RD)sc_real(sc_cmul(y, g)) : RD(0);
+    RD yy = lane < k ? (RD)sc_abs2(y) : RD(0);
+    warp_sum2(yg, yy, lane);
+    RD iy = RD(2) - yy;  // 1 / yy, yy close to 1: Newton steps from 1
+    iy *= fma(-yy, iy, RD(2));
+    iy *= fma(-yy, iy, RD(2));
+    const RD dd = yg * iy;
+    const float room = (float)((RD)s - dd), ddf = (float)dd;  // room: at most the gap to the next eigenvalue
+    if (!(room >= 1.05e-5f * (float)hinf && ddf > 1e-24f * (float)hinf)) return false;
     const S r = lane < k ? sc_cast<S>(g - dd * y) : sc_zero<S>();
     const S dx = correction(r, R(room));
-    const double step = sqrt((double)warp_sum(lane < k ? sc_abs2(dx) : R(0)));
+    const float step = sqrtf((float)warp_sum(lane < k ? sc_abs2(dx) : R(0)));
     if (lane < k) y += sc_cast<SD>(dx);
     // the next correction would be about step * (step / before)
-    done = step * step <= 1e-14 * before;
-    if (!done && it > 0 && !(step <= 0.5 * before)) return false;
+    done = step * step <= 1e-14f * before;
+    if (!done && it > 0 && !(step <= 0.5f * before)) return false;
     before = step;
     __syncwarp();
   }
   if (!done) return false;
   const RD n2 = warp_sum(lane < k ? (RD)sc_abs2(y) : RD(0));
-  *x_out = RD(1.0 / sqrt((double)n2)) * y;
+  RD inv2 = fma(RD(-0.5), n2, RD(1.5));  // 1 / sqrt(n2), n2 close to 1: Newton steps from 1
+  inv2 *= fma(RD(-0.5) * n2 * inv2, inv2, RD(1.5));
+  inv2 *= fma(RD(-0.5) * n2 * inv2, inv2, RD(1.5));
+  *x_out = inv2 * y;
   return true;
+}
+
+// T w for the rows of the tile (w in wv) over its nonzeros: the rows in I_j to
+// their places in vv, the sum of squares of the others (||A_j w - v||^2, as v
+// takes the rows in I_j) returned.
+template <class SD, int MMAX, int LDT>
+__device__ __forceinline__ double split_rows(const SD* Ts, const int32_t* inI,
+                                             const uint32_t (&rowmask)[MMAX / DIAF_WARP], const SD* wv, SD* vv, int m,
+                                             int lane) {
+  RealOf<SD> r2 = RealOf<SD>(0);
+#pragma unroll
+  for (int u = 0; u < MMAX / DIAF_WARP; ++u) {
+    const int r = lane + DIAF_WARP * u;
+    if (r >= m) continue;
+    SD t = sc_zero<SD>();
+    for (uint32_t b = rowmask[u]; b; b &= b - 1) {
+      const int q = __ffs(b) - 1;
+      t = sc_madd(t, Ts[r + q * LDT], wv[q]);
+    }
+    if (inI[r] >= 0) vv[inI[r]] = t;
+    else r2 += sc_abs2(t);
+  }
+  return (double)warp_sum(r2);
 }
