@@ -154,37 +154,60 @@ __device__ void gather_tile(const ColArgs& a, int j, int k, int m, int me, SD* T
 // came to flipping when the keys carry an error.
 // K: the key type (double in the FP64 kernels; float in the mixed ones, whose
 // keys are FP32 values and are compared as such).
-template <class K>
+// A lane holds its rows' keys (NR of them, r = lane + 32u) and admissibility in
+// registers, so a pick is one warp maximum and a few ballots; the picks go to
+// pick[] at the end.
+template <int NR, class K>
 __device__ inline double select_rows_greedy(const int32_t* rs, const K* hk, int32_t* pick, int m, int rule,
                                             int j, int s, double tau, int lane, const int32_t* blk) {
   K margin = std::numeric_limits<K>::max();
-  for (int r = lane; r < m; r += DIAF_WARP) pick[r] = 0;
-  __syncwarp();
+  K h[NR];
+  bool cand[NR], picked[NR];
+#pragma unroll
+  for (int u = 0; u < NR; ++u) {
+    const int r = lane + DIAF_WARP * u;
+    h[u] = r < m ? hk[r] : K(0);
+    cand[u] = r < m && admissible_row(rule, rs[r], j, blk);
+    picked[u] = false;
+  }
+  auto lowest = [&](const bool(&f)[NR]) {  // the lowest row with f
+    int row = INT_MAX;
+#pragma unroll
+    for (int u = NR - 1; u >= 0; --u) {
+      const unsigned b = __ballot_sync(DIAF_FULL, f[u]);
+      if (b) row = DIAF_WARP * u + __ffs(b) - 1;
+    }
+    return row;
+  };
   for (int t = 0; t < s; ++t) {
     K hm = -std::numeric_limits<K>::max();
-    for (int r = lane; r < m; r += DIAF_WARP)
-      if (!pick[r] && admissible_row(rule, rs[r], j, blk)) hm = dmax(hm, hk[r]);
+#pragma unroll
+    for (int u = 0; u < NR; ++u)
+      if (cand[u]) hm = dmax(hm, h[u]);
     hm = warp_max(hm);
-    int rmax = INT_MAX;
-    for (int r = lane; r < m; r += DIAF_WARP)
-      if (!pick[r] && admissible_row(rule, rs[r], j, blk) && hk[r] == hm) rmax = dmin(rmax, r);
-    rmax = warp_min(rmax);
+    bool f[NR];
+#pragma unroll
+    for (int u = 0; u < NR; ++u) f[u] = cand[u] && h[u] == hm;
+    const int rmax = lowest(f);
     const K thr = hm - K(tau);
-    int best = INT_MAX;
-    for (int r = lane; r < m; r += DIAF_WARP)
-      if (!pick[r] && admissible_row(rule, rs[r], j, blk)) {
-        if (r != rmax) margin = dmin(margin, (K)fabs(hk[r] - thr));
-        if (hk[r] >= thr) best = dmin(best, r);
-      }
-    best = warp_min(best);
-    if (best == INT_MAX) {  // no key reaches the threshold (non-finite keys): the lowest remaining admissible row
-      for (int r = lane; r < m; r += DIAF_WARP)
-        if (!pick[r] && admissible_row(rule, rs[r], j, blk)) best = dmin(best, r);
-      best = warp_min(best);
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+      if (cand[u] && lane + DIAF_WARP * u != rmax) margin = dmin(margin, (K)fabs(h[u] - thr));
+      f[u] = cand[u] && h[u] >= thr;
     }
-    if (lane == 0 && best < m) pick[best] = 1;
-    __syncwarp();
+    int best = lowest(f);
+    if (best == INT_MAX) best = lowest(cand);  // no key reaches the threshold (non-finite keys)
+#pragma unroll
+    for (int u = 0; u < NR; ++u)
+      if (lane + DIAF_WARP * u == best) {
+        cand[u] = false;
+        picked[u] = true;
+      }
   }
+#pragma unroll
+  for (int u = 0; u < NR; ++u)
+    if (lane + DIAF_WARP * u < m) pick[lane + DIAF_WARP * u] = picked[u] ? 1 : 0;
+  __syncwarp();
   return (double)warp_min(margin);
 }
 
@@ -454,7 +477,7 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
   const R piv = R(1e-14) * rdmax;
   if (k > 0 && (a.rule != DIAF_RULE_FIXED || ALG == DIAF_ALG_Q))
     warp_leverage_rows<S, S, LDT, KP>(Ts, Rs, Tw, hk, rinv, m, k, piv, lane);
-  if (a.rule != DIAF_RULE_FIXED) select_rows_greedy(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
+  if (a.rule != DIAF_RULE_FIXED) select_rows_greedy<MMAX / DIAF_WARP>(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
   const int jpos = build_I(a, j, m, l, ix, lane);
 
   for (int t = lane; t < l; t += DIAF_WARP) vv[t] = sc_zero<S>();
@@ -478,7 +501,7 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
     uint32_t rowmask[MMAX / DIAF_WARP];
     if constexpr (kSmallestFits<S, KMAX>) {
       copy_tile<S, S, KMAX, MMAX, LDT>(Ts, ix.inI, Tw, m, k, lane, rowmask);
-      direct = warp_smallest_vector<S, S, KMAX, MMAX, LDT, KP>(Ts, ix.inI, Tw, rowmask, wv, vv, m, k, lane, &xw);
+      direct = warp_smallest_vector<S, S, KMAX, MMAX, LDT, KP>(Ts, ix.inI, Tw, rowmask, Rs, wv, vv, m, k, lane, &xw);
     }
     __syncwarp();
     if (direct) {

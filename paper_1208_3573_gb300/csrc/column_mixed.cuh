@@ -116,20 +116,9 @@ template <int KMAX, int MMAX, int LDT, int KP>
 __device__ bool warp_gram_keys(const float* W, const uint32_t (&rowmask)[MMAX / DIAF_WARP], float* Ms, float* buf,
                                float* hk, int m, int k, int lane, float* kap2) {
   float acc[KMAX];
-  {
-    uint32_t colmask[MMAX / DIAF_WARP];
-    tile_gram<float, KMAX, MMAX, LDT>(W, m, k, lane, acc, colmask);
-  }
-  float hqq = 0.0f;
-  if (lane < k) {
-#pragma unroll
-    for (int p = 0; p < KMAX; ++p)
-      if (p < k) {
-        Ms[p + lane * KP] = acc[p];
-        if (p == lane) hqq = acc[p];
-      }
-  }
-  __syncwarp();
+  uint32_t colmask[MMAX / DIAF_WARP];
+  tile_gram<float, KMAX, MMAX, LDT, KP>(W, rowmask, Ms, m, k, lane, colmask);
+  const float hqq = lane < k ? Ms[lane + lane * KP] : 0.0f;
   float piv = 1.0f, scale = 1.0f;
   warp_sweep_inverse<float, KMAX, KP>(Ms, 0.0f, k, acc, buf, lane, &piv, &scale);
   const float k2 = warp_max(lane < k ? (piv > 0.0f ? hqq / piv : INFINITY) : 0.0f);
@@ -271,7 +260,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
       if (warp_gram_keys<KMAX, MMAX, LDT, KP>(Tw, rowmask, Rs, reinterpret_cast<float*>(wv), hk, m, k, lane, &kap2)) {
         keyed = a.rule == DIAF_RULE_FIXED;
         if (!keyed) {
-          const double margin = select_rows_greedy(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
+          const double margin = select_rows_greedy<MMAX / DIAF_WARP>(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
           keyed = l <= 1 || margin > 2.0 * kMixedDeltaScale * (m + k) * (double)FLT_EPSILON * (double)kap2;
         }
       }
@@ -313,7 +302,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
   warp_leverage_rows<S, SD, LDT, KP>(Ts, Rs, Tw, hk, rinv, m, k, R(0), lane);
   DIAF_PHASE(3);
   if (a.rule != DIAF_RULE_FIXED) {
-    const double margin = select_rows_greedy(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
+    const double margin = select_rows_greedy<MMAX / DIAF_WARP>(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
     // bound on the FP32 key error: backward error of the FP32 QR and of the
     // row solves, amplified by the (column-scaled) conditioning of T
     const double delta = kMixedDeltaScale * (m + k) * (double)FLT_EPSILON * (double)kap;
@@ -338,7 +327,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
       for (int c = lane; c < k; c += DIAF_WARP) rdmax = dmax(rdmax, sc_abs(Rq[c + c * KP]));
       rdmax = warp_max(rdmax);
       warp_leverage_rows<SD, SD, LDT, KP>(Ts, Rq, Tq, hd, rinvD, m, k, RealOf<SD>(1e-14) * rdmax, lane);
-      select_rows_greedy(ix.rs, hd, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
+      select_rows_greedy<MMAX / DIAF_WARP>(ix.rs, hd, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
 #ifdef DIAF_PHASE_TIMING
       if (lane == 0 && a.phase) atomicAdd(&a.phase[24 + 2], 1ull);
 #endif
@@ -359,7 +348,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     copy_tile<S, SD, KMAX, MMAX, LDT>(Ts, ix.inI, Tw, m, k, lane, rowmask);
     SD xw = sc_zero<SD>();
     const bool direct =
-        warp_smallest_vector<S, SD, KMAX, MMAX, LDT, KP>(Ts, ix.inI, Tw, rowmask, gg, zz, m, k, lane, &xw);
+        warp_smallest_vector<S, SD, KMAX, MMAX, LDT, KP>(Ts, ix.inI, Tw, rowmask, Rs, gg, zz, m, k, lane, &xw);
 #ifdef DIAF_PHASE_TIMING
     if (lane == 0 && a.phase && !direct) atomicAdd(&a.phase[24 + 5], 1ull);
 #endif

@@ -88,34 +88,87 @@ __device__ __forceinline__ void copy_tile(const SD* Ts, const int32_t* inI, S* T
   __syncwarp();
 }
 
-// Column `lane` of W^* W in acc (two lanes per column, alternate rows, for up
-// to 16 columns; both end with the whole) and the rows of the lane's share
-// with a nonzero in that column.
-template <class S, int KMAX, int MMAX, int LDT>
-__device__ __forceinline__ void tile_gram(const S* W, int m, int k, int lane, S (&acc)[KMAX],
-                                          uint32_t (&colmask)[MMAX / DIAF_WARP]) {
+// H = W^* W (k x k, leading dimension KP; W's leading dimension LDT) and the
+// rows with a nonzero in column `lane` (up to 16 columns: in column lane mod 16,
+// the rows of the lane's half).  rowmask: a superset of the columns that the
+// lane's rows have.  Tiles of up to 16 columns: a lane forms a column in
+// registers, the half-warps alternate rows.  Wider ones, where the rows are
+// short (a stencil's 7 of 25): lane q goes over its column's rows and each
+// row's columns only, adding into its own column of H; m k steps per lane
+// otherwise.
+template <class S, int KMAX, int MMAX, int LDT, int KP>
+__device__ __forceinline__ void tile_gram(const S* W, const uint32_t (&rowmask)[MMAX / DIAF_WARP], S* H, int m, int k,
+                                          int lane, uint32_t (&colmask)[MMAX / DIAF_WARP]) {
   constexpr bool kHalf = KMAX <= 16;
+  constexpr int NR = MMAX / DIAF_WARP;
+  const int q = kHalf ? lane & 15 : lane;
+  const bool own = q < k;
+  if constexpr (!kHalf) {
+    int steps = 0;
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+      colmask[u] = 0;
+      for (int r = DIAF_WARP * u; r < m && r < DIAF_WARP * (u + 1); ++r) {  // row r's columns to their lanes
+        const uint32_t b = __shfl_sync(DIAF_FULL, rowmask[u], r & 31);
+        const bool has = own && (b >> lane & 1u) &&
+                         (sc_real(W[r + q * LDT]) != RealOf<S>(0) || sc_imag(W[r + q * LDT]) != RealOf<S>(0));
+        if (has) {
+          colmask[u] |= 1u << (r & 31);
+          steps += __popc(b);
+        }
+      }
+    }
+    if (__reduce_max_sync(DIAF_FULL, steps) * 10 < m * (k + 20)) {
+      if (own)
+        for (int p = 0; p < k; ++p) H[p + q * KP] = sc_zero<S>();
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        uint32_t c = colmask[u];
+        while (__any_sync(DIAF_FULL, c != 0)) {  // whole warp: the row masks come by shuffle
+          const int r5 = c ? __ffs(c) - 1 : 0;
+          uint32_t b = __shfl_sync(DIAF_FULL, rowmask[u], r5);
+          if (c == 0) b = 0;
+          const int r = DIAF_WARP * u + r5;
+          const S x = b ? W[r + q * LDT] : sc_zero<S>();
+          for (; b; b &= b - 1) {
+            const int p = __ffs(b) - 1;
+            H[p + q * KP] = sc_cmadd(H[p + q * KP], W[r + p * LDT], x);
+          }
+          c &= c - 1;
+        }
+      }
+      __syncwarp();
+      return;
+    }
+  }
+  S acc[KMAX];
 #pragma unroll
   for (int p = 0; p < KMAX; ++p) acc[p] = sc_zero<S>();
+  if constexpr (kHalf) {
 #pragma unroll
-  for (int u = 0; u < MMAX / DIAF_WARP; ++u) colmask[u] = 0;
-  const int q = kHalf ? lane & 15 : lane;
-  if (q < k) {
+    for (int u = 0; u < NR; ++u) colmask[u] = 0;
+  }
+  if (own) {
     const S* wq = W + q * LDT;
+    for (int r = kHalf ? lane >> 4 : 0; r < m; r += kHalf ? 2 : 1) {
+      const S x = wq[r];
+      if constexpr (kHalf)
+        if (sc_real(x) != RealOf<S>(0) || sc_imag(x) != RealOf<S>(0)) colmask[r >> 5] |= 1u << (r & 31);
 #pragma unroll
-    for (int u = 0; u < MMAX / DIAF_WARP; ++u)
-      for (int r = DIAF_WARP * u + (kHalf ? lane >> 4 : 0); r < m && r < DIAF_WARP * (u + 1); r += kHalf ? 2 : 1) {
-        const S x = wq[r];
-        if (sc_real(x) != RealOf<S>(0) || sc_imag(x) != RealOf<S>(0)) colmask[u] |= 1u << (r & 31);
-#pragma unroll
-        for (int p = 0; p < KMAX; ++p)
-          if (p < k) acc[p] = sc_cmadd(acc[p], W[r + p * LDT], x);
-      }
+      for (int p = 0; p < KMAX; ++p)
+        if (p < k) acc[p] = sc_cmadd(acc[p], W[r + p * LDT], x);
+    }
   }
   if constexpr (kHalf) {
 #pragma unroll
     for (int p = 0; p < KMAX; ++p) acc[p] += shfl_xor(acc[p], 16);
   }
+  if (lane < k) {
+#pragma unroll
+    for (int p = 0; p < KMAX; ++p)
+      if (p < k) H[p + lane * KP] = acc[p];
+  }
+  __syncwarp();
 }
 
 // Warp-wide sums of two values at once: the halves of the warp take one each
@@ -212,37 +265,28 @@ __device__ __forceinline__ S warp_inverse_mul(const S (&a)[KMAX], RealOf<S> scal
 
 // Ts: the tile (type SD, leading dimension LDT), Tw: a copy of it in the
 // working type with the I_j rows zeroed (overwritten), rowmask: the columns
-// that the lane's rows have (copy_tile), inI: the rows in I_j (>= 0), gg / zz:
-// KMAX / m scratch in SD.  The FP64 products run over the tile's nonzeros only
+// that the lane's rows have (copy_tile), inI: the rows in I_j (>= 0), Hs: KP x
+// KMAX scratch, gg / zz: KMAX / m scratch in SD.  The FP64 products run over the tile's nonzeros only
 // (stencil tiles are 10 to 40 % full, and an FP64 instruction holds a sub-core
 // for 64 cycles).  On success returns true and lane q < k has entry q of the
 // unit vector in *x_out.
 template <class S, class SD, int KMAX, int MMAX, int LDT, int KP>
 __device__ bool warp_smallest_vector(const SD* Ts, const int32_t* inI, S* Tw,
-                                     const uint32_t (&rowmask)[MMAX / DIAF_WARP], SD* gg, SD* zz, int m, int k,
+                                     const uint32_t (&rowmask)[MMAX / DIAF_WARP], S* Hs, SD* gg, SD* zz, int m, int k,
                                      int lane, SD* x_out) {
   using R = RealOf<S>;
-  static_assert(KP + 3 <= LDT && (KP * KMAX * sizeof(S)) % 16 == 0, "H, the pivot columns and x fit the tile");
+  static_assert(3 <= LDT, "the pivot columns and x fit the tile");
   if (k < 2 || m < k) return false;
-  S acc[KMAX];
   uint32_t colmask[MMAX / DIAF_WARP];
-  tile_gram<S, KMAX, MMAX, LDT>(Tw, m, k, lane, acc, colmask);
-  __syncwarp();  // the tile has been read
-  S* Hs = Tw;
-  S* buf = Hs + KP * KMAX;
+  tile_gram<S, KMAX, MMAX, LDT, KP>(Tw, rowmask, Hs, m, k, lane, colmask);
+  S* buf = Tw;  // the tile has been read
   S* xs = buf + 2 * KMAX;
   R hrow = R(0), hqq = R(0);
   if (lane < k) {
-#pragma unroll
-    for (int p = 0; p < KMAX; ++p)
-      if (p < k) {
-        Hs[p + lane * KP] = acc[p];
-        hrow += fabs(sc_real(acc[p])) + fabs(sc_imag(acc[p]));
-        if (p == lane) hqq = sc_real(acc[p]);
-      }
+    for (int p = 0; p < k; ++p) hrow += fabs(sc_real(Hs[p + lane * KP])) + fabs(sc_imag(Hs[p + lane * KP]));
+    hqq = sc_real(Hs[lane + lane * KP]);
   }
   const R hinf = warp_max(hrow);
-  __syncwarp();
   // ---- inverse, conditioning, inverse iteration
   S inv[KMAX];
   R piv = R(1), scale = R(1);
