@@ -751,7 +751,8 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
   }
   r2 = qsum(r2, qm);
   const double resj = sqrt(r2);
-  if (zeros != 0 && resj == 0.0) flags |= DIAF_FLAG_RANK_DEFICIENT;  // otherwise sigma_min > 1e-12 sigma_max
+  // (no zero column: sigma_min > 1e-12 sigma_max; ||H||_inf <= k sigma_max^2)
+  if (zeros != 0 && resj <= 1e-14 * (double)sqrtf(hinf / (float)k)) flags |= DIAF_FLAG_RANK_DEFICIENT;
   finite &= isfinite(resj);
   double* Wout = reinterpret_cast<double*>(a.Wv) + a.Wcp[j];
   for (int q = sub; q < k; q += 4) {
