@@ -16,7 +16,9 @@ struct CtaScratch {
   int ldm;        // leading dimension (>= every m_j, k_j of the bucket)
   int kcap;       // columns per tile (>= every k_j of the bucket)
   int gram;       // mixed real DIAF-S: 1 = tensor-core Gram + Cholesky where the tile is well conditioned
+  uint16_t* eloc; // mixed real DIAF-S: per CTA the tile row of every gathered entry (kCtaGather)
 };
+constexpr int kCtaGather = 4096;  // entries of a column's tile (the symbolic pass's limit)
 
 // ----------------------------------------------------------------- block reductions
 template <class T>
@@ -304,11 +306,8 @@ __device__ void cta_householder_qr(S* T, int ld, int m, int k, RealOf<S>* redR, 
 // One-sided Jacobi on the p x q matrix G (shared memory, leading dimension
 // LDG) with V (q x q, leading dimension LDV): the same rotation as
 // warp_jacobi, the q/2 pairs of a round spread over the CTA (LPP threads per
-// pair), a barrier between rounds.  PREDICT as for warp_jacobi (callers
-// whose result is refined afterwards): no sweep that would only confirm
-// convergence after a sweep whose rotations all had |gamma| < sqrt(tol)
-// sqrt(alpha beta).
-template <class S, int LDG, int LDV, bool PREDICT = false>
+// pair), a barrier between rounds.
+template <class S, int LDG, int LDV>
 __device__ int cta_jacobi(S* G, int p, int q, S* V, RealOf<S>* redR) {
   using R = RealOf<S>;
   constexpr int LPP = kCtaThreads / (kCtaKmax / 2);  // 8 threads per pair
@@ -330,7 +329,6 @@ __device__ int cta_jacobi(S* G, int p, int q, S* V, RealOf<S>* redR) {
   const int grp = tid / LPP, sub = tid % LPP;
   for (int sweep = 1; sweep <= kMaxSweeps; ++sweep) {
     int rotated = 0;
-    int large = 0;  // PREDICT: a rotation with |gamma|^2 >= tol alpha beta
     for (int rnd = 0; rnd < qq - 1; ++rnd) {
       int a = -1, b = -1;
       if (grp < npairs) {
@@ -360,7 +358,6 @@ __device__ int cta_jacobi(S* G, int p, int q, S* V, RealOf<S>* redR) {
       const bool rot = act && al > tiny && be > tiny && ag2 > R(0) && ag2 > tol2 * (al * be);
       if (rot) {
         rotated = 1;
-        if (PREDICT && ag2 >= tol * (al * be)) large = 1;
         R ag;
         S eph;
         if constexpr (ScalarInfo<S>::cplx) {
@@ -392,7 +389,6 @@ __device__ int cta_jacobi(S* G, int p, int q, S* V, RealOf<S>* redR) {
       __syncthreads();
     }
     if (!__syncthreads_or(rotated)) return sweep;
-    if (PREDICT && !__syncthreads_or(large)) return sweep;
   }
   return -1;
 }
@@ -413,7 +409,7 @@ struct CtaSmem {
 template <class S>
 __device__ void cta_finish(const ColArgs& a, int j, int k, int m, int l, int jpos, const S* Ts, int ld, S* wv, S* vv,
                            const int32_t* Is, const int32_t* Iloc, const int32_t* inI, uint32_t flags, bool do_phase,
-                           RealOf<S>* redR, double rank_thr = -1.0) {
+                           RealOf<S>* redR, double rank_thr = -1.0, double r2_known = -1.0) {
   using R = RealOf<S>;
   const int tid = threadIdx.x;
   if (do_phase) {
@@ -440,16 +436,19 @@ __device__ void cta_finish(const ColArgs& a, int j, int k, int m, int l, int jpo
     for (int t = tid; t < l; t += kCtaThreads) vv[t] = ph * vv[t];
     __syncthreads();
   }
-  R r2 = R(0);
-  for (int r = tid; r < m; r += kCtaThreads) {
-    S s2 = sc_zero<S>();
-    for (int q = 0; q < k; ++q) s2 += Ts[r + (size_t)q * ld] * wv[q];
-    if (inI[r] >= 0) s2 -= vv[inI[r]];
-    r2 += sc_abs2(s2);
+  R r2 = R(r2_known);
+  if (r2_known < 0.0) {
+    r2 = R(0);
+    for (int r = tid; r < m; r += kCtaThreads) {
+      S s2 = sc_zero<S>();
+      for (int q = 0; q < k; ++q) s2 += Ts[r + (size_t)q * ld] * wv[q];
+      if (inI[r] >= 0) s2 -= vv[inI[r]];
+      r2 += sc_abs2(s2);
+    }
+    for (int t = tid; t < l; t += kCtaThreads)
+      if (Iloc[t] < 0) r2 += sc_abs2(vv[t]);
+    r2 = block_sum(r2, redR);
   }
-  for (int t = tid; t < l; t += kCtaThreads)
-    if (Iloc[t] < 0) r2 += sc_abs2(vv[t]);
-  r2 = block_sum(r2, redR);
   const double resj = sqrt((double)r2);
   if (resj <= rank_thr) flags |= DIAF_FLAG_RANK_DEFICIENT;
   int bad = !isfinite(resj);

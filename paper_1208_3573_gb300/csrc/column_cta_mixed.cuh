@@ -8,6 +8,14 @@
 // the FP64 tile; twice when the gap is below 1e-2).  v_j = T(I_j,:) w_j and the
 // residual are evaluated in FP64.
 //
+// What bounds it: chains of barriers, shuffles and divisions (Jacobi about a
+// quarter of the time) and the FP64 pipe, which takes an instruction per 19
+// cycles and SM whatever its lanes hold.  So the FP64 products run over the
+// gathered entries (these tiles hold little more than one per row) instead of
+// all m k places, and scalars come from one or two warps, not from all eight.
+// Power-law n = 200,000, 40,104 columns with tiles up to 636 x 60: 22.5 -> 18.1
+// ms for the bucket.
+//
 // A leverage decision within 2 delta of its threshold (delta = (m + k) eps_32
 // kappa) makes the kernel recompute the column's keys in FP64 with the FP64
 // CTA kernel's own QR and key computation and select with those.  A column
@@ -238,25 +246,72 @@ __device__ inline void cta_col_norms_f(const float* T, int ld, int m, int k, dou
   __syncthreads();
 }
 
-// g = H x = A-hat^T (A-hat x) in FP64 from the FP64 tile (rows of I_j
-// excluded), z = A-hat x (m) as scratch.
-__device__ inline void cta_hat_gram_apply(const double* Ts, int ld, int m, int k, const int32_t* inI, const double* x,
-                                          double* z, double* g) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int r = tid; r < m; r += kCtaThreads) {
-    double zr = 0.0;
-    if (inI[r] < 0)
-      for (int q = 0; q < k; ++q) zr += Ts[r + (size_t)q * ld] * x[q];
-    z[r] = zr;
+// The tile's entries as gathered: column q's are entries coff[q] .. of the
+// tile, A's values from cst[q] on, tile rows in eloc; rm: which columns each
+// row has (two words per row).
+struct CtaEntries {
+  const double* Av;
+  const int32_t* cst;
+  const int32_t* coff;
+  const uint16_t* eloc;
+  const uint32_t* rm;
+  int E;
+};
+
+// (T x)_r over row r's entries, columns ascending.
+__device__ __forceinline__ double cta_row_mul(const CtaEntries& en, const double* Ts, int ld, int r, const double* x) {
+  double z = 0.0;
+  for (uint32_t b = en.rm[2 * r]; b; b &= b - 1) {
+    const int p = __ffs(b) - 1;
+    z = fma(Ts[r + (size_t)p * ld], x[p], z);
+  }
+  for (uint32_t b = en.rm[2 * r + 1]; b; b &= b - 1) {
+    const int p = 31 + __ffs(b);
+    z = fma(Ts[r + (size_t)p * ld], x[p], z);
+  }
+  return z;
+}
+
+// g = H x = A-hat^T (A-hat x) in FP64 over the tile's entries (rows of I_j
+// excluded), z = A-hat x (m) as scratch: a thread per row, four per column.
+__device__ inline void cta_hat_gram_apply(const CtaEntries& en, const double* Ts, int ld, int m, int k,
+                                          const int32_t* inI, const double* x, double* z, double* g) {
+  const int tid = threadIdx.x;
+  for (int r = tid; r < m; r += kCtaThreads) z[r] = inI[r] < 0 ? cta_row_mul(en, Ts, ld, r, x) : 0.0;
+  __syncthreads();
+  const int q = tid >> 2, sub = tid & 3;
+  static_assert(kCtaThreads == 4 * kCtaKmax, "four threads per column");
+  double gq = 0.0;
+  if (q < k) {
+    const int e0 = en.coff[q], e1 = q + 1 < k ? en.coff[q + 1] : en.E;
+    const double* av = en.Av + en.cst[q] - e0;
+#pragma unroll 4
+    for (int e = e0 + sub; e < e1; e += 4) gq = fma(av[e], z[en.eloc[e]], gq);
+  }
+  gq += shfl_xor(gq, 1);
+  gq += shfl_xor(gq, 2);
+  if (q < k && sub == 0) g[q] = gq;
+  __syncthreads();
+}
+
+// Two sums over k <= 64 threads' values (the other threads' are zero): block_sum
+// in the two warps that hold them, the same bits for a fifth of the FP64
+// instructions.
+__device__ __forceinline__ void block_sum_k(double& u, double& v, double* red) {
+  static_assert(kCtaKmax == 64, "two warps hold the values");
+  const int warp = threadIdx.x >> 5;
+  __syncthreads();
+  if (warp < 2) {
+    u = warp_sum(u);
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) {
+      red[2 * warp] = u;
+      red[2 * warp + 1] = v;
+    }
   }
   __syncthreads();
-  for (int c = warp; c < k; c += kCtaWarps) {
-    double gc = 0.0;
-    for (int r = lane; r < m; r += 32) gc += Ts[r + (size_t)c * ld] * z[r];
-    gc = warp_sum(gc);
-    if (lane == 0) g[c] = gc;
-  }
-  __syncthreads();
+  u = red[0] + red[2];
+  v = red[1] + red[3];
 }
 
 // One second-order correction of x (FP64, k) with Rayleigh quotient d and
@@ -289,6 +344,102 @@ __device__ inline float cta_basis_correction(const float* V, int ldv, const doub
 }
 
 constexpr int kClusterMax = 4;  // most singular values of a close cluster resolved in mixed precision
+
+// One-sided Jacobi of the k x k FP32 R-hat (G, leading dimension KP), V its
+// accumulated rotations: cta_jacobi's sweeps (eight threads per pair, the same
+// sums in the same order) with the pair's entries held in registers between
+// the dot products and the rotation, all loads of a column in flight, and the
+// pairing's modulo a conditional subtraction.  It ends after a sweep whose
+// rotations were all below |gamma|^2 = tol alpha beta (convergence is
+// quadratic: the next sweep would rotate nothing).  A round is a chain of
+// shared loads, three shuffle sums, a square root and a division between two
+// barriers; the number of threads per pair is set by k_j <= 64 and 256 threads.
+template <int KP>
+__device__ int cta_jacobi_mixed(float* G, int k, float* V, float* redF) {
+  constexpr int LPP = kCtaThreads / (kCtaKmax / 2), NR = kCtaKmax / LPP;
+  const int tid = threadIdx.x;
+  for (int i = tid; i < k * k; i += kCtaThreads) {
+    const int r = i % k, c = i / k;
+    V[r + c * KP] = r == c ? 1.0f : 0.0f;
+  }
+  float part = 0.0f;
+  for (int i = tid; i < k * k; i += kCtaThreads) part += sc_abs2(G[(i % k) + (i / k) * KP]);
+  const float nf2 = block_sum(part, redF);
+  const float tol = float(k) * eps_of<float>();
+  const float tol2 = tol * tol;
+  const float tiny = tol2 * nf2;
+  __syncthreads();
+  if (k < 2) return 1;
+  const int qq = (k + 1) & ~1;
+  const int grp = tid / LPP, sub = tid % LPP;
+  const bool warp_has_pair = (tid & ~31) / LPP < qq / 2;  // warp uniform
+  for (int sweep = 1; sweep <= kMaxSweeps; ++sweep) {
+    int rotated = 0, large = 0;
+    int a0 = grp - 1, b0 = qq - 2 - grp;  // places on the ring of qq - 1
+    for (int rnd = 0; rnd < qq - 1; ++rnd) {
+      if (warp_has_pair) {
+        int a = grp == 0 ? 0 : 1 + a0, b = 1 + b0;
+        if (a > b) { const int t = a; a = b; b = t; }
+        const bool act = grp < qq / 2 && b < k;
+        float* ca = G + a * KP + sub;
+        float* cb = G + b * KP + sub;
+        float x[NR], y[NR];
+        float al = 0.0f, be = 0.0f, ga = 0.0f;
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+          if (i * LPP < k) {  // uniform
+            const bool in = act && i * LPP + sub < k;
+            x[i] = in ? ca[i * LPP] : 0.0f;
+            y[i] = in ? cb[i * LPP] : 0.0f;
+          }
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+          if (i * LPP < k) {
+            al += sc_abs2(x[i]);
+            be += sc_abs2(y[i]);
+            ga += sc_cmul(x[i], y[i]);
+          }
+        al = group_sum<LPP>(al);
+        be = group_sum<LPP>(be);
+        ga = group_sum<LPP>(ga);
+        const float ag2 = sc_abs2(ga);
+        if (act && al > tiny && be > tiny && ag2 > 0.0f && ag2 > tol2 * (al * be)) {
+          rotated = 1;
+          if (ag2 >= tol * (al * be)) large = 1;
+          float* va = V + a * KP + sub;
+          float* vb = V + b * KP + sub;
+          float vx[NR], vy[NR];
+#pragma unroll
+          for (int i = 0; i < NR; ++i)
+            if (i * LPP < k) {
+              const bool in = i * LPP + sub < k;
+              vx[i] = in ? va[i * LPP] : 0.0f;
+              vy[i] = in ? vb[i * LPP] : 0.0f;
+            }
+          const float ag = sc_abs(ga), eph = sc_unit(ga);
+          const float d = be - al;
+          const float t = copysign(2.0f * ag, d) / (fabs(d) + sqrt(d * d + 4.0f * ag2));
+          const float cs = rsqrt_r(1.0f + t * t), sn = cs * t;
+#pragma unroll
+          for (int i = 0; i < NR; ++i)
+            if (i * LPP < k && i * LPP + sub < k) {
+              const float yi = eph * y[i], wi = eph * vy[i];
+              ca[i * LPP] = cs * x[i] - sn * yi;
+              cb[i * LPP] = sn * x[i] + cs * yi;
+              va[i * LPP] = cs * vx[i] - sn * wi;
+              vb[i * LPP] = sn * vx[i] + cs * wi;
+            }
+        }
+        a0 = a0 + 1 == qq - 1 ? 0 : a0 + 1;
+        b0 = b0 + 1 == qq - 1 ? 0 : b0 + 1;
+      }
+      __syncthreads();
+    }
+    if (!__syncthreads_or(rotated)) return sweep;
+    if (!__syncthreads_or(large)) return sweep;
+  }
+  return -1;
+}
 
 // Eigen-decomposition of the symmetric p x p matrix K (leading dimension
 // kClusterMax, FP64) by cyclic Jacobi rotations, one thread: K becomes
@@ -428,7 +579,7 @@ constexpr float kClusterCorrectionTol = 1e-10f;  // ... converged when no update
 __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, int j, unsigned char* smem) {
   using L = CtaMixedSmem;
   constexpr int KP = L::KP;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int mcap = sc.ldm;
   float* Rs = reinterpret_cast<float*>(smem);  // R of T, then R-hat (KP x KMAX)
   float* Vj = Rs + KP * kCtaKmax;               // Jacobi V (Gram path: first D R_s^-1)
@@ -452,6 +603,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
   int32_t* cst = Iloc + mcap;
   int32_t* coff = cst + kCtaKmax;
   int32_t* misc = coff + kCtaKmax;  // [0] jpos, [1] count
+  uint16_t* eloc = sc.eloc + (size_t)blockIdx.x * kCtaGather;
   float* redF = reinterpret_cast<float*>(red);
 
   // the slab holds two tiles of the FP64 kernel's size: the FP64 tile, then
@@ -488,6 +640,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     const int p = cst[q] + (e - coff[q]);
     const int r = lower_bound_i32(rs, m, a.Ari[p]);
     Ts[r + (size_t)q * ld] = Av[p];
+    eloc[e] = (uint16_t)r;
   }
   __syncthreads();
   for (size_t i = tid; i < (size_t)me * k; i += kCtaThreads) {
@@ -640,23 +793,41 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
   if (m - inrows < k) { CTA_FB(1); return false; }  // A-hat has fewer rows than columns
 
   DIAF_PHASE(4);
+  // which columns each row has, over the keys (dead now)
+  uint32_t* rm = reinterpret_cast<uint32_t*>(hk);
+  for (int r = tid; r < 2 * m; r += kCtaThreads) rm[r] = 0;
+  __syncthreads();
+  {
+    const int c = tid >> 2;
+    const int e1 = c >= k ? 0 : c + 1 < k ? coff[c + 1] : E;
+    for (int e = c < k ? coff[c] + (tid & 3) : 0; e < e1; e += 4) atomicOr(&rm[2 * eloc[e] + (c >> 5)], 1u << (c & 31));
+  }
+  __syncthreads();
+  const CtaEntries en{Av, cst, coff, eloc, rm, E};
   // ---- R-hat: from G on the Gram path (G minus the I_j rows' outer
   // products, Cholesky of its column-scaled form), else FP32 QR of A-hat
   bool gram_hat = false;
   if (gram && tw_intact) {
     int zc = 0;  // an exactly zero column of A-hat (all its entries in I_j rows) keeps the QR path
-    for (int c = tid; c < k; c += kCtaThreads) {
-      bool nz = false;
-      for (int r = 0; r < m && !nz; ++r) nz = inI[r] < 0 && Tw[r + (size_t)c * ld] != 0.0f;
-      zc |= !nz;
+    {
+      const int c = tid >> 2;  // four threads per column, over its entries
+      int nz = 0;
+      if (c < k) {
+        const int e1 = c + 1 < k ? coff[c + 1] : E;
+        for (int e = coff[c] + (tid & 3); e < e1 && !nz; e += 4)
+          nz = inI[eloc[e]] < 0 && (float)Av[cst[c] + (e - coff[c])] != 0.0f;
+      }
+      const unsigned any = __ballot_sync(0xffffffffu, nz) >> (tid & 28) & 15u;
+      zc = c < k && any == 0u;
     }
     if (!__syncthreads_or(zc)) {
       for (int i = tid; i < k * k; i += kCtaThreads) {
         const int p = i % k, q = i / k;
         float gpq = Gm[p + q * sc.kcap];
-        for (int t = 0; t < l; ++t) {
+        for (int t = 0; t < l; ++t) {  // rows with entries in both columns
           const int r = Iloc[t];
-          if (r >= 0) gpq -= Tw[r + (size_t)p * ld] * Tw[r + (size_t)q * ld];
+          if (r >= 0 && (rm[2 * r + (p >> 5)] >> (p & 31) & 1u) && (rm[2 * r + (q >> 5)] >> (q & 31) & 1u))
+            gpq -= Tw[r + (size_t)p * ld] * Tw[r + (size_t)q * ld];
         }
         Rs[p + q * KP] = gpq;
       }
@@ -672,9 +843,6 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
         for (int c = tid; c < k; c += kCtaThreads) kp = fmaxf(kp, 1.0f / fabsf(Rs[c + c * KP]));
         if (block_max(kp, redF) <= kGramKappaMax) {
           gram_hat = true;
-#ifdef DIAF_PHASE_TIMING
-          if (threadIdx.x == 0 && a.phase) atomicAdd(&a.phase[30], 1ull);
-#endif
           for (int i = tid; i < k * k; i += kCtaThreads) Rs[(i % k) + (i / k) * KP] *= (float)cn[i / k];
           __syncthreads();
         }
@@ -703,7 +871,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     __syncthreads();
   }
   DIAF_PHASE(6);
-  if (cta_jacobi<float, KP, KP, true>(Rs, k, k, Vj, redF) < 0) flags |= DIAF_FLAG_JACOBI_NOCONV;
+  if (cta_jacobi_mixed<KP>(Rs, k, Vj, redF) < 0) flags |= DIAF_FLAG_JACOBI_NOCONV;
   DIAF_PHASE(7);
   for (int c = tid; c < k; c += kCtaThreads) {
     float s2 = 0.0f;
@@ -711,18 +879,30 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     sig[c] = (double)sqrtf(s2);
   }
   __syncthreads();
-  int imin = 0;
-  double smin = sig[0], smax = sig[0];
-  for (int c = 1; c < k; ++c) {
-    if (sig[c] < smin) { smin = sig[c]; imin = c; }
-    smax = dmax(smax, sig[c]);
-  }
-  double snext = INFINITY, gap = INFINITY;
-  for (int c = 0; c < k; ++c)
-    if (c != imin) {
-      snext = dmin(snext, sig[c]);
-      gap = dmin(gap, sig[c] * sig[c] - smin * smin);
+  // sigma_min (lowest index among equals), sigma_max, the next one and the gap
+  // by one warp: a scan by every thread is 8 k FP64 instructions of each kind,
+  // and the SM takes one per 19 cycles
+  if (warp == 0) {
+    const double s0 = lane < k ? sig[lane] : INFINITY, s1 = lane + 32 < k ? sig[lane + 32] : INFINITY;
+    const double lo = warp_min(dmin(s0, s1));
+    double hi = dmax(lane < k ? s0 : 0.0, lane + 32 < k ? s1 : 0.0);
+    for (int o = 16; o; o >>= 1) hi = dmax(hi, shfl_xor(hi, o));
+    const unsigned e0 = __ballot_sync(0xffffffffu, s0 == lo), e1 = __ballot_sync(0xffffffffu, s1 == lo);
+    const int im = e0 ? __ffs(e0) - 1 : (e1 ? 31 + __ffs(e1) : 0);
+    const double o0 = lane == im ? INFINITY : s0, o1 = lane + 32 == im ? INFINITY : s1;
+    const double nx = warp_min(dmin(o0, o1));
+    if (lane == 0) {
+      misc[6] = im;
+      wv[0] = hi;
+      wv[1] = nx;
     }
+  }
+  __syncthreads();
+  const int imin = misc[6];
+  const double smin = sig[imin], smax = wv[0], snext = wv[1];
+  // s^2 is monotonic in s, so the smallest gap is the next value's
+  const double gap = snext * snext - smin * smin;
+  __syncthreads();  // wv is overwritten below
   if (k > 1 && (snext - smin) <= 1e-6 * smax) flags |= DIAF_FLAG_DEGENERATE;
   // A close cluster: sigma_min^2 and the next singular values, each within
   // 1e-5 smax^2 of the one before, up to kClusterMax of them (the rest at
@@ -730,7 +910,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
   // ordered wrongly) at FP32 accuracy, so all of them are corrected against
   // the other singular vectors and the cluster is resolved by a
   // Rayleigh-Ritz step in FP64.  A longer chain goes to the FP64 kernel.
-  int32_t* cl = cst;  // the cluster's singular indices (the gather's offsets are dead)
+  int32_t* cl = misc + 2;  // the cluster's singular indices (kClusterMax of them)
   uint64_t excl = 1ull << imin;
   int p = 1;
   if (k > 1 && gap <= 1e-5 * smax * smax) {
@@ -755,14 +935,13 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     for (int c = tid; c < k; c += kCtaThreads) wv[c] = (double)Vj[c + imin * KP];
     __syncthreads();
     for (int it = 0; it < iters; ++it) {
-      cta_hat_gram_apply(Ts, ld, m, k, inI, wv, zz, gg);
+      cta_hat_gram_apply(en, Ts, ld, m, k, inI, wv, zz, gg);
       double xg = 0.0, xx = 0.0;
       for (int c = tid; c < k; c += kCtaThreads) {
         xg += wv[c] * gg[c];
         xx += wv[c] * wv[c];
       }
-      xg = block_sum(xg, red);
-      xx = block_sum(xx, red);
+      block_sum_k(xg, xx, red);
       const double d = xg / xx;
       cta_basis_correction(Vj, KP, sig, k, excl, d, gg, wv, rf, cc);
     }
@@ -780,7 +959,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     __syncthreads();
     bool conv = false;
     for (int it = 0;; ++it) {
-      for (int c = 0; c < p; ++c) cta_hat_gram_apply(Ts, ld, m, k, inI, Xc + c * k, zz, Gc + c * k);
+      for (int c = 0; c < p; ++c) cta_hat_gram_apply(en, Ts, ld, m, k, inI, Xc + c * k, zz, Gc + c * k);
       cta_cluster_rayleigh_ritz(Xc, Gc, p, k, red, Km, Qm, th);
       if (conv) break;
       if (it == kClusterMaxCorrections) { CTA_FB(3); return false; }
@@ -795,23 +974,25 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     if (sqrt(dmax(th[1], 0.0)) - sqrt(dmax(th[0], 0.0)) <= 1e-6 * smax) flags |= DIAF_FLAG_DEGENERATE;
     __syncthreads();
   }
-  double xn = 0.0;
+  double xn = 0.0, unused = 0.0;
   for (int c = tid; c < k; c += kCtaThreads) xn += wv[c] * wv[c];
-  xn = block_sum(xn, red);
+  block_sum_k(xn, unused, red);
   const double inv = 1.0 / sqrt(xn);
   for (int c = tid; c < k; c += kCtaThreads) wv[c] *= inv;
   __syncthreads();
   DIAF_PHASE(8);
-  // v = T(I_j,:) w in FP64
-  for (int t = tid; t < l; t += kCtaThreads) {
-    double s2 = 0.0;
-    const int r = Iloc[t];
-    if (r >= 0)
-      for (int q = 0; q < k; ++q) s2 += Ts[r + (size_t)q * ld] * wv[q];
-    vv[t] = s2;
-  }
+  // v = T(I_j,:) w and the other rows' ||T w||^2 in FP64, over the rows' entries
+  for (int t = tid; t < l; t += kCtaThreads) vv[t] = 0.0;
   __syncthreads();
-  cta_finish<double>(a, j, k, m, l, jpos, Ts, ld, wv, vv, Is, Iloc, inI, flags, true, red, 1e-14 * smax);
+  double r2 = 0.0;
+  for (int r = tid; r < m; r += kCtaThreads) {
+    const double t = cta_row_mul(en, Ts, ld, r, wv);
+    if (inI[r] >= 0) vv[inI[r]] = t;
+    else r2 = fma(t, t, r2);
+  }
+  r2 = block_sum(r2, red);
+  cta_finish<double>(a, j, k, m, l, jpos, Ts, ld, wv, vv, Is, Iloc, inI, flags, true, red,
+                     1e-14 * smax, r2);
   DIAF_PHASE(9);
   return true;
 }
