@@ -58,7 +58,7 @@ struct ColArgs {
   const int32_t* list_count;  // device count of the list
   int32_t* work_counter;      // zeroed before launch
   uint32_t extra_flags;       // OR-ed into every column's flags (FP64 fallback of the mixed form)
-  int32_t* fb_list;           // mixed form: columns handed to the FP64 kernel
+  int32_t* fb_list;           // mixed form: columns handed to the FP64 kernel (~j: with I_j decided, in Vri)
   int32_t* fb_count;
   void* Wv;
   int32_t* Vri;
@@ -211,13 +211,24 @@ __device__ inline double select_rows_greedy(const int32_t* rs, const K* hk, int3
   return (double)warp_min(margin);
 }
 
-// I_j from the picks (rule) or the fixed pattern; fills Is, Iloc, inI; returns
-// the position of j in I_j (-1 if absent).
-__device__ inline int build_I(const ColArgs& a, int j, int m, int l, const ColumnIdx& ix, int lane) {
+// I_j's rows at the host: the rows, then the column's word.
+__device__ inline void publish_I(const ColArgs& a, int j, int l, const int32_t* Is, int lane) {
+  const int v0 = a.Vcp[j];
+  for (int t = lane; t < l; t += DIAF_WARP) a.Hri[v0 + t] = Is[t];
+  __threadfence_system();
+  __syncwarp();
+  if (lane == 0) store_release_sys(a.Hgen + j, a.gen);
+}
+
+// I_j from the picks (rule), the fixed pattern or, with `given`, Vri (the mixed
+// kernel decided it); fills Is, Iloc, inI; returns the position of j in I_j
+// (-1 if absent).
+__device__ inline int build_I(const ColArgs& a, int j, int m, int l, const ColumnIdx& ix, int lane,
+                              bool given = false) {
   if (lane == 0) ix.misc[0] = -1;
   __syncwarp();
-  if (a.rule == DIAF_RULE_FIXED) {
-    const int32_t* Vf = a.Vfri + a.Vfcp[j];
+  if (given || a.rule == DIAF_RULE_FIXED) {
+    const int32_t* Vf = given ? a.Vri + a.Vcp[j] : a.Vfri + a.Vfcp[j];
     for (int t = lane; t < l; t += DIAF_WARP) {
       int row = Vf[t];
       int r = lower_bound_i32(ix.rs, m, row);
@@ -267,7 +278,7 @@ __device__ inline int build_I(const ColArgs& a, int j, int m, int l, const Colum
 template <class SD, int LDT>
 __device__ void finish_column(const ColArgs& a, int j, int k, int m, int l, int jpos, const SD* Ts, SD* wv, SD* vv,
                               const ColumnIdx& ix, uint32_t flags, bool do_phase, int lane,
-                              double rank_thr = -1.0, double r2_known = -1.0) {
+                              double rank_thr = -1.0, double r2_known = -1.0, bool given = false) {
   using R = RealOf<SD>;
   if (do_phase) {
     SD ph = sc_real_s<SD>(R(1));
@@ -326,12 +337,7 @@ __device__ void finish_column(const ColArgs& a, int j, int k, int m, int l, int 
     a.res[j] = resj;
     a.flags[j] = flags | a.extra_flags;
   }
-  if (a.Hri) {  // the final I_j to the host: rows, then the column's word
-    for (int t = lane; t < l; t += DIAF_WARP) a.Hri[v0 + t] = ix.Is[t];
-    __threadfence_system();
-    __syncwarp();
-    if (lane == 0) store_release_sys(a.Hgen + j, a.gen);
-  }
+  if (a.Hri && !given) publish_I(a, j, l, ix.Is, lane);  // (given: the host has it and may have reused the mirror)
   __syncwarp();
 }
 
@@ -437,7 +443,7 @@ __device__ S stabilise_q_warp(const ColArgs& a, const S* Ts, S* Tw, const S* Rs,
 }
 
 template <class S, int KMAX, int MMAX, int ALG>
-__device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, int lane) {
+__device__ void solve_column_warp(const ColArgs& a, int j, bool given, unsigned char* smem, int lane) {
   using R = RealOf<S>;
   using L = WarpLayout<S, KMAX, MMAX>;
   constexpr int LDT = L::LDT, KP = L::KP;
@@ -475,10 +481,11 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
   for (int c = lane; c < k; c += DIAF_WARP) rdmax = dmax(rdmax, sc_abs(Rs[c + c * KP]));
   rdmax = warp_max(rdmax);
   const R piv = R(1e-14) * rdmax;
-  if (k > 0 && (a.rule != DIAF_RULE_FIXED || ALG == DIAF_ALG_Q))
+  const bool select = !given && a.rule != DIAF_RULE_FIXED;
+  if (k > 0 && (select || ALG == DIAF_ALG_Q))
     warp_leverage_rows<S, S, LDT, KP>(Ts, Rs, Tw, hk, rinv, m, k, piv, lane);
-  if (a.rule != DIAF_RULE_FIXED) select_rows_greedy<MMAX / DIAF_WARP>(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
-  const int jpos = build_I(a, j, m, l, ix, lane);
+  if (select) select_rows_greedy<MMAX / DIAF_WARP>(ix.rs, hk, ix.pick, m, a.rule, j, l - 1, a.tie_tol, lane, a.blk);
+  const int jpos = build_I(a, j, m, l, ix, lane, given);
 
   for (int t = lane; t < l; t += DIAF_WARP) vv[t] = sc_zero<S>();
   for (int q = lane; q < k; q += DIAF_WARP) wv[q] = sc_zero<S>();
@@ -579,7 +586,7 @@ __device__ void solve_column_warp(const ColArgs& a, int j, unsigned char* smem, 
     if (lane < k) wv[lane] = x;
     __syncwarp();
   }
-  finish_column<S, LDT>(a, j, k, m, l, jpos, Ts, wv, vv, ix, flags, k > 0 || ALG == DIAF_ALG_Q, lane);
+  finish_column<S, LDT>(a, j, k, m, l, jpos, Ts, wv, vv, ix, flags, k > 0 || ALG == DIAF_ALG_Q, lane, -1.0, -1.0, given);
 }
 
 template <class S, int KMAX, int MMAX, int ALG>
@@ -593,6 +600,7 @@ __global__ void column_warp_kernel(ColArgs a) {
     if (lane == 0) idx = atomicAdd(a.work_counter, 1);
     idx = __shfl_sync(DIAF_FULL, idx, 0);
     if (idx >= count) break;
-    solve_column_warp<S, KMAX, MMAX, ALG>(a, list_at(a, count, idx), smem, lane);
+    const int j = list_at(a, count, idx);  // ~j: I_j decided by the mixed kernel
+    solve_column_warp<S, KMAX, MMAX, ALG>(a, j < 0 ? ~j : j, j < 0, smem, lane);
   }
 }
