@@ -506,17 +506,16 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
   np.wpb[1] = tuning ? tuning->warps_per_block[1] : 0;
 
   uint32_t* status;
-  int32_t *stats, *big_count;
+  PlanCounters* pc;
   int64_t* bs64;
   int32_t* bs32;
   PlanArgs pa{};
   DIAF_CU(F->alloc(&status, 1));
   F->status = status;
   // the symbolic scratch in one allocation; the small counters in one block
-  // (stats[4], then the bucket counts, then the large-tile count: one memset)
   {
     Carve c;
-    c.add(&stats, 4 + kNumBuckets + 1);
+    c.add(&pc, 1);
     c.add(&np.work, kWorkCounters);
     c.add(&pa.k, n);
     c.add(&pa.E, n);
@@ -530,15 +529,18 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
     c.add(&bs32, scan_blocksums_size(n));
     DIAF_CU(pool.carve(c));
   }
-  np.bucket_count = stats + 4;
-  big_count = stats + 4 + kNumBuckets;
+  np.bucket_count = pc->bucket_count;
   DIAF_CU(cudaMemsetAsync(status, 0, sizeof(uint32_t), s));
-  DIAF_CU(cudaMemsetAsync(stats, 0, sizeof(int32_t) * (4 + kNumBuckets + 1), s));
+  DIAF_CU(cudaMemsetAsync(pc, 0, sizeof(PlanCounters), s));
 
   // ---- input checks on the device (sorted, in range)
-  DIAF_CU(check_csc(n, A->colptr, A->rowidx, A->nnz, status, s));
-  DIAF_CU(check_csc(n, PW->colptr, PW->rowidx, PW->nnz, status, s));
-  if (V->rule == DIAF_RULE_FIXED) DIAF_CU(check_csc(n, V->fixed->colptr, V->fixed->rowidx, V->fixed->nnz, status, s));
+  {
+    CscCheck c;
+    c.add(A->colptr, A->rowidx, A->nnz);
+    c.add(PW->colptr, PW->rowidx, PW->nnz);
+    if (V->rule == DIAF_RULE_FIXED) c.add(V->fixed->colptr, V->fixed->rowidx, V->fixed->nnz);
+    DIAF_CU(check_csc(n, c, status, s));
+  }
 
   // ---- symbolic pass 1: k_j, E_j
   pa.n = n;
@@ -553,57 +555,51 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
   pa.edge_m1 = tuning && tuning->m_edge1 > 0 ? tuning->m_edge1 : 64;
   pa.bucket_list = np.bucket_list;
   pa.bucket_count = np.bucket_count;
-  pa.big_count = big_count;
-  pa.stats = stats;
+  pa.big_count = &pc->big_count;
+  pa.stats = pc->stats;
   pa.status = status;
 
-  uint32_t h_status = 0;
-  int64_t h_Etot = 0;
+  PlanCounters h{};
   if (n > 0) {
     // the count kernel reads J_j only when the input check (earlier on the
     // stream) passed: it tests the status flag itself, so no sync here
     DIAF_CU(plan_count(pa, s));
-    DIAF_CU(exclusive_scan_i32_to_i64(pa.E, pa.Eoff, n, bs64, s));
-    DIAF_CU(cudaMemcpyAsync(&h_Etot, pa.Eoff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    DIAF_CU(cudaMemcpyAsync(&h_status, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    DIAF_CU(exclusive_scan_i32_to_i64(pa.E, pa.Eoff, n, bs64, s, ScanTail{&pc->Etot, status, &pc->status}));
+    DIAF_CU(cudaMemcpyAsync(&h, pc, sizeof(h), cudaMemcpyDeviceToHost, s));
     PT_DEV(s);
     PT_HOST();
     DIAF_CU(cudaStreamSynchronize(s));
     PT_HOST();
-    if (h_status & DEV_ST_BAD_INPUT) return fail(DIAF_EINVAL, "unsorted or out-of-range indices in A, PW or V");
+    if (h.status & DEV_ST_BAD_INPUT) return fail(DIAF_EINVAL, "unsorted or out-of-range indices in A, PW or V");
   }
-  DIAF_CU(pool.get(&pa.rows, (size_t)h_Etot));
+  DIAF_CU(pool.get(&pa.rows, (size_t)h.Etot));
   DIAF_CU(F->alloc(&F->Vcp, n + 1));
   if (n > 0) {
     DIAF_CU(plan_rows(pa, s));
-    DIAF_CU(exclusive_scan_i32(pa.l, F->Vcp, n, bs32, s));
+    DIAF_CU(exclusive_scan_i32(pa.l, F->Vcp, n, bs32, s, ScanTail{&pc->nnzv, status, &pc->status}));
   } else {
     DIAF_CU(cudaMemsetAsync(F->Vcp, 0, sizeof(int32_t), s));
   }
-  int32_t h_nnzv = 0, h_blk[4 + kNumBuckets] = {0};  // stats, then the bucket counts
-  int32_t* const h_stats = h_blk;
   if (n > 0) {
-    DIAF_CU(cudaMemcpyAsync(&h_nnzv, F->Vcp + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    DIAF_CU(cudaMemcpyAsync(h_blk, stats, sizeof(h_blk), cudaMemcpyDeviceToHost, s));
-    DIAF_CU(cudaMemcpyAsync(&h_status, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    DIAF_CU(cudaMemcpyAsync(&h, pc, sizeof(h), cudaMemcpyDeviceToHost, s));
     PT_DEV(s);
     PT_HOST();
     DIAF_CU(cudaStreamSynchronize(s));
     PT_HOST();
   }
-  for (int b = 0; b < kNumBuckets; ++b) np.h_bc[b] = h_blk[4 + b];
-  if (h_status & DEV_ST_CAPACITY)
+  for (int b = 0; b < kNumBuckets; ++b) np.h_bc[b] = h.bucket_count[b];
+  if (h.status & DEV_ST_CAPACITY)
     return fail(DIAF_EUNSUPPORTED, "a column needs more than 4096 gathered entries or a tile beyond 1024 x 64");
-  F->nnz_v = h_nnzv;
+  F->nnz_v = h.nnzv;
   F->info.n = n;
   F->info.dtype = A->dtype;
   F->info.alg = alg;
   F->info.prec = prec;
   F->info.nnz_w = PW->nnz;
-  F->info.nnz_v = h_nnzv;
-  F->info.max_k = h_stats[0];
-  F->info.max_m = h_stats[1];
-  F->info.max_l = h_stats[2];
+  F->info.nnz_v = h.nnzv;
+  F->info.max_k = h.stats[0];
+  F->info.max_m = h.stats[1];
+  F->info.max_l = h.stats[2];
   F->info.n_buckets = kNumBuckets;
   for (int b = 0; b < kNumBuckets; ++b) F->info.bucket_cols[b] = np.h_bc[b];
 
@@ -613,8 +609,8 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
     c.add(&F->Wcp, n + 1);
     c.add(&F->Wri, PW->nnz);
     c.add((char**)&F->Wv, esz * PW->nnz);
-    c.add(&F->Vri, h_nnzv);
-    c.add((char**)&F->Vv, esz * h_nnzv);
+    c.add(&F->Vri, h.nnzv);
+    c.add((char**)&F->Vv, esz * h.nnzv);
     c.add(&F->res, n);
     c.add(&F->flags, n);
     if (prec == DIAF_PREC_MIXED32) c.add(&F->fb_counts, kNumBuckets);
@@ -662,8 +658,8 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
     // bucket 0 of real DIAF-S: four lanes per column (unless the tuning asks for the warp kernel)
     const int small = tuning ? tuning->small_tiles : 0;
     if (!np.cplx && alg == DIAF_ALG_S && np.h_bc[0] > 0 && small != 2 && V->rule != DIAF_RULE_FIXED) {
-      const int M = h_stats[1] < pa.edge_m0 ? h_stats[1] : pa.edge_m0;
-      const int K = h_stats[0] < kThreadKMax ? h_stats[0] : kThreadKMax;
+      const int M = h.stats[1] < pa.edge_m0 ? h.stats[1] : pa.edge_m0;
+      const int K = h.stats[0] < kThreadKMax ? h.stats[0] : kThreadKMax;
       if (M >= 1 && K >= 1) {
         DIAF_CU(thread_columns_shape(M, K, np.h_bc[0], &np.tsh));
         np.ta.M = M;
@@ -679,9 +675,9 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
   const int bl = kNumBuckets - 1;
   if (np.h_bc[bl] > 0) {
     // large tiles: one CTA per column, FP64 in both precisions (tiles in scratch slabs)
-    const int mk = h_stats[1] > h_stats[0] ? h_stats[1] : h_stats[0];
+    const int mk = h.stats[1] > h.stats[0] ? h.stats[1] : h.stats[0];
     np.cs.ldm = (mk + 31) / 32 * 32;
-    np.cs.kcap = h_stats[0] > 0 ? h_stats[0] : 1;
+    np.cs.kcap = h.stats[0] > 0 ? h.stats[0] : 1;
     np.cs.gram = (tuning && tuning->large_tiles == 2) ? 0 : 1;  // the tensor-core Gram path unless asked off
     np.cta_grid = cta_columns_grid(A->dtype, alg, np.cs.ldm, np.h_bc[bl]);
     if (np.cta_grid <= 0) return fail(DIAF_EUNSUPPORTED, "large-tile kernel does not fit this tile size");

@@ -18,8 +18,10 @@ __device__ __forceinline__ bool admissible(int rule, int i, int j, const int32_t
 }
 
 // Input check: column pointers monotone, rows in range and strictly increasing.
-__global__ void check_csc_kernel(int n, const int32_t* __restrict__ cp, const int32_t* __restrict__ ri, int64_t nnz,
-                                 uint32_t* status) {
+__global__ void check_csc_kernel(int n, CscCheck c, uint32_t* status) {
+  const int32_t* __restrict__ cp = c.cp[blockIdx.y];
+  const int32_t* __restrict__ ri = c.ri[blockIdx.y];
+  const int64_t nnz = c.nnz[blockIdx.y];
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   int a = cp[j], b = cp[j + 1];
@@ -422,10 +424,20 @@ __global__ void scan_blocksums_kernel(TO* blocksums, int nb) {
   if (threadIdx.x == 0) blocksums[nb] = carry;
 }
 
+// With blocksums already scanned, or (sums) still the blocks' own totals, which
+// every block then adds up itself.
 template <class TI, class TO>
-__global__ void scan_apply_kernel(const TI* in, TO* out, int n, const TO* blocksums, int nb) {
+__global__ void scan_apply_kernel(const TI* in, TO* out, int n, const TO* blocksums, bool sums, ScanTail tail) {
   __shared__ TO sh[kScanThreads / 32];
   int base = blockIdx.x * kScanBlock;
+  TO before = TO(0);
+  if (sums) {
+    TO v = TO(0);
+    for (int i = threadIdx.x; i < blockIdx.x; i += kScanThreads) v += blocksums[i];
+    block_exclusive_scan<TO, TO>(v, sh, before);
+  } else {
+    before = blocksums[blockIdx.x];
+  }
   TO vals[kScanItems];
   TO s = 0;
   for (int i = 0; i < kScanItems; ++i) {
@@ -434,23 +446,38 @@ __global__ void scan_apply_kernel(const TI* in, TO* out, int n, const TO* blocks
     s += vals[i];
   }
   TO total;
-  TO ex = block_exclusive_scan<TI, TO>(s, sh, total) + blocksums[blockIdx.x];
+  TO ex = block_exclusive_scan<TI, TO>(s, sh, total) + before;
   for (int i = 0; i < kScanItems; ++i) {
     int idx = base + threadIdx.x * kScanItems + i;
     if (idx < n) out[idx] = ex;
     ex += vals[i];
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = blocksums[nb];
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+    out[n] = before + total;
+    if (tail.total) *static_cast<TO*>(tail.total) = before + total;
+    if (tail.status_copy) *tail.status_copy = *tail.status;
+  }
 }
 
+// One block: one launch.  Up to kScanSelfSum blocks: two, every block adding up
+// the totals before it (at most 8 loads a thread, which cost less than the
+// third launch of the general form in a stream of kernels of 2 to 3 us).
+// Beyond, the totals are scanned once by a kernel of their own.
+constexpr int kScanSelfSum = 8 * kScanThreads;
+
 template <class TI, class TO>
-cudaError_t exclusive_scan(const TI* in, TO* out, int n, TO* blocksums, cudaStream_t s) {
+cudaError_t exclusive_scan(const TI* in, TO* out, int n, TO* blocksums, cudaStream_t s, const ScanTail& tail) {
   int nb = ceil_div(n > 0 ? n : 1, kScanBlock);
-  scan_reduce_kernel<TI, TO><<<nb, kScanThreads, 0, s>>>(in, n, blocksums);
-  DIAF_COUNT_LAUNCH();
-  scan_blocksums_kernel<TO><<<1, kScanThreads, 0, s>>>(blocksums, nb);
-  DIAF_COUNT_LAUNCH();
-  scan_apply_kernel<TI, TO><<<nb, kScanThreads, 0, s>>>(in, out, n, blocksums, nb);
+  const bool sums = nb <= kScanSelfSum;
+  if (nb > 1) {
+    scan_reduce_kernel<TI, TO><<<nb, kScanThreads, 0, s>>>(in, n, blocksums);
+    DIAF_COUNT_LAUNCH();
+  }
+  if (!sums) {
+    scan_blocksums_kernel<TO><<<1, kScanThreads, 0, s>>>(blocksums, nb);
+    DIAF_COUNT_LAUNCH();
+  }
+  scan_apply_kernel<TI, TO><<<nb, kScanThreads, 0, s>>>(in, out, n, blocksums, sums, tail);
   DIAF_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -459,18 +486,20 @@ cudaError_t exclusive_scan(const TI* in, TO* out, int n, TO* blocksums, cudaStre
 
 int scan_blocksums_size(int n) { return ceil_div(n > 0 ? n : 1, kScanBlock) + 1; }
 
-cudaError_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int n, int64_t* blocksums, cudaStream_t s) {
+cudaError_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int n, int64_t* blocksums, cudaStream_t s,
+                                      const ScanTail& tail) {
   return exclusive_scan<int32_t, long long>(in, reinterpret_cast<long long*>(out), n,
-                                            reinterpret_cast<long long*>(blocksums), s);
+                                            reinterpret_cast<long long*>(blocksums), s, tail);
 }
 
-cudaError_t exclusive_scan_i32(const int32_t* in, int32_t* out, int n, int32_t* blocksums, cudaStream_t s) {
-  return exclusive_scan<int32_t, int>(in, out, n, blocksums, s);
+cudaError_t exclusive_scan_i32(const int32_t* in, int32_t* out, int n, int32_t* blocksums, cudaStream_t s,
+                               const ScanTail& tail) {
+  return exclusive_scan<int32_t, int>(in, out, n, blocksums, s, tail);
 }
 
-cudaError_t check_csc(int n, const int32_t* cp, const int32_t* ri, int64_t nnz, uint32_t* status, cudaStream_t s) {
+cudaError_t check_csc(int n, const CscCheck& c, uint32_t* status, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  check_csc_kernel<<<ceil_div(n, 256), 256, 0, s>>>(n, cp, ri, nnz, status);
+  check_csc_kernel<<<dim3(ceil_div(n, 256), c.count), 256, 0, s>>>(n, c, status);
   DIAF_COUNT_LAUNCH();
   return cudaGetLastError();
 }

@@ -50,7 +50,38 @@ struct PlanArgs {
 // Host-side launches (plan.cu).
 cudaError_t plan_count(const PlanArgs& a, cudaStream_t s);
 cudaError_t plan_rows(const PlanArgs& a, cudaStream_t s);
-cudaError_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int n, int64_t* blocksums, cudaStream_t s);
-cudaError_t exclusive_scan_i32(const int32_t* in, int32_t* out, int n, int32_t* blocksums, cudaStream_t s);
+// What the last block of a scan leaves for the host beside out[n].
+struct ScanTail {
+  void* total = nullptr;                // the total again (the scan's output type)
+  const uint32_t* status = nullptr;     // copied to status_copy
+  uint32_t* status_copy = nullptr;
+};
+cudaError_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int n, int64_t* blocksums, cudaStream_t s,
+                                      const ScanTail& tail = ScanTail());
+cudaError_t exclusive_scan_i32(const int32_t* in, int32_t* out, int n, int32_t* blocksums, cudaStream_t s,
+                               const ScanTail& tail = ScanTail());
 int scan_blocksums_size(int n);
-cudaError_t check_csc(int n, const int32_t* cp, const int32_t* ri, int64_t nnz, uint32_t* status, cudaStream_t s);
+struct CscCheck {  // up to three column structures of n columns, checked in one launch
+  int count = 0;
+  const int32_t* cp[3];
+  const int32_t* ri[3];
+  int64_t nnz[3];
+  void add(const int32_t* colptr, const int32_t* rowidx, int64_t entries) {
+    cp[count] = colptr;
+    ri[count] = rowidx;
+    nnz[count++] = entries;
+  }
+};
+cudaError_t check_csc(int n, const CscCheck& c, uint32_t* status, cudaStream_t s);
+// The symbolic pass's counters, one block: the host reads it with one copy per
+// synchronisation (a copy of a few bytes to pageable memory holds the host
+// until it is done; five such copies and six more launches made set-up and
+// first solve of the 32^2 convection-diffusion problem 353 us, now 311 us).
+struct PlanCounters {
+  int64_t Etot;
+  int32_t stats[4];
+  int32_t bucket_count[kNumBuckets];
+  int32_t big_count;
+  int32_t nnzv;
+  uint32_t status;
+};
