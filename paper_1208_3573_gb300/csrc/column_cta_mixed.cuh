@@ -354,6 +354,10 @@ constexpr int kClusterMax = 4;  // most singular values of a close cluster resol
 // quadratic: the next sweep would rotate nothing).  A round is a chain of
 // shared loads, three shuffle sums, a square root and a division between two
 // barriers; the number of threads per pair is set by k_j <= 64 and 256 threads.
+// The fused multiply-adds are spelled out, not left to the compiler: they give
+// cta_jacobi's bits.  Where the gap to the next singular value is small, the one
+// or two corrections that follow leave a trace of the FP32 basis's last bits in
+// w (up to 1e-7), and which bits those are should not change with the build.
 template <int KP>
 __device__ int cta_jacobi_mixed(float* G, int k, float* V, float* redF) {
   constexpr int LPP = kCtaThreads / (kCtaKmax / 2), NR = kCtaKmax / LPP;
@@ -418,16 +422,16 @@ __device__ int cta_jacobi_mixed(float* G, int k, float* V, float* redF) {
             }
           const float ag = sc_abs(ga), eph = sc_unit(ga);
           const float d = be - al;
-          const float t = copysign(2.0f * ag, d) / (fabs(d) + sqrt(d * d + 4.0f * ag2));
+          const float t = copysign(2.0f * ag, d) / (fabs(d) + sqrt(fmaf(d, d, __fmul_rn(4.0f, ag2))));
           const float cs = rsqrt_r(1.0f + t * t), sn = cs * t;
 #pragma unroll
           for (int i = 0; i < NR; ++i)
             if (i * LPP < k && i * LPP + sub < k) {
               const float yi = eph * y[i], wi = eph * vy[i];
-              ca[i * LPP] = cs * x[i] - sn * yi;
-              cb[i * LPP] = sn * x[i] + cs * yi;
-              va[i * LPP] = cs * vx[i] - sn * wi;
-              vb[i * LPP] = sn * vx[i] + cs * wi;
+              ca[i * LPP] = fmaf(cs, x[i], -__fmul_rn(sn, yi));
+              cb[i * LPP] = fmaf(sn, x[i], __fmul_rn(cs, yi));
+              va[i * LPP] = fmaf(cs, vx[i], -__fmul_rn(sn, wi));
+              vb[i * LPP] = fmaf(sn, vx[i], __fmul_rn(cs, wi));
             }
         }
         a0 = a0 + 1 == qq - 1 ? 0 : a0 + 1;
