@@ -52,8 +52,8 @@ enum { DIAF_F64 = 0, DIAF_C128 = 1 };
 enum { DIAF_ALG_Q = 1, DIAF_ALG_S = 2 };
 
 /* Arithmetic of the numeric phase.  DIAF_PREC_FP64: everything in FP64
- * (complex128 for DIAF_C128).  DIAF_PREC_MIXED32: QR, leverage keys and
- * Jacobi in FP32 (complex64) on an FP64 tile, then an FP64 refinement of
+ * (complex128 for DIAF_C128).  DIAF_PREC_MIXED32: factors, leverage keys and
+ * singular vectors in FP32 (complex64) on an FP64 tile, then an FP64 refinement of
  * (w_j, v_j) against the FP64 tile and an FP64 residual.  A column whose FP32
  * leverage decision lies within the FP32 error bound of its threshold gets
  * its leverage keys recomputed in FP64 (the FP64 path's own QR and key

@@ -29,9 +29,10 @@
 // k^2 / 2 rotations of 6 k flops for them; the two inverses cost k^3 each and
 // a correction 6 k^2, all of it independent multiply-adds.  (LDL^* factors
 // with triangular solves have half the arithmetic, but every solve is a chain
-// of 2 k dependent shuffles.)  Numeric pass before and after, on one GB300:
-// lognormal 64^3 (k = 25) 65.8 -> 33.7 ms, FP64 convection-diffusion 129^2
-// (k = 13) 11.3 -> 2.4 ms, complex Helmholtz 512^2 (k = 9) 13.3 -> 12.4 ms.
+// of 2 k dependent shuffles.)  Numeric pass before and after, on one GB300,
+// with the Gram matrices and FP64 products over the rows' nonzeros: lognormal
+// 64^3 (k = 25) 65.8 -> 16.3 ms, FP64 convection-diffusion 129^2 (k = 13)
+// 11.3 -> 2.4 ms, complex Helmholtz 512^2 (k = 9) 13.3 -> 9.4 ms.
 // What bounds it now is latency: three to four warps per scheduler on chains
 // of shuffles and shared-memory reads.
 #pragma once
