@@ -685,6 +685,7 @@ diaf_status symbolic_pass(const diaf_csc* A, const diaf_pattern* PW, const diaf_
     np.cta_grid_mixed = np.mixed ? cta_columns_grid_mixed(A->dtype, alg, np.cs.ldm, np.h_bc[bl]) : 0;
     const int slabs = np.cta_grid > np.cta_grid_mixed ? np.cta_grid : np.cta_grid_mixed;
     nc.add((char**)&np.cs.slab, (size_t)slabs * 2 * np.cs.ldm * np.cs.kcap * esz);
+    static_assert(kCtaGather == kMaxGather, "the planner refuses columns with more entries");
     if (np.cta_grid_mixed > 0) nc.add(&np.cs.eloc, (size_t)np.cta_grid_mixed * kCtaGather);
   }
   if (!nc.reqs.empty()) DIAF_CU(pool.carve(nc));  // the numeric pass's scratch, one allocation

@@ -198,42 +198,6 @@ __device__ void cta_upper_inverse_scaled(const float* Rsm, int ldr, int k, const
   __syncthreads();
 }
 
-// Greedy V rule of Sec. 3.1 on the keys hk (as select_rows_greedy, at CTA
-// level): s picks among the admissible rows, ties within tau to the lower row.
-// Returns the smallest distance of a non-leading candidate key from a
-// threshold it was compared with (the FP32 decision margin).
-__device__ inline double cta_select_rows(const int32_t* rs, const double* hk, int32_t* pick, int m, int rule, int j,
-                                         int s, double tau, double* red, const int32_t* blk) {
-  const int tid = threadIdx.x;
-  double margin = DBL_MAX;
-  for (int t = 0; t < s; ++t) {
-    double hm = -DBL_MAX;
-    for (int r = tid; r < m; r += kCtaThreads)
-      if (!pick[r] && admissible_row(rule, rs[r], j, blk)) hm = dmax(hm, hk[r]);
-    hm = block_max(hm, red);
-    int rmax = INT_MAX;
-    for (int r = tid; r < m; r += kCtaThreads)
-      if (!pick[r] && admissible_row(rule, rs[r], j, blk) && hk[r] == hm) rmax = dmin(rmax, r);
-    rmax = block_min(rmax, reinterpret_cast<int*>(red));
-    const double thr = hm - tau;
-    int best = INT_MAX;
-    for (int r = tid; r < m; r += kCtaThreads)
-      if (!pick[r] && admissible_row(rule, rs[r], j, blk)) {
-        if (r != rmax) margin = dmin(margin, fabs(hk[r] - thr));
-        if (hk[r] >= thr) best = dmin(best, r);
-      }
-    best = block_min(best, reinterpret_cast<int*>(red));
-    if (best == INT_MAX) {  // no key reaches the threshold (non-finite keys): the lowest remaining admissible row
-      for (int r = tid; r < m; r += kCtaThreads)
-        if (!pick[r] && admissible_row(rule, rs[r], j, blk)) best = dmin(best, r);
-      best = block_min(best, reinterpret_cast<int*>(red));
-    }
-    if (tid == 0 && best < m) pick[best] = 1;
-    __syncthreads();
-  }
-  return block_min(margin, red);
-}
-
 // column norms of the m x k FP32 tile (warp per column)
 __device__ inline void cta_col_norms_f(const float* T, int ld, int m, int k, double* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
