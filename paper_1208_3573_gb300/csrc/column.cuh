@@ -33,6 +33,17 @@ constexpr double kMixedDeltaScale = DIAF_MIXED_DELTA_SCALE;
 // the Gram paths of the mixed kernels are used only up to this column-scaled
 // kappa (the Householder QR otherwise).
 constexpr float kGramKappaMax = 30.0f;
+// Column norms outside these leave FP32: their squares, sums and reciprocals
+// would not all be normal numbers.
+constexpr float kColNormMin = 0x1p-55f, kColNormMax = 0x1p55f;
+
+// One column's cn / |R_cc| (cn: its norm, d = |R_cc|).  Infinite, so that the
+// tile goes to FP64, when the norm is out of range or the quotient no number:
+// a NaN here would drop out of the maximum over the columns, and the keys that
+// come after it would differ between the lanes that share a decision.
+__device__ __forceinline__ float scaled_kappa(float cn, float d) {
+  return d > 0.0f && cn >= kColNormMin && cn <= kColNormMax ? cn / d : INFINITY;
+}
 
 struct ColArgs {
   int n;

@@ -626,8 +626,9 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
   if (sc.gram && m >= k) {
     int zero = 0;
     for (int c = tid; c < k; c += kCtaThreads) {
-      rf[c] = cn[c] > 0.0 ? (float)(1.0 / cn[c]) : 0.0f;
-      zero |= !(cn[c] > 0.0);
+      const bool fits = cn[c] >= kColNormMin && cn[c] <= kColNormMax;
+      rf[c] = fits ? (float)(1.0 / cn[c]) : 0.0f;
+      zero |= !fits;
     }
     if (!__syncthreads_or(zero)) {
       DIAF_PHASE(11);
@@ -665,7 +666,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     float kp = 0.0f;
     for (int c = tid; c < k; c += kCtaThreads) {
       const float d = fabsf(Rs[c + c * KP]);
-      kp = fmaxf(kp, d > 0.0f ? (float)cn[c] / d : INFINITY);
+      kp = fmaxf(kp, scaled_kappa((float)cn[c], d));
       rinv[c] = d > 0.0f ? 1.0f / Rs[c + c * KP] : 0.0f;
     }
     kap = block_max(kp, redF);
@@ -829,7 +830,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     float kh = 0.0f;
     for (int c = tid; c < k; c += kCtaThreads) {  // exact zero columns of A-hat: exact zero singular values
       const float d = fabsf(Tw[c + (size_t)c * ld]);
-      kh = fmaxf(kh, d > 0.0f ? (float)cn[c] / d : (cn[c] > 0.0 ? INFINITY : 0.0f));
+      kh = fmaxf(kh, d > 0.0f || cn[c] > 0.0 ? scaled_kappa((float)cn[c], d) : 0.0f);
     }
     if (!(block_max(kh, redF) <= kMixedKappaMax)) { CTA_FB(2); return false; }
     for (int i = tid; i < k * k; i += kCtaThreads) {

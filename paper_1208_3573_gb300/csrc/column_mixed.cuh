@@ -110,8 +110,11 @@ __device__ bool warp_gram_cholesky(const float* W, int m, int k, float* Rs, doub
 // FP32 leverage keys of the real m x k tile W (m >= k; leading dimension LDT;
 // rowmask: the columns that the lane's rows have) from its Gram matrix's
 // inverse: hk[r] = w_r^T (W^T W)^-1 w_r.  Ms: KP x KMAX scratch, buf: 2 KMAX,
-// 16-byte aligned.  False (uniformly) unless the column-scaled kappa is at
-// most kGramKappaMax; *kap2 receives its square.
+// 16-byte aligned.  False (uniformly: every lane's column is tested by itself
+// and the warp votes) unless the column norms are in FP32's range and the
+// column-scaled kappa is at most kGramKappaMax; *kap2 receives its square.  An
+// entry whose square overflows makes its column's pivot and norm infinite and
+// their quotient a NaN, which a maximum over the lanes keeps in one lane only.
 template <int KMAX, int MMAX, int LDT, int KP>
 __device__ bool warp_gram_keys(const float* W, const uint32_t (&rowmask)[MMAX / DIAF_WARP], float* Ms, float* buf,
                                float* hk, int m, int k, int lane, float* kap2) {
@@ -121,9 +124,10 @@ __device__ bool warp_gram_keys(const float* W, const uint32_t (&rowmask)[MMAX / 
   const float hqq = lane < k ? Ms[lane + lane * KP] : 0.0f;
   float piv = 1.0f, scale = 1.0f;
   warp_sweep_inverse<float, KMAX, KP>(Ms, 0.0f, k, acc, buf, lane, &piv, &scale);
-  const float k2 = warp_max(lane < k ? (piv > 0.0f ? hqq / piv : INFINITY) : 0.0f);
-  if (!(k2 <= kGramKappaMax * kGramKappaMax)) return false;
-  *kap2 = k2;
+  const bool fits = piv > 0.0f && hqq <= kGramKappaMax * kGramKappaMax * piv && hqq >= kColNormMin * kColNormMin &&
+                    hqq <= kColNormMax * kColNormMax;
+  if (!__all_sync(DIAF_FULL, lane >= k || fits)) return false;
+  *kap2 = warp_max(lane < k ? hqq / piv : 0.0f);
   if (lane < k) {
 #pragma unroll
     for (int i = 0; i < KMAX; ++i)
@@ -304,8 +308,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
   }
   DIAF_PHASE(2);
   for (int c = lane; c < k; c += DIAF_WARP) {
-    float d = (float)sc_abs(Rs[c + c * KP]);
-    kap = fmaxf(kap, d > 0.0f ? (float)cn[c] / d : INFINITY);
+    kap = fmaxf(kap, scaled_kappa((float)cn[c], (float)sc_abs(Rs[c + c * KP])));
   }
   kap = warp_max(kap);
   if (!(kap <= kMixedKappaMax)) { hand_back(1); return; }
@@ -414,7 +417,7 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     float kh = 0.0f;
     for (int c = lane; c < k; c += DIAF_WARP) {
       const float d = (float)sc_abs(Rs[c + c * KP]);
-      kh = fmaxf(kh, d > 0.0f ? (float)cn[c] / d : (cn[c] > 0.0 ? INFINITY : 0.0f));
+      kh = fmaxf(kh, d > 0.0f || cn[c] > 0.0 ? scaled_kappa((float)cn[c], d) : 0.0f);
     }
     kh = warp_max(kh);
     if (!(kh <= kMixedKappaMax)) { hand_back(3); return; }

@@ -330,7 +330,7 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
     rinv[q] = 0.0f;
     if (q < k) {
       const float d = QS(W, q + q * m);
-      kap = fmaxf(kap, fabsf(d) > 0.0f ? cn[q] / fabsf(d) : INFINITY);
+      kap = fmaxf(kap, scaled_kappa(cn[q], fabsf(d)));
       rinv[q] = __fdividef(1.0f, d);
     }
   }

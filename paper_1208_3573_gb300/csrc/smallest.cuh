@@ -293,7 +293,7 @@ __device__ bool warp_smallest_vector(const SD* Ts, const int32_t* inI, S* Tw,
   R piv = R(1), scale = R(1);
   warp_sweep_inverse<S, KMAX, KP>(Hs, R(0), k, inv, buf, lane, &piv, &scale);
   constexpr R kmax = smallest_kappa_max<R>();
-  if (!__all_sync(DIAF_FULL, lane >= k || (piv > R(0) && hqq <= kmax * kmax * piv))) return false;
+  if (!__all_sync(DIAF_FULL, lane >= k || (isfinite(hqq) && piv > R(0) && hqq <= kmax * kmax * piv))) return false;
   S x = lane < k ? sc_real_s<S>(R((lane * 37 + 11) % 17) - R(8.3)) : sc_zero<S>();
   R d = R(0);
 #pragma unroll 1
