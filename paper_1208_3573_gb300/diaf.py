@@ -533,7 +533,11 @@ ONE_PASS_KEEP = 64
 
 def sparsified_powers(A: DeviceCSC, k: int = 2, p_l: int = 0, keep: int = 0, stream=None) -> DeviceCSC:
     """W pattern by sparsified powers (diaf_sparsified_rows / _pack when at most
-    ONE_PASS_KEEP entries per column are kept, else diaf_sparsified_count / _fill)."""
+    ONE_PASS_KEEP entries per column are kept, else diaf_sparsified_count / _fill).
+
+    On a stream other than the current one the work starts after what the current
+    stream has enqueued, and is done when this returns: the arrays are the current
+    stream's, which knows nothing of the other."""
     L = lib()
     a = A.csc_t()
     s = _stream(stream)
@@ -541,6 +545,11 @@ def sparsified_powers(A: DeviceCSC, k: int = 2, p_l: int = 0, keep: int = 0, str
     colptr = torch.empty(A.n + 1, dtype=torch.int32, device=dev)
     nnz = ctypes.c_int64()
     one_pass = 1 <= keep <= ONE_PASS_KEEP
+    current = torch.cuda.current_stream(dev)
+    side = None
+    if s != current.cuda_stream:
+        side = torch.cuda.ExternalStream(s, device=dev) if s else torch.cuda.default_stream(dev)
+        side.wait_stream(current)
     if one_pass:
         rows = torch.empty(max(A.n * keep, 1), dtype=torch.int32, device=dev)
         _check(L.diaf_sparsified_rows(ctypes.byref(a), k, p_l, keep, _ptr(rows), _ptr(colptr), ctypes.byref(nnz), s))
@@ -549,10 +558,10 @@ def sparsified_powers(A: DeviceCSC, k: int = 2, p_l: int = 0, keep: int = 0, str
     rowidx = torch.empty(max(int(nnz.value), 1), dtype=torch.int32, device=dev)
     if one_pass:
         _check(L.diaf_sparsified_pack(A.n, keep, _ptr(rows), _ptr(colptr), _ptr(rowidx), s))
-        if s != torch.cuda.current_stream(dev).cuda_stream:  # rows goes back to its own stream's pool
-            rows.record_stream(torch.cuda.ExternalStream(s, device=dev))
     else:
         _check(L.diaf_sparsified_fill(ctypes.byref(a), k, p_l, keep, _ptr(colptr), _ptr(rowidx), s))
+    if side is not None:
+        side.synchronize()
     return DeviceCSC(A.n, colptr, rowidx[:int(nnz.value)])
 
 
