@@ -45,6 +45,28 @@ __device__ __forceinline__ float scaled_kappa(float cn, float d) {
   return d > 0.0f && cn >= kColNormMin && cn <= kColNormMax ? cn / d : INFINITY;
 }
 
+// The unit of a tile in mixed precision.  The mixed kernels work on 2^-e T: FP32
+// sums of squares, and the products of two of them that the Jacobi rotations and
+// the inverse iteration form, neither overflow nor lose their digits while the
+// largest entry lies in 2^kUnitMin .. 2^kUnitMax, and outside of that e is its
+// exponent (a power of two, so that every rounding stays the same; inside e = 0,
+// and nothing is done).  W (DIAF-Q) or V and the residual (DIAF-S) take 2^-e or
+// 2^e back at the end.  Without it a matrix times 1e12 lost its FP32 singular
+// vectors (1e10: rotations stop, as alpha beta overflows).
+constexpr int kUnitMin = -20, kUnitMax = 24;
+constexpr int kUnitLimit = 900;  // beyond 2^+-900 the FP64 kernel takes the column
+
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// |x| as its upper 32 bits (exponent and leading digits): integers in the same order
+__device__ __forceinline__ uint32_t top_word(double x) { return __double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t top_word(Cx<double> x) { return max(top_word(x.re), top_word(x.im)); }
+// e from the tile's largest top_word; false: not finite, zero or beyond the limit.
+__device__ __forceinline__ bool tile_unit(uint32_t top, int* e) {
+  const int x = (int)(top >> 20) - 1023;
+  *e = x < kUnitMin || x > kUnitMax ? x : 0;
+  return x >= -kUnitLimit && x <= kUnitLimit;
+}
+
 struct ColArgs {
   int n;
   const int32_t* Acp;
@@ -102,7 +124,7 @@ struct ColumnIdx {
   int32_t* Iloc;  // tile row of Is[t] or -1
   int32_t* cst;   // column starts of J_j in A (KMAX)
   int32_t* coff;  // exclusive offsets of the gathered entries (KMAX)
-  int32_t* misc;  // [0] = position of j in I_j
+  int32_t* misc;  // [0] = position of j in I_j, [1] = exponent of the tile's unit (mixed form)
 };
 template <int KMAX, int MMAX>
 constexpr size_t idx_bytes() { return sizeof(int32_t) * (5 * MMAX + 2 * KMAX + 8); }
@@ -122,8 +144,9 @@ __device__ ColumnIdx carve_idx(int32_t* base) {
 }
 
 // Loads R_j and gathers T = A(R_j, J_j) (zero padded to me rows) into Ts.
+// Returns the largest top_word of the lane's entries.
 template <class SD, int KMAX, int MMAX, int LDT>
-__device__ void gather_tile(const ColArgs& a, int j, int k, int m, int me, SD* Ts, const ColumnIdx& ix, int lane) {
+__device__ uint32_t gather_tile(const ColArgs& a, int j, int k, int m, int me, SD* Ts, const ColumnIdx& ix, int lane) {
   const int32_t* Rj = a.rows + a.Eoff[j];
   const int32_t* J = a.Wri + a.Wcp[j];
   const SD* Av = reinterpret_cast<const SD*>(a.Av);
@@ -148,14 +171,18 @@ __device__ void gather_tile(const ColArgs& a, int j, int k, int m, int me, SD* T
   if (lane < k) ix.coff[lane] = incl - len;
   const int E = __shfl_sync(DIAF_FULL, incl, 31);
   __syncwarp();
+  uint32_t top = 0;
   for (int e = lane; e < E; e += DIAF_WARP) {
     int q = 0;
     while (q + 1 < k && ix.coff[q + 1] <= e) ++q;
     int p = ix.cst[q] + (e - ix.coff[q]);
     int r = lower_bound_i32(ix.rs, m, a.Ari[p]);
-    Ts[r + q * LDT] = Av[p];
+    const SD v = Av[p];
+    top = max(top, top_word(v));
+    Ts[r + q * LDT] = v;
   }
   __syncwarp();
+  return top;
 }
 
 // Greedy selection of s admissible rows by key hk (Sec. 3.1 with ties within
@@ -285,11 +312,13 @@ __device__ inline int build_I(const ColArgs& a, int j, int m, int l, const Colum
 
 // Phase (v_jj real >= 0, else the largest |w_q| real), residual
 // ||A_j w - v|| (r2_known >= 0: its square, known to the caller), finiteness,
-// and the scatter of column j.
+// and the scatter of column j.  wexp, vexp: W's and V's powers of two (the
+// tile's unit; the residual has V's).
 template <class SD, int LDT>
 __device__ void finish_column(const ColArgs& a, int j, int k, int m, int l, int jpos, const SD* Ts, SD* wv, SD* vv,
                               const ColumnIdx& ix, uint32_t flags, bool do_phase, int lane,
-                              double rank_thr = -1.0, double r2_known = -1.0, bool given = false) {
+                              double rank_thr = -1.0, double r2_known = -1.0, bool given = false, int wexp = 0,
+                              int vexp = 0) {
   using R = RealOf<SD>;
   if (do_phase) {
     SD ph = sc_real_s<SD>(R(1));
@@ -329,8 +358,13 @@ __device__ void finish_column(const ColArgs& a, int j, int k, int m, int l, int 
       if (ix.Iloc[t] < 0) r2 += sc_abs2(vv[t]);
     r2 = warp_sum(r2);
   }
-  const double resj = sqrt((double)r2);
+  double resj = sqrt((double)r2);
   if (resj <= rank_thr) flags |= DIAF_FLAG_RANK_DEFICIENT;  // DIAF-S: res = ||A-hat w|| = sigma_min
+  if (wexp != 0 || vexp != 0) {  // uniform
+    resj *= pow2(vexp);
+    for (int q = lane; q < k; q += DIAF_WARP) wv[q] = R(pow2(wexp)) * wv[q];
+    for (int t = lane; t < l; t += DIAF_WARP) vv[t] = R(pow2(vexp)) * vv[t];
+  }
   bool finite = isfinite(resj);
   for (int q = lane; q < k; q += DIAF_WARP) finite &= isfinite(sc_real(wv[q])) && isfinite(sc_imag(wv[q]));
   for (int t = lane; t < l; t += DIAF_WARP) finite &= isfinite(sc_real(vv[t])) && isfinite(sc_imag(vv[t]));

@@ -405,11 +405,12 @@ struct CtaSmem {
 // Phase (v_jj real >= 0), residual ||A w_j - v_j|| from its definition (in
 // the tile's precision), NaN/Inf check and scatter of column j -- the end of
 // every CTA column kernel.  rank_thr: a residual at or below it marks the
-// column RANK_DEFICIENT (DIAF-S, where res = ||A-hat w|| = sigma_min).
+// column RANK_DEFICIENT (DIAF-S, where res = ||A-hat w|| = sigma_min).  vexp:
+// the power of two of V and the residual (the tile's unit).
 template <class S>
 __device__ void cta_finish(const ColArgs& a, int j, int k, int m, int l, int jpos, const S* Ts, int ld, S* wv, S* vv,
                            const int32_t* Is, const int32_t* Iloc, const int32_t* inI, uint32_t flags, bool do_phase,
-                           RealOf<S>* redR, double rank_thr = -1.0, double r2_known = -1.0) {
+                           RealOf<S>* redR, double rank_thr = -1.0, double r2_known = -1.0, int vexp = 0) {
   using R = RealOf<S>;
   const int tid = threadIdx.x;
   if (do_phase) {
@@ -449,8 +450,12 @@ __device__ void cta_finish(const ColArgs& a, int j, int k, int m, int l, int jpo
       if (Iloc[t] < 0) r2 += sc_abs2(vv[t]);
     r2 = block_sum(r2, redR);
   }
-  const double resj = sqrt((double)r2);
+  double resj = sqrt((double)r2);
   if (resj <= rank_thr) flags |= DIAF_FLAG_RANK_DEFICIENT;
+  if (vexp != 0) {
+    resj *= pow2(vexp);
+    for (int t = tid; t < l; t += kCtaThreads) vv[t] = R(pow2(vexp)) * vv[t];
+  }
   int bad = !isfinite(resj);
   for (int q = tid; q < k; q += kCtaThreads) bad |= !(isfinite(sc_real(wv[q])) && isfinite(sc_imag(wv[q])));
   for (int t = tid; t < l; t += kCtaThreads) bad |= !(isfinite(sc_real(vv[t])) && isfinite(sc_imag(vv[t])));

@@ -220,6 +220,7 @@ struct CtaEntries {
   const uint16_t* eloc;
   const uint32_t* rm;
   int E;
+  int unit;  // exponent of the tile's unit (A's values are in their own)
 };
 
 // (T x)_r over row r's entries, columns ascending.
@@ -254,7 +255,7 @@ __device__ inline void cta_hat_gram_apply(const CtaEntries& en, const double* Ts
   }
   gq += shfl_xor(gq, 1);
   gq += shfl_xor(gq, 2);
-  if (q < k && sub == 0) g[q] = gq;
+  if (q < k && sub == 0) g[q] = en.unit != 0 ? pow2(-en.unit) * gq : gq;
   __syncthreads();
 }
 
@@ -570,7 +571,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
   int32_t* Iloc = Is + mcap;
   int32_t* cst = Iloc + mcap;
   int32_t* coff = cst + kCtaKmax;
-  int32_t* misc = coff + kCtaKmax;  // [0] jpos, [1] count
+  int32_t* misc = coff + kCtaKmax;  // [0] jpos, [1] count, [2 ..] close cluster, [6] sigma_min, [7] largest top_word
   uint16_t* eloc = sc.eloc + (size_t)blockIdx.x * kCtaGather;
   float* redF = reinterpret_cast<float*>(red);
 
@@ -600,19 +601,28 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     pick[r] = 0;
   }
   for (size_t i = tid; i < (size_t)me * k; i += kCtaThreads) Ts[(i % me) + (i / me) * ld] = 0.0;
+  if (tid == 0) misc[7] = 0;
   cta_gather_offsets(a.Acp, J, k, cst, coff, misc + 1);
   __syncthreads();
   const int E = misc[1];
+  uint32_t top = 0;
   for (int e = tid; e < E; e += kCtaThreads) {
     const int q = upper_bound_i32(coff, k, e) - 1;
     const int p = cst[q] + (e - coff[q]);
     const int r = lower_bound_i32(rs, m, a.Ari[p]);
-    Ts[r + (size_t)q * ld] = Av[p];
+    const double v = Av[p];
+    top = max(top, top_word(v));
+    Ts[r + (size_t)q * ld] = v;
     eloc[e] = (uint16_t)r;
   }
+  top = __reduce_max_sync(DIAF_FULL, top);
+  if (lane == 0) atomicMax(&misc[7], (int)top);
   __syncthreads();
+  int unit;
+  if (!tile_unit((uint32_t)misc[7], &unit)) { CTA_FB(0); return false; }
   for (size_t i = tid; i < (size_t)me * k; i += kCtaThreads) {
     const size_t o = (i % me) + (i / me) * ld;
+    if (unit != 0) Ts[o] *= pow2(-unit);
     Tw[o] = (float)Ts[o];
   }
   __syncthreads();
@@ -772,7 +782,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
     for (int e = c < k ? coff[c] + (tid & 3) : 0; e < e1; e += 4) atomicOr(&rm[2 * eloc[e] + (c >> 5)], 1u << (c & 31));
   }
   __syncthreads();
-  const CtaEntries en{Av, cst, coff, eloc, rm, E};
+  const CtaEntries en{Av, cst, coff, eloc, rm, E, unit};
   // ---- R-hat: from G on the Gram path (G minus the I_j rows' outer
   // products, Cholesky of its column-scaled form), else FP32 QR of A-hat
   bool gram_hat = false;
@@ -784,7 +794,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
       if (c < k) {
         const int e1 = c + 1 < k ? coff[c + 1] : E;
         for (int e = coff[c] + (tid & 3); e < e1 && !nz; e += 4)
-          nz = inI[eloc[e]] < 0 && (float)Av[cst[c] + (e - coff[c])] != 0.0f;
+          nz = inI[eloc[e]] < 0 && (float)Ts[eloc[e] + (size_t)c * ld] != 0.0f;
       }
       const unsigned any = __ballot_sync(0xffffffffu, nz) >> (tid & 28) & 15u;
       zc = c < k && any == 0u;
@@ -961,7 +971,7 @@ __device__ bool solve_column_cta_mixed(const ColArgs& a, const CtaScratch& sc, i
   }
   r2 = block_sum(r2, red);
   cta_finish<double>(a, j, k, m, l, jpos, Ts, ld, wv, vv, Is, Iloc, inI, flags, true, red,
-                     1e-14 * smax, r2);
+                     1e-14 * smax, r2, unit);
   DIAF_PHASE(9);
   return true;
 }

@@ -254,7 +254,18 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
   }
 
   DIAF_PHASE_START();
-  gather_tile<SD, KMAX, MMAX, LDT>(a, j, k, m, me, Ts, ix, lane);
+  {
+    const uint32_t top = __reduce_max_sync(DIAF_FULL, gather_tile<SD, KMAX, MMAX, LDT>(a, j, k, m, me, Ts, ix, lane));
+    int unit;
+    if (!tile_unit(top, &unit)) { hand_back(1); return; }
+    if (lane == 0) ix.misc[1] = unit;
+    if (unit != 0)
+      for (int i = lane; i < me * k; i += DIAF_WARP) {
+        SD& t = Ts[(i % me) + (i / me) * LDT];
+        t = RealOf<SD>(pow2(-unit)) * t;
+      }
+    __syncwarp();
+  }
   DIAF_PHASE(0);
 
   // ---- the keys of wide real tiles from the inverse of T's Gram matrix: h_r =
@@ -673,7 +684,9 @@ __device__ void solve_column_mixed(const ColArgs& a, int j, unsigned char* smem,
     }
   }
   DIAF_PHASE(9);
-  finish_column<SD, LDT>(a, j, k, m, l, jpos, Ts, wv, vv, ix, flags, true, lane, rank_thr, r2_known);
+  const int unit = ix.misc[1];
+  finish_column<SD, LDT>(a, j, k, m, l, jpos, Ts, wv, vv, ix, flags, true, lane, rank_thr, r2_known, false,
+                         ALG == DIAF_ALG_Q ? -unit : 0, ALG == DIAF_ALG_Q ? 0 : unit);
   DIAF_PHASE(10);
 }
 

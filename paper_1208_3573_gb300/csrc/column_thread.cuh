@@ -286,6 +286,7 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
       }
   }
   __syncwarp(qm);
+  uint32_t top = 0;
   for (int q = 0; q < k; ++q) {
     const int2 be = CR(q);
     for (int p = be.x + sub; p < be.y; p += 4) {
@@ -301,11 +302,25 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
         }
       }
       const double v = Av[p];
+      top = max(top, top_word(v));
       G[((r >> 2) * KMAX + q) * gstride + (r & 3)] = v;
       QS(W, r + q * m) = (float)v;
     }
   }
+  top = max(top, __shfl_xor_sync(qm, top, 1));
+  top = max(top, __shfl_xor_sync(qm, top, 2));
   __syncwarp(qm);
+  int unit;
+  if (!tile_unit(top, &unit)) { defer(); return; }
+  if (unit != 0) {
+    for (int q = 0; q < k; ++q)
+      for (int r = sub; r < m; r += 4) {
+        double& g = G[((r >> 2) * KMAX + q) * gstride + (r & 3)];
+        g *= pow2(-unit);
+        QS(W, r + q * m) = (float)g;
+      }
+    __syncwarp(qm);
+  }
   float cn[KMAX];
 #pragma unroll
   for (int q = 0; q < KMAX; ++q) {
@@ -740,12 +755,13 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
     ph = wsel < 0.0 ? -1.0 : 1.0;
   }
   bool finite = true;
+  const double pv = copysign(pow2(unit), ph);
   for (int t = 0; t < nown; ++t) {
     const int r = sub + 4 * t;
     if ((inI >> r) & 1u) {
       const int pos = pos_of(r);
-      const double vt = Vout[pos];
-      Vout[pos] = ph * vt;
+      const double vt = pv * Vout[pos];
+      Vout[pos] = vt;
       finite &= isfinite(vt);
     }
   }
@@ -763,7 +779,7 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
   const unsigned fin = __ballot_sync(qm, finite) & qm;
   if (fin != qm) flags |= DIAF_FLAG_NONFINITE;
   if (sub == 0) {
-    a.res[j] = resj;
+    a.res[j] = unit != 0 ? pow2(unit) * resj : resj;
     a.flags[j] = flags | a.extra_flags;
   }
   if (a.Hri) {  // the final I_j to the host (the rows as written above), then the column's word
