@@ -57,9 +57,6 @@ constexpr int kUnitMin = -20, kUnitMax = 24;
 constexpr int kUnitLimit = 900;  // beyond 2^+-900 the FP64 kernel takes the column
 
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-// |x| as its upper 32 bits (exponent and leading digits): integers in the same order
-__device__ __forceinline__ uint32_t top_word(double x) { return __double2hiint(x) & 0x7fffffffu; }
-__device__ __forceinline__ uint32_t top_word(Cx<double> x) { return max(top_word(x.re), top_word(x.im)); }
 // e from the tile's largest top_word; false: not finite, zero or beyond the limit.
 __device__ __forceinline__ bool tile_unit(uint32_t top, int* e) {
   const int x = (int)(top >> 20) - 1023;

@@ -113,6 +113,10 @@ template <> __device__ __forceinline__ Cx<float> sc_cast<Cx<float>, Cx<double>>(
 template <> __device__ __forceinline__ Cx<double> sc_cast<Cx<double>, Cx<float>>(Cx<float> a) { return {(double)a.re, (double)a.im}; }
 template <> __device__ __forceinline__ Cx<float> sc_cast<Cx<float>, Cx<float>>(Cx<float> a) { return a; }
 
+// |x| as its upper 32 bits (exponent and leading digits): integers in the same order
+__device__ __forceinline__ uint32_t top_word(double x) { return __double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t top_word(Cx<double> x) { return max(top_word(x.re), top_word(x.im)); }
+
 // 16 bytes of scalars, for vector loads
 template <class S>
 struct alignas(16) Pack16 {

@@ -67,6 +67,20 @@ __device__ __forceinline__ SD tile_adj_mul(const SD* Ts, const SD* zz, int m, in
   return g;
 }
 
+// x in the working type; what underflows there becomes its smallest number, not
+// zero: the FP64 products go by the places that are not zero.
+template <class S, class SD>
+__device__ __forceinline__ S cast_keep(SD x) {
+  if constexpr (std::is_same<S, SD>::value) {
+    return x;
+  } else if constexpr (ScalarInfo<SD>::cplx) {
+    return {cast_keep<float>(x.re), cast_keep<float>(x.im)};
+  } else {
+    const float v = (float)x;
+    return v == 0.0f && (top_word(x) | __double2loint(x)) != 0u ? __uint_as_float(1u) : v;
+  }
+}
+
 // Copies the tile to the working type (rows in I_j as zeros when inI is given)
 // and notes which columns each of the lane's rows (lane + 32u) has, all of
 // them, I_j's too.
@@ -80,7 +94,7 @@ __device__ __forceinline__ void copy_tile(const SD* Ts, const int32_t* inI, S* T
     if (r < m) {
       const bool out = inI && inI[r] >= 0;
       for (int c = 0; c < k; ++c) {
-        const S v = sc_cast<S>(Ts[r + c * LDT]);
+        const S v = cast_keep<S>(Ts[r + c * LDT]);
         if (sc_real(v) != RealOf<S>(0) || sc_imag(v) != RealOf<S>(0)) rowmask[u] |= 1u << c;
         Tw[r + c * LDT] = out ? sc_zero<S>() : v;
       }
