@@ -62,6 +62,11 @@ __device__ __forceinline__ float scaled(double x, double r, double d) {
   return d > 0.0 ? (float)(r > 1e-300 && r < 1e300 ? x * r : x / d) : 0.0f;
 }
 
+// A difference of two logarithms keeps its absolute error (up to 1e-13 for
+// diagonals near 1e300), which is below FP32's rounding of it from 1e-4 on; for
+// nearer diagonals f4 comes from their difference.
+constexpr uint32_t kLogNear = 0x3f1a36e2u;  // top_word(1e-4)
+
 // Features of candidate c of column j (one warp per column; lane l takes the
 // candidates l, l + 32, l + 64, l + 96):
 //   f0 diagonal (c == j)            f1 c is a row of A(:,j)
@@ -72,7 +77,8 @@ __device__ __forceinline__ float scaled(double x, double r, double d) {
 // What bounded it was the one FP64 pipe (an instruction per 64 cycles and
 // sub-core): square roots of squares, three divisions and a logarithm per
 // candidate.  Moduli are taken directly, the divisors' reciprocals once per
-// column, the logarithms once per row of A (f4 as their difference):
+// column, the logarithms once per row of A (f4 as their difference, but for
+// nearly equal diagonals):
 // lognormal 40^3 (64,000 columns of 25 candidates) 0.93 -> 0.42 ms.
 template <class S>
 __global__ void __launch_bounds__(kFeatWarps * 32)
@@ -161,7 +167,9 @@ __global__ void __launch_bounds__(kFeatWarps * 32)
     f[1] = acj[u] > 0.0 ? 1.0f : 0.0f;
     f[2] = scaled(acj[u], raj, aj_max);
     f[3] = scaled(a2c[u], ra2, a2max);
-    const double lr = (dc.x > 0.0 && ajj > 0.0) ? dc.y - dj.y : 0.0;
+    double lr = (dc.x > 0.0 && ajj > 0.0) ? dc.y - dj.y : 0.0;
+    if (top_word(lr) < kLogNear && __double_as_longlong(dc.x) != __double_as_longlong(ajj) && dc.x > 0.0 && ajj > 0.0)
+      lr = log1p((dc.x - ajj) / ajj);
     f[4] = (float)(lr > 10.0 ? 10.0 : (lr < -10.0 ? -10.0 : lr));
     f[5] = scaled(ajc, rjj, ajj);
     f[6] = na > 0 ? (float)(Acp[c + 1] - Acp[c]) / (float)na : 0.0f;
