@@ -699,7 +699,7 @@ __device__ void solve_column_quad(const ColArgs& a, const ThreadArgs& ta, int j,
       const double step = sqrtf(quad_dot<KU>(dx, dx, qm));
 #pragma unroll
       for (int u = 0; u < KU; ++u) xd[u] += (double)dx[u];
-      done = step * step <= 1e-14 * before;  // the next correction: about step (step / before)
+      done = step * step <= kCorrectTol * before;  // the next correction: about step (step / before)
       if (!done && it > 0 && !(step <= 0.5 * before)) { defer(); return; }
       before = step;
     }
