@@ -1161,8 +1161,6 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   const bool cplx = F->dtype == DIAF_C128;
   const size_t esz = cplx ? 16 : 8;
   const size_t nnzv = (size_t)F->nnz_v;
-  int32_t* work;
-  DIAF_CU(F->alloc(&work, n + scan_blocksums_size(n)));
   // V's structure is walked on the host (level of every row, its place in
   // its level, the numbering of every row's entries, the diagonals) -- when F
   // holds the mirror, while the numeric pass still writes V's columns there;
@@ -1203,16 +1201,67 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
     DIAF_CU(ce);
   }
   ce = cudaEventRecord(ev[0], s);
-  // W to rows, on the side stream when there is one (its own scratch)
+  // The device arrays (sizes known now; the level count is at most n), so that
+  // only copies and kernels follow the walk: what the solves keep, the
+  // preparation's scratch, V's level-ordered rows, and the packed form's arrays.
+  // The walk decides between the two forms; the other one goes back with the
+  // scratch.  Without the memory for the packed form the rows do.
+  cudaStream_t ws = side_stream();
+  LevelCsr& Vl = F->Vl;
+  int32_t *work = nullptr, *wwork = nullptr, *pos = nullptr, *dblk = nullptr;
+  uint32_t* zflag = nullptr;
+  int32_t *poff = nullptr, *moff = nullptr;
+  double* mval = nullptr;
+  void* pval = nullptr;
+  uint32_t* pflags = nullptr;
+  void *scratch = nullptr, *rows_blk = nullptr, *pack_blk = nullptr, *merge_blk = nullptr;
   F->Wr.n = n;
   F->Wr.nnz = F->nnz_w;
-  if (ce == cudaSuccess) ce = F->alloc(&F->Wr.rowptr, n + 1);
-  if (ce == cudaSuccess) ce = F->alloc(&F->Wr.colidx, F->nnz_w);
-  if (ce == cudaSuccess) ce = F->alloc((char**)&F->Wr.vals, esz * F->nnz_w);
-  cudaStream_t ws = side_stream();
-  int32_t* wwork = work;
+  Vl.n = n;
+  Vl.nnz = F->nnz_v - n;
+  if (ce == cudaSuccess) {
+    Carve kept, scr, rows;
+    kept.add(&F->Wr.rowptr, n + 1);
+    kept.add((char**)&F->Wr.vals, esz * F->nnz_w);
+    kept.add(&F->Wl.colidx, F->nnz_w);
+    kept.add(&Vl.lvlptr, n + 1);
+    kept.add((char**)&Vl.dinv, esz * n);
+    kept.add(&Vl.xrow, n);
+    kept.add((char**)&F->tbuf, esz * n);
+    scr.add(&work, n + scan_blocksums_size(n));
+    if (ws) scr.add(&wwork, n + scan_blocksums_size(n));
+    scr.add(&F->Wr.colidx, F->nnz_w);
+    scr.add(&pos, n);
+    scr.add(&dblk, blk);
+    scr.add(&zflag, 1);
+    rows.add(&Vl.rowptr, n + 1);
+    rows.add(&Vl.colidx, Vl.nnz > 0 ? Vl.nnz : 0);
+    rows.add((char**)&Vl.vals, esz * (Vl.nnz > 0 ? Vl.nnz : 0));
+    // (a real V's packed form has its merged entries' positions in the rows' place)
+    const size_t merged = cplx ? 0 : sizeof(int32_t) * kMergeEntries * n;
+    char* spare = nullptr;
+    if (merged > rows.total()) rows.add(&spare, merged - rows.total());
+    ce = F->carve(kept);
+    if (ce == cudaSuccess) ce = F->carve(scr, &scratch);
+    if (ce == cudaSuccess) ce = F->carve(rows, &rows_blk);
+  }
+  if (ce == cudaSuccess && n > 0) {
+    Carve pack, merge;
+    pack.add(&poff, (size_t)kPackEntries * n);
+    pack.add((char**)&pval, esz * kPackEntries * n);
+    pack.add(&pflags, 1);
+    merge.add(&moff, (size_t)kMergeStride * n);
+    merge.add(&mval, (size_t)kMergeEntries * n);
+    cudaError_t pe = F->carve(pack, &pack_blk);
+    if (pe == cudaSuccess && !cplx) pe = F->carve(merge, &merge_blk);
+    if (pe != cudaSuccess) {
+      (void)cudaGetLastError();
+      poff = nullptr;  // (what there is of it goes back below)
+    }
+  }
+  // W to rows, on the side stream when there is one (its own scratch)
+  if (!ws) wwork = work;
   if (ws && ce == cudaSuccess) {
-    ce = F->alloc(&wwork, n + scan_blocksums_size(n));
     for (int i = 0; i < 2 && ce == cudaSuccess; ++i)
       if (!F->wev[i]) ce = cudaEventCreateWithFlags(&F->wev[i], cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventRecord(F->wev[0], s);
@@ -1222,49 +1271,6 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   if (ce == cudaSuccess)
     ce = csc_to_csr(n, F->nnz_w, F->Wcp, F->Wri, F->Wv, cplx, F->Wr.rowptr, F->Wr.colidx, F->Wr.vals, wwork, wsx);
   if (ws && ce == cudaSuccess) ce = cudaEventRecord(F->wev[1], ws);  // diaf_free waits for it
-  // the level-ordered copy of V and its inputs (sizes known now; the level
-  // count is at most n), so that only copies and kernels follow the walk
-  LevelCsr& Vl = F->Vl;
-  int32_t *pos = nullptr, *dblk = nullptr;
-  uint32_t* zflag = nullptr;
-  Vl.n = n;
-  Vl.nnz = F->nnz_v - n;
-  {
-    Carve c;
-    c.add(&Vl.lvlptr, n + 1);
-    c.add(&Vl.rowptr, n + 1);
-    c.add(&Vl.colidx, Vl.nnz > 0 ? Vl.nnz : 0);
-    c.add((char**)&Vl.vals, esz * (Vl.nnz > 0 ? Vl.nnz : 0));
-    c.add((char**)&Vl.dinv, esz * n);
-    c.add(&Vl.xrow, n);
-    c.add(&pos, n);
-    c.add(&dblk, blk);
-    c.add(&zflag, 1);
-    c.add(&F->Wl.colidx, F->nnz_w);
-    c.add((char**)&F->tbuf, esz * n);
-    if (ce == cudaSuccess) ce = F->carve(c);
-  }
-  // the packed form's arrays (used when the walk finds the rows short enough);
-  // without the memory for them the level-ordered rows above do
-  int32_t *poff = nullptr, *mpos = nullptr, *moff = nullptr;
-  double* mval = nullptr;
-  void* pval = nullptr;
-  uint32_t* pflags = nullptr;
-  if (ce == cudaSuccess && n > 0) {
-    Carve c;
-    c.add(&poff, (size_t)kPackEntries * n);
-    c.add((char**)&pval, esz * kPackEntries * n);
-    if (!cplx) {
-      c.add(&mpos, (size_t)kMergeEntries * n);
-      c.add(&moff, (size_t)kMergeStride * n);
-      c.add(&mval, (size_t)kMergeEntries * n);
-    }
-    c.add(&pflags, 1);
-    if (F->carve(c) != cudaSuccess) {
-      (void)cudaGetLastError();
-      poff = nullptr;
-    }
-  }
   if (ce == cudaSuccess) ce = cudaMemsetAsync(zflag, 0, sizeof(uint32_t), s);
   int32_t* const wl_colidx = F->Wl.colidx;
   PT_DEV(s);
@@ -1343,7 +1349,7 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   Vl.r = poff ? level_group(cplx, lw.maxrow, nlev, ptr, &Vl.maxg) : 0;
   Vl.poff = poff;
   Vl.pval = pval;
-  Vl.mpos = mpos;
+  Vl.mpos = static_cast<int32_t*>(rows_blk);
   Vl.moff = moff;
   Vl.mval = mval;
   Vl.pflags = pflags;
@@ -1406,6 +1412,25 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   if (ast != DIAF_OK) return ast;
   PT_HOST();
   F->apply_ready = true;
+  if (*applied) {  // s has waited for the side stream: what the solves do not use goes back
+    F->give_back(Vl.r > 0 ? rows_blk : pack_blk, s);
+    if (Vl.r <= 1) F->give_back(merge_blk, s);
+    F->give_back(scratch, s);
+    F->Wr = F->Wl;
+    if (Vl.r > 0) {
+      Vl.rowptr = Vl.colidx = nullptr;
+      Vl.vals = nullptr;
+    } else {
+      Vl.poff = nullptr;
+      Vl.pval = nullptr;
+      Vl.pflags = nullptr;
+    }
+    if (Vl.r <= 1) {
+      Vl.moff = nullptr;
+      Vl.mval = nullptr;
+    }
+    Vl.mpos = nullptr;
+  }
   return DIAF_OK;
 }
 

@@ -1,6 +1,7 @@
 // The factorisation handle behind the opaque diaf_factors of include/diaf.h.
 #pragma once
 
+#include <algorithm>
 #include <vector>
 
 #include "plan.cuh"
@@ -82,7 +83,7 @@ struct diaf_factors {
   cudaEvent_t wev[2] = {};
   bool w_pending = false;
   bool v_upper = true;
-  Csr Wr;  // W's rows (V goes straight to its level-ordered form Vl)
+  Csr Wr;  // W's rows (block-diagonal V)
   void* tbuf = nullptr;
   // level-scheduled V solve: V in level order, W's columns renumbered to it
   LevelCsr Vl;
@@ -101,10 +102,18 @@ struct diaf_factors {
     *p = static_cast<T*>(q);
     return cudaSuccess;
   }
-  cudaError_t carve(const Carve& c) {
+  cudaError_t carve(const Carve& c, void** block = nullptr) {
     unsigned char* base = nullptr;
     cudaError_t e = alloc(&base, c.total());
     if (e == cudaSuccess) c.assign(base);
+    if (block) *block = base;
     return e;
+  }
+  // One of F's allocations given back before F is, after its last use on s.
+  void give_back(void* p, cudaStream_t s) {
+    auto it = std::find(owned.begin(), owned.end(), p);
+    if (!p || it == owned.end()) return;
+    owned.erase(it);
+    diaf_dev_free(p, s);
   }
 };

@@ -38,8 +38,8 @@ struct LevelCsr {
   void* dinv = nullptr;         // n
   int32_t* xrow = nullptr;      // n
   int maxw = 0;                 // rows of the widest level (picks the solve kernel)
-  // The packed form (r > 0; then a real V's rowptr, colidx and vals are not filled), for
-  // a V of at most kPackEntries off-diagonal entries per row: entry q of
+  // The packed form (r > 0; rowptr, colidx and vals are then scratch of the
+  // preparation, which a real V does not use), for a V of at most kPackEntries off-diagonal entries per row: entry q of
   // position p at [kPackEntries p + q], its column position (-1: none) and its
   // value.  Levels are solved in groups of r: with r > 1 the rows of a
   // group also have merged entries (kMergeEntries each), which refer to rows of
@@ -49,7 +49,7 @@ struct LevelCsr {
   int maxg = 0;                 // rows of the widest group
   int32_t* poff = nullptr;      // kPackEntries n
   void* pval = nullptr;         // kPackEntries n
-  int32_t* mpos = nullptr;      // kMergeEntries n (r > 1): the merged entries' column positions
+  int32_t* mpos = nullptr;      // kMergeEntries n (r > 1): the merged entries' column positions (preparation only)
   int32_t* moff = nullptr;      // kMergeStride n: their slots in the solve's window, then their number
   double* mval = nullptr;       // kMergeEntries n (r > 1)
   uint32_t* pflags = nullptr;   // device: what the solve has to know of the entries (kPackMergeFull, kPackFar)
