@@ -262,6 +262,14 @@ long long diaf_launch_count(void);
  * (Instrumentation, no passage of the paper; never fails.) */
 void diaf_apply_prep_counts(int64_t* streamed, int64_t* copied);
 
+/* How factors that have been applied hold a triangular V: *group = levels
+ * solved between two barriers (0: rows of any length, one level at a time; also
+ * for a block-diagonal V), *flags = what keeps a packed V from being solved so
+ * (bit 0: a row's merged entries do not fit, then one level at a time; bit 1: an
+ * entry lies beyond the solve's shared-memory window).  Synchronises `stream`.
+ * (Instrumentation, no passage of the paper.)  Errors: EINVAL, ECUDA. */
+diaf_status diaf_apply_form(diaf_factors* F, int32_t* group, uint32_t* flags, void* stream);
+
 /* Caps the device memory that the setup and apply paths (diaf_factor,
  * diaf_factor_tuned, diaf_plan_*, diaf_apply and the factor handles they
  * keep) may hold at one time, over all handles of the process: bytes > 0 is

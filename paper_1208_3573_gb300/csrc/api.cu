@@ -1434,6 +1434,18 @@ static diaf_status prepare_apply(diaf_factors* F, cudaStream_t s, const void* x,
   return DIAF_OK;
 }
 
+diaf_status diaf_apply_form(diaf_factors* F, int32_t* group, uint32_t* flags, void* stream) {
+  if (!F || !group || !flags) return fail(DIAF_EINVAL, "NULL argument");
+  if (!F->apply_ready) return fail(DIAF_EINVAL, "the factors have not been applied yet");
+  *group = F->v_block ? 0 : F->Vl.r;
+  *flags = 0;
+  if (*group == 0) return DIAF_OK;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  DIAF_CU(cudaMemcpyAsync(flags, F->Vl.pflags, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  DIAF_CU(cudaStreamSynchronize(s));
+  return DIAF_OK;
+}
+
 diaf_status diaf_level_schedule(int32_t n, const int32_t* colptr, const int32_t* rowidx, int32_t* level,
                                 int32_t* nlev, int32_t* upper) {
   g_last_error.clear();

@@ -463,7 +463,10 @@ __global__ void __launch_bounds__(kDeepThreads, 1)
 
 // The merged entries of group blockIdx.x, level by level: the row's own
 // entries of earlier groups, and for each entry of its own group v times that
-// row's merged entries.
+// row's merged entries.  Products beyond kMergeMax (or not numbers) are not
+// formed into a solve: infinite, they would turn the zeros of a sparse
+// right-hand side into NaN, which the level by level solve does not.
+constexpr uint32_t kMergeMax = 0x54b249adu;  // top_word(1e100)
 __global__ void __launch_bounds__(256) merge_kernel(int nlev, int r, const int32_t* __restrict__ lvlptr,
                                                     const int32_t* __restrict__ poff, const double* __restrict__ pval,
                                                     int32_t* mpos, int32_t* moff, double* mval, uint32_t* pflags) {
@@ -497,6 +500,7 @@ __global__ void __launch_bounds__(256) merge_kernel(int nlev, int r, const int32
         const int32_t col = poff[kPackEntries * (size_t)p + q];
         if (col < 0) continue;
         const double val = -pval[kPackEntries * (size_t)p + q];
+        full |= top_word(val) > kMergeMax;
         if (col < gs) {
           add(col, val);
         } else {
@@ -505,16 +509,17 @@ __global__ void __launch_bounds__(256) merge_kernel(int nlev, int r, const int32
             add(mpos[kMergeEntries * (size_t)col + u], -val * mval[kMergeEntries * (size_t)col + u]);
         }
       }
-      if (full) atomicOr(pflags, kPackMergeFull);
       int cnt = 0;
 #pragma unroll
       for (int q = 0; q < kMergeEntries; ++q) {
         cnt += c[q] >= 0;
+        full |= top_word(v[q]) > kMergeMax;
         mpos[kMergeEntries * (size_t)p + q] = c[q];
         moff[kMergeStride * (size_t)p + q] = c[q] & (level_window<double>() - 1);
         mval[kMergeEntries * (size_t)p + q] = -v[q];  // (the solve subtracts)
       }
       moff[kMergeStride * (size_t)p + kMergeEntries] = cnt;
+      if (full) atomicOr(pflags, kPackMergeFull);
     }
     __syncthreads();  // the level's merged rows are visible to the block
   }

@@ -59,7 +59,7 @@ constexpr int kMergeEntries = 6;
 constexpr int kMergeStride = 8;
 constexpr int kGroupRows = 1024;  // rows of a group of levels: one thread each
 enum : uint32_t {
-  kPackMergeFull = 1u,  // a merged row has more than kMergeEntries entries: the solve goes level by level
+  kPackMergeFull = 1u,  // a merged row has more than kMergeEntries entries, or one beyond kMergeMax: level by level
   kPackFar = 2u,        // an entry lies further back than the solve's shared-memory window
 };
 // Levels per group for a V of `maxrow` off-diagonal entries per row at most

@@ -141,6 +141,7 @@ def lib() -> ctypes.CDLL:
         L.diaf_launch_count.restype = ctypes.c_longlong
         L.diaf_apply_prep_counts.argtypes = [ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
         L.diaf_apply_prep_counts.restype = None
+        L.diaf_apply_form.argtypes = [vp, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_uint32), vp]
         L.diaf_set_device_memory_limit.argtypes = [ctypes.c_int64]
         L.diaf_device_memory_in_use.restype = ctypes.c_int64
         L.diaf_factor_fallbacks.argtypes = [vp, ctypes.POINTER(ctypes.c_int32), ctypes.c_int32]
@@ -317,6 +318,12 @@ class Factors:
         given; apply() must have run once on these factors)."""
         _check(lib().diaf_apply_static(self._own.ptr, _ptr(x), _ptr(y), _stream(stream)))
         return y
+
+    def apply_form(self, stream=None) -> tuple:
+        """(levels solved between two barriers, flags) of factors that have been applied (diaf_apply_form)."""
+        r, f = ctypes.c_int32(), ctypes.c_uint32()
+        _check(lib().diaf_apply_form(self._own.ptr, ctypes.byref(r), ctypes.byref(f), _stream(stream)))
+        return int(r.value), int(f.value)
 
     def sync(self, stream=None) -> None:
         _check(lib().diaf_sync(self._own.ptr, _stream(stream)))
