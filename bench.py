@@ -90,10 +90,10 @@ def dominant_kernel(bucket: int, prec: str, alg: str, cplx: bool) -> str:
 
 
 def algorithmic_flops(m: np.ndarray, k: np.ndarray, l: np.ndarray, alg: str, cplx: bool,
-                      sweeps: float = JACOBI_SWEEPS, svd: bool = True) -> tuple[float, float]:
+                      sweeps: float = JACOBI_SWEEPS, svd: bool | np.ndarray = True) -> tuple[float, float]:
     """(all flops, FP64 flops) the method does per factorisation, summed over
     the columns: QR of the m x k tile 2k^2(m - k/3), leverage keys m k^2,
-    then DIAF-S: with `svd` QR of the tile without the I_j rows and one-sided
+    then DIAF-S: with `svd` (of all columns, or by column) QR of the tile without the I_j rows and one-sided
     Jacobi on its k x k R -- `sweeps` sweeps of k(k-1)/2 rotations, each a
     2k-flop inner product and two 6k-flop column-pair updates (R and V) --,
     else that tile's Gram matrix (m k^2) and two swept inverses (2 k^3); one FP64
@@ -103,16 +103,21 @@ def algorithmic_flops(m: np.ndarray, k: np.ndarray, l: np.ndarray, alg: str, cpl
     m = m.astype(np.float64); k = k.astype(np.float64); l = l.astype(np.float64)
     f32 = 2 * k**2 * (m - k / 3) + m * k**2
     if alg == "S":
-        if svd:
-            f32 += 2 * k**2 * (np.maximum(m - l, k) - k / 3) + sweeps * k * (k - 1) / 2 * 14 * k
-        else:
-            f32 += m * k**2 + 2 * k**3
+        f32 += np.where(svd, 2 * k**2 * (np.maximum(m - l, k) - k / 3) + sweeps * k * (k - 1) / 2 * 14 * k,
+                        m * k**2 + 2 * k**3)
         f64 = 4 * m * k + 2 * m * k
     else:
         f32 += sweeps * k * (k - 1) / 2 * (8 * l + 6 * k)
         f64 = 4 * m * k + 2 * k**2 + 2 * m * k
     c = 4 if cplx else 1
     return float((f32 + f64).sum() * c), float(f64.sum() * c)
+
+
+def svd_columns(m: np.ndarray, k: np.ndarray, alg: str, prec: str, cplx: bool) -> np.ndarray:
+    """Columns whose kernel runs a Jacobi SVD: all but DIAF-S on the small and
+    mid-size tiles (buckets 0 and 1) of a real type or in mixed precision."""
+    large = (k > 32) | (m > 64)
+    return np.full(m.shape, True) if alg != "S" or (cplx and prec == "fp64") else large
 
 
 def gathered_bytes(w) -> float:
@@ -558,8 +563,7 @@ def main():
     # the kernel of the bucket that took the most time
     bucket_mean = np.mean(np.array(kern_ms, dtype=np.float64), axis=0)
     dom = int(np.argmax(bucket_mean))
-    # the small and mid-size DIAF-S tiles run without an SVD, but for complex FP64
-    svd = args.alg != "S" or dom == 2 or (cplx and args.prec == "fp64")
+    svd = svd_columns(m, k, args.alg, args.prec, cplx)
     flops, flops64 = algorithmic_flops(m, k, lcount, args.alg, cplx, svd=svd)
     achieved = flops / (kern / 1e3)
     kname = dominant_kernel(dom, args.prec, args.alg, cplx)
@@ -574,8 +578,8 @@ def main():
     roof = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": traffic, "kernel": f"{kname} (size bucket {dom}, {bucket_mean[dom] / kern:.0%} of the numeric pass; "
                                                         "the figures cover the whole pass)",
-            "kernel_ms": kern, "algorithmic_flops": flops, "jacobi_sweeps_assumed": JACOBI_SWEEPS if svd else 0,
-            "peak_source": src,
+            "kernel_ms": kern, "algorithmic_flops": flops, "jacobi_sweeps_assumed": JACOBI_SWEEPS if svd.any() else 0,
+            "jacobi_columns": int(svd.sum()), "peak_source": src,
             "fp64": {"flops": flops64, "achieved": flops64 / (kern / 1e3) / 1e12, "peak": FP64_NOMINAL_TFLOPS,
                      "unit": "TFLOP/s", "frac": flops64 / (kern / 1e3) / (FP64_NOMINAL_TFLOPS * 1e12)},
             "gather": {"bytes": gbytes, "achieved": gbytes / (kern / 1e3) / 1e9, "peak": peaks["hbm_gbs"],
