@@ -321,8 +321,9 @@ constexpr int kClusterMax = 4;  // most singular values of a close cluster resol
 // barriers; the number of threads per pair is set by k_j <= 64 and 256 threads.
 // The fused multiply-adds are spelled out, not left to the compiler: they give
 // cta_jacobi's bits.  Where the gap to the next singular value is small, the one
-// or two corrections that follow leave a trace of the FP32 basis's last bits in
-// w (up to 1e-7), and which bits those are should not change with the build.
+// or two corrections that follow stop short of the converged vector (by up to
+// 1.3e-6 of it on the power-law operator), so that w keeps a trace of the FP32
+// basis's last bits, and which bits those are should not change with the build.
 template <int KP>
 __device__ int cta_jacobi_mixed(float* G, int k, float* V, float* redF) {
   constexpr int LPP = kCtaThreads / (kCtaKmax / 2), NR = kCtaKmax / LPP;

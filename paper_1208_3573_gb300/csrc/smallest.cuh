@@ -32,7 +32,7 @@
 // of 2 k dependent shuffles.)  Numeric pass before and after, on one GB300,
 // with the Gram matrices and FP64 products over the rows' nonzeros: lognormal
 // 64^3 (k = 25) 65.8 -> 16.3 ms, FP64 convection-diffusion 129^2 (k = 13)
-// 11.3 -> 2.4 ms, complex Helmholtz 512^2 (k = 9) 13.3 -> 9.4 ms.
+// 11.3 -> 2.4 ms, complex Helmholtz 512^2 (k = 9) 13.3 -> 8.5 ms.
 // What bounds it now is latency: three to four warps per scheduler on chains
 // of shuffles and shared-memory reads.
 #pragma once
